@@ -36,3 +36,25 @@ def test_zero_upper_clears_the_strict_upper_triangle_only(lib, n, pad, off):
         want[off + r * ldc:off + r * ldc + n] = 0
         want[off + r * ldc:off + r * ldc + r + 1] = ref[r, :r + 1]
     assert np.array_equal(buf.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("p", [13, 65521, 1000003, 2**31 - 1])
+@pytest.mark.parametrize("rows,cols,off", [(1, 1, 0), (3, 2, 1), (5, 3, 3), (9, 4, 0), (7, 4, 2),
+                                           (8, 5, 0), (2, 127, 1), (3, 1024, 0), (2, 2051, 1)])
+def test_split_of_ragged_and_unaligned_rows(lib, p, rows, cols, off):
+    """Digits and pair sums of every entry, zeros in the row padding."""
+    import torch
+    from paper_2101_01025_gb300 import testing as T
+    b, L, _, ns = T.digit_spec(p, with_sums=True)
+    X = synth.residues(17 * rows + cols, (rows, cols), p, balanced=True)
+    ld = cols + off
+    buf = torch.zeros(off + rows * ld + 4, dtype=torch.int32, device="cuda")
+    view = torch.as_strided(buf, (rows, cols), (ld, 1), off)
+    view.copy_(torch.from_numpy(X))
+    got = T.split(view, p).float().cpu().numpy().astype(np.int64)
+    assert not got[:, :, cols:].any()
+    d = got[:, :, :cols]
+    assert np.array_equal(sum(d[i] << (b * i) for i in range(L)), X.astype(np.int64))
+    pairs = [(i, j) for i in range(L) for j in range(i + 1, L)][:ns]
+    for q, (i, j) in enumerate(pairs):
+        assert np.array_equal(d[L + q], d[i] + d[j])
