@@ -162,7 +162,7 @@ AAT_API int64_t aat_modp_host_d2h_bytes(int64_t n, uint32_t flags);
  * Autotuning of Low(A A^T) mod p on the tensor-core leaf for one shape.
  * The choices tuned: the recursion depth (the cut-off of Algorithm 1's
  * recursion, Sec. 3; the paper leaves it to the implementation, Sec. 7), the
- * leaf kernel form (form 1: one CTA per 128 x 256 tile; form 2: CTA pairs,
+ * leaf kernel form (form 1: one CTA per 128 x 256 or 128 x 64 tile; form 2: CTA pairs,
  * 256 x 256 tiles), the digit-product form (plain_digits 1: one product per
  * digit pair) and Winograd's form for the last level's general products
  * (winograd 1, as AAT_WINOGRAD).  aat_tune_modp runs every candidate on

@@ -267,15 +267,20 @@ __device__ __forceinline__ OutView tile_out(const Params &P, int t) {
 //   work is latency-bound at 2 warps per scheduler: the 128 live
 //   accumulators leave few registers for independent temporaries); the
 //   price is 96 registers per thread (and some spills).
-template <bool PAIR, int EW = 8>
+//   TN: tile columns.  64 instead of 256 in the narrow one-CTA form
+//   (leaf_form): four times as many CTAs share the work of a product with
+//   few tiles, and each epilogue thread converts, multiplies and stores 32
+//   entries instead of 128; at full rate its MMAs (M=128 N=64) would read 192
+//   bytes of shared memory per clock, more than there are, so they run slower.
+template <bool PAIR, int EW = 8, int TN = 256>
 struct Shape {
   static constexpr int EPI_WARPS = EW;
   static constexpr int THREADS = 64 + EW * 32;
-  static constexpr int VALS = 1024 / EW;          // accumulators per thread
+  static constexpr int VALS = 4 * TN / EW;        // accumulators per thread
   static constexpr int XB = EW == 8 ? 16 : 8;     // staged store block width
   static constexpr int TM = PAIR ? 256 : 128;     // output tile rows
-  static constexpr int YROWS = PAIR ? 128 : 256;  // rows of Y per CTA and stage
-  static constexpr int STAGES = PAIR ? 6 : 4;
+  static constexpr int YROWS = PAIR ? TN / 2 : TN;  // rows of Y per CTA and stage
+  static constexpr int STAGES = PAIR ? 6 : TN == 256 ? 4 : 8;
   static constexpr int A_BYTES = BM * BK * 2;
   static constexpr int B_BYTES = YROWS * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
@@ -291,17 +296,17 @@ struct Shape {
   // (bit 4), A and B BF16 (bits 7, 10), both K-major, N >> 3 at bit 17,
   // M >> 4 at bit 24.
   static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) |
-                                    ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+                                    ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
 };
 
 // Epilogue warps of the single-problem launches and of the batched launch
 // (whose tiles are mostly short in K, so the per-tile epilogue dominates).
 constexpr int kEwLeaf = 8, kEwBatch = 16;
 
-template <int MODE, bool PAIR, int EW>
-__global__ void __launch_bounds__(Shape<PAIR, EW>::THREADS, 1)
+template <int MODE, bool PAIR, int EW, int TN = BN>
+__global__ void __launch_bounds__(Shape<PAIR, EW, TN>::THREADS, 1)
     leaf_tc_kernel(const __grid_constant__ Params P) {
-  using S = Shape<PAIR, EW>;
+  using S = Shape<PAIR, EW, TN>;
   constexpr int EPI_WARPS = S::EPI_WARPS, VALS = S::VALS, XB = S::XB;
   constexpr int STAGES = S::STAGES;
   extern __shared__ uint8_t smem_raw[];
@@ -378,7 +383,7 @@ __global__ void __launch_bounds__(Shape<PAIR, EW>::THREADS, 1)
       for (int t = (int)unit0; t < P.ntiles && ok; t += (int)nunits) {
         const TileView v = tile_view<MODE>(P, t);
         const int rowx = v.I * S::TM + (int)rank * BM;
-        const int rowy = v.J * BN + (int)rank * S::YROWS;
+        const int rowy = v.J * TN + (int)rank * S::YROWS;
         for (int gi = 0; gi < v.ng && ok; ++gi) {
           const Group g = v.g[gi];
           for (int kb = g.kb0; kb < g.kb1; ++kb) {
@@ -536,7 +541,7 @@ __global__ void __launch_bounds__(Shape<PAIR, EW>::THREADS, 1)
         const OutView o = tile_out<MODE>(P, t);
         const int2 ij = tile_ij<MODE>(P, t);
         const int64_t r0 = (int64_t)ij.x * S::TM + (int64_t)rank * BM + quarter * 32;
-        const int64_t c0 = (int64_t)ij.y * BN + cpart * VALS;
+        const int64_t c0 = (int64_t)ij.y * TN + cpart * VALS;
         live = r0 < o.M && c0 < o.N && !(o.lower && c0 > r0 + 31);
       }
       int32_t acc[VALS];
@@ -567,8 +572,10 @@ __global__ void __launch_bounds__(Shape<PAIR, EW>::THREADS, 1)
             const uint32_t ta = tmem + lane_base + buf * ACC_COLS + (uint32_t)(cpart * VALS);
             tmem_drain16<0>(ta, acc);
             tmem_drain16<16>(ta + 16u, acc);
-            tmem_drain16<32>(ta + 32u, acc);
-            tmem_drain16<48>(ta + 48u, acc);
+            if constexpr (VALS >= 64) {
+              tmem_drain16<32>(ta + 32u, acc);
+              tmem_drain16<48>(ta + 48u, acc);
+            }
             if constexpr (VALS == 128) {
               tmem_drain16<64>(ta + 64u, acc);
               tmem_drain16<80>(ta + 80u, acc);
@@ -592,7 +599,7 @@ __global__ void __launch_bounds__(Shape<PAIR, EW>::THREADS, 1)
       if (!live) continue;
       const int2 ij = tile_ij<MODE>(P, t);
       const int64_t row = (int64_t)ij.x * S::TM + (int64_t)rank * BM + quarter * 32 + lane;
-      const int64_t col0 = (int64_t)ij.y * BN + cpart * VALS;
+      const int64_t col0 = (int64_t)ij.y * TN + cpart * VALS;
       // final value, canonical, in place: the last group is the final
       // multiplier, whose Horner step left every entry balanced
 #pragma unroll
@@ -646,10 +653,11 @@ __global__ void __launch_bounds__(Shape<PAIR, EW>::THREADS, 1)
         __syncwarp();
         if constexpr (EW == 8) {
           // accumulating product (8 epilogue warps): the old values are
-          // loaded four at a time, so four DRAM latencies overlap instead of
-          // one round trip per store
+          // loaded four at a time (sixteen where the narrow tile leaves the
+          // registers), so as many DRAM latencies overlap instead of one
+          // round trip per store
           if (accum) {
-            constexpr int G = 4;
+            constexpr int G = VALS > 32 ? 4 : 16;
 #pragma unroll 1
             for (int i0 = 0; i0 < XB; i0 += G) {
               int32_t oldv[G];
@@ -718,7 +726,7 @@ __global__ void __launch_bounds__(Shape<PAIR, EW>::THREADS, 1)
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 std::mutex g_mu;
-std::map<std::tuple<int, int64_t, int64_t, int, int>, std::pair<int2 *, int>> g_tiles;
+std::map<std::tuple<int, int64_t, int64_t, int, int, int>, std::pair<int2 *, int>> g_tiles;
 std::map<int, bool> g_attr_set;
 std::map<int, int> g_pair_units;  // co-resident CTA pairs per device
 
@@ -763,14 +771,14 @@ int64_t band_rows() {
   return v;
 }
 
-void tile_order(int64_t M, int64_t N, int lower, int tm, std::vector<int2> &v) {
-  const int64_t TI = (M + tm - 1) / tm, TJ = (N + BN - 1) / BN;
+void tile_order(int64_t M, int64_t N, int lower, int tm, int tn, std::vector<int2> &v) {
+  const int64_t TI = (M + tm - 1) / tm, TJ = (N + tn - 1) / tn;
   const int64_t band = std::max<int64_t>(1, band_rows() / tm);
   for (int64_t bi = 0; bi < TI; bi += band) {
     const int64_t iend = std::min(TI, bi + band);
     for (int64_t j = 0; j < TJ; ++j)
       for (int64_t i = bi; i < iend; ++i) {
-        if (lower && j * BN > i * tm + tm - 1) continue;
+        if (lower && j * tn > i * tm + tm - 1) continue;
         v.push_back(make_int2((int)i, (int)j));
       }
   }
@@ -785,8 +793,9 @@ cudaError_t upload(const std::vector<T> &v, T **out) {
   return cudaMemcpy(*out, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
 }
 
-cudaError_t get_tiles(int dev, int64_t M, int64_t N, int lower, int tm, int2 **out, int *count) {
-  auto key = std::make_tuple(dev, M, N, lower, tm);
+cudaError_t get_tiles(int dev, int64_t M, int64_t N, int lower, int tm, int tn, int2 **out,
+                      int *count) {
+  auto key = std::make_tuple(dev, M, N, lower, tm, tn);
   auto it = g_tiles.find(key);
   if (it != g_tiles.end()) {
     *out = it->second.first;
@@ -794,7 +803,7 @@ cudaError_t get_tiles(int dev, int64_t M, int64_t N, int lower, int tm, int2 **o
     return cudaSuccess;
   }
   std::vector<int2> v;
-  tile_order(M, N, lower, tm, v);
+  tile_order(M, N, lower, tm, tn, v);
   int2 *d = nullptr;
   cudaError_t e = upload(v, &d);
   if (e != cudaSuccess) return e;
@@ -810,8 +819,8 @@ cudaError_t get_tiles(int dev, int64_t M, int64_t N, int lower, int tm, int2 **o
 std::map<std::vector<int64_t>, std::pair<int4 *, int>> g_mtiles;
 
 cudaError_t get_multi_tiles(int dev, const TcLeafArgs *as, const int *order, int count, int tm,
-                            int4 **out, int *ntiles) {
-  std::vector<int64_t> key = {dev, tm};
+                            int tn, int4 **out, int *ntiles) {
+  std::vector<int64_t> key = {dev, tm, tn};
   for (int q = 0; q < count; ++q) {
     const TcLeafArgs &a = as[order[q]];
     key.insert(key.end(), {(int64_t)order[q], a.M, a.N, (int64_t)a.lower});
@@ -827,7 +836,7 @@ cudaError_t get_multi_tiles(int dev, const TcLeafArgs *as, const int *order, int
   for (int q = 0; q < count; ++q) {
     const TcLeafArgs &a = as[order[q]];
     one.clear();
-    tile_order(a.M, a.N, a.lower, tm, one);
+    tile_order(a.M, a.N, a.lower, tm, tn, one);
     for (const int2 &t : one) v.push_back(make_int4(order[q], t.x, t.y, 0));
   }
   int4 *d = nullptr;
@@ -1030,6 +1039,69 @@ int pair_override() {
   return v;
 }
 
+int sm_count(int dev) {
+  int sms = 148;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
+// Tiles of tm x tn of an M x N product (lower: those that touch i >= j).
+int64_t tile_count(int64_t M, int64_t N, int lower, int tm, int tn) {
+  const int64_t TI = (M + tm - 1) / tm, TJ = (N + tn - 1) / tn;
+  if (!lower) return TI * TJ;
+  int64_t c = 0;
+  for (int64_t i = 0; i < TI; ++i) c += std::min(TJ, (i * tm + tm - 1) / tn + 1);
+  return c;
+}
+
+constexpr int kTnNarrow = 64;
+enum Form { kCta = 1, kPair = 2, kNarrow = 3 };
+int form_tm(Form f) { return f == kPair ? 256 : 128; }
+int form_tn(Form f) { return f == kNarrow ? kTnNarrow : BN; }
+
+// Plane products per ring multiply-add of a leaf.
+int term_count(const TcLeafArgs &a) {
+  return a.dx.nsum > 0 ? std::min(a.x.L, a.y.L) : a.x.L * a.y.L;
+}
+
+// The form of one launch over `count` products.  CTA pairs when their tiles
+// fill every co-resident pair (or AAT_LEAF_PAIR / TcLeafArgs::form says so).
+// Otherwise one CTA per tile, 256 or 64 columns wide, by the modelled length
+// of the longest CTA in SM cycles: waves of tiles times (K blocks of the MMA,
+// 512 cycles wide and ~200 narrow; per plane product a Horner step and a
+// drain, 4600 wide and 1150 narrow; prologue, fill and store).  Measured at
+// 1001 x 1001 x 3001
+// (lower) mod 2^31 - 1, 20 wide or 72 narrow tiles: 178 -> 127 us; the four and
+// the one product of 512 x 512 mod 131071 with one level, 23.5 -> 11.8 and
+// 38.1 -> 14.0 us.
+Form leaf_form(const TcLeafArgs *as, int count, int units, int sms) {
+  const int ov = as[0].form > 0 ? as[0].form - 1 : pair_override();
+  if (units > 0) {
+    bool big = true;
+    int64_t pt = 0;
+    for (int i = 0; i < count; ++i) {
+      big = big && as[i].M >= 256;
+      const int64_t t = ((as[i].M + 255) / 256) * ((as[i].N + BN - 1) / BN);
+      pt += as[i].lower ? t / 2 : t;
+    }
+    if (big && (ov >= 0 ? ov > 0 : pt >= units)) return kPair;
+  }
+  double cost[2];
+  for (int w = 0; w < 2; ++w) {
+    double work = 0.0;
+    int64_t tiles = 0;
+    for (int i = 0; i < count; ++i) {
+      const TcLeafArgs &a = as[i];
+      const int64_t t = tile_count(a.M, a.N, a.lower, BM, w ? kTnNarrow : BN);
+      const double kb = (double)((a.K + BK - 1) / BK), terms = term_count(a);
+      work += t * (w ? terms * (200.0 * kb + 1150.0) + 2500.0 : terms * (512.0 * kb + 4600.0) + 8000.0);
+      tiles += t;
+    }
+    cost[w] = work / (double)tiles * (double)((tiles + sms - 1) / sms);
+  }
+  return cost[1] < cost[0] ? kNarrow : kCta;
+}
+
 }  // namespace
 
 cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) {
@@ -1046,22 +1118,15 @@ cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) 
   int dev = 0;
   cudaGetDevice(&dev);
 
-  // the form: CTA pairs when there are enough 256 x 256 tiles to keep every
-  // co-resident pair busy
-  const int units = pair_units(dev);
-  bool pair = false;
-  if (units > 0 && a.M >= 256) {
-    const int64_t pt = ((a.M + 255) / 256) * ((a.N + BN - 1) / BN);
-    const int ov = a.form > 0 ? a.form - 1 : pair_override();
-    pair = ov >= 0 ? ov > 0 : (a.lower ? pt / 2 : pt) >= units;
-  }
-  const int tm = pair ? Shape<true>::TM : Shape<false>::TM;
+  const int units = pair_units(dev), sms = sm_count(dev);
+  const Form form = leaf_form(&a, 1, units, sms);
+  const bool pair = form == kPair;
+  const int tm = form_tm(form), tn = form_tn(form);
 
   Params *P = new Params;
   std::memset(P, 0, sizeof(Params));
   if ((e = encode_planes(&P->tmx, a.x, BM)) != cudaSuccess ||
-      (e = encode_planes(&P->tmy, a.y, pair ? Shape<true>::YROWS : Shape<false>::YROWS)) !=
-          cudaSuccess) {
+      (e = encode_planes(&P->tmy, a.y, pair ? Shape<true>::YROWS : tn)) != cudaSuccess) {
     delete P;
     return e;
   }
@@ -1083,7 +1148,7 @@ cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) 
   P->status = device_status_ptr();
   int2 *tiles = nullptr;
   int nt = 0;
-  if ((e = get_tiles(dev, a.M, a.N, a.lower, tm, &tiles, &nt)) != cudaSuccess) {
+  if ((e = get_tiles(dev, a.M, a.N, a.lower, tm, tn, &tiles, &nt)) != cudaSuccess) {
     delete P;
     return e;
   }
@@ -1093,11 +1158,13 @@ cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) 
     e = cudaFuncSetAttribute(leaf_tc_kernel<kSingle, false, kEwLeaf>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)Shape<false, kEwLeaf>::SMEM);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(leaf_tc_kernel<kSingle, false, kEwLeaf, kTnNarrow>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)Shape<false, kEwLeaf, kTnNarrow>::SMEM);
     if (e != cudaSuccess) { delete P; return e; }
     g_attr_set[dev] = true;
   }
-  int sms = 148;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (nt > 0) {
     // algorithmic tensor work: one BF16 product of the ring MACs per plane
     // product with a non-zero weight
@@ -1119,6 +1186,10 @@ cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) 
       cfg.numAttrs = 1;
       e = cudaLaunchKernelEx(&cfg, leaf_tc_kernel<kSingle, true, kEwLeaf>, *P);
       if (e != cudaSuccess) { delete P; return e; }
+    } else if (form == kNarrow) {
+      leaf_tc_kernel<kSingle, false, kEwLeaf, kTnNarrow>
+          <<<std::max(1, std::min(nt, sms)), Shape<false, kEwLeaf, kTnNarrow>::THREADS,
+             Shape<false, kEwLeaf, kTnNarrow>::SMEM, st>>>(*P);
     } else {
       leaf_tc_kernel<kSingle, false, kEwLeaf>
           <<<std::max(1, std::min(nt, sms)), Shape<false, kEwLeaf>::THREADS,
@@ -1127,14 +1198,6 @@ cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) 
   }
   delete P;
   return cudaGetLastError();
-}
-
-int64_t tile_count(int64_t M, int64_t N, int lower, int tm) {
-  const int64_t TI = (M + tm - 1) / tm, TJ = (N + BN - 1) / BN;
-  if (!lower) return TI * TJ;
-  int64_t c = 0;
-  for (int64_t i = 0; i < TI; ++i) c += std::min(TJ, (i * tm + tm - 1) / BN + 1);
-  return c;
 }
 
 // Whether one launch over the tiles of several products beats one launch
@@ -1154,8 +1217,7 @@ int leaf_tc_terms(const TcLeafArgs &a, const ModP &m) {
 bool leaf_tc_fuse_pays(const TcLeafArgs *as, int count) {
   int dev = 0;
   cudaGetDevice(&dev);
-  int sms = 148;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = sm_count(dev);
   int units = 0;
   {
     std::lock_guard<std::mutex> lock(g_mu);
@@ -1164,14 +1226,9 @@ bool leaf_tc_fuse_pays(const TcLeafArgs *as, int count) {
   double idle = 0.0, all = 0.0;
   for (int i = 0; i < count; ++i) {
     const TcLeafArgs &a = as[i];
-    bool pair = false;
-    if (units > 0 && a.M >= 256) {
-      const int64_t pt = ((a.M + 255) / 256) * ((a.N + BN - 1) / BN);
-      const int ov = a.form > 0 ? a.form - 1 : pair_override();
-      pair = ov >= 0 ? ov > 0 : (a.lower ? pt / 2 : pt) >= units;
-    }
+    const bool pair = leaf_form(&a, 1, units, sms) == kPair;
     const int u = pair ? units : sms;
-    const double nt = (double)tile_count(a.M, a.N, a.lower, pair ? 256 : 128);
+    const double nt = (double)tile_count(a.M, a.N, a.lower, pair ? 256 : 128, BN);
     const double slots = std::ceil(nt / u) * u;
     const double kb = (double)((a.K + BK - 1) / BK);
     idle += (slots - nt) * kb;
@@ -1203,21 +1260,10 @@ cudaError_t launch_leaf_tc_multi(const TcLeafArgs *as, int count, const ModP &m,
   int dev = 0;
   cudaGetDevice(&dev);
 
-  // the form, as for one product, over the tiles of all of them
-  const int units = pair_units(dev);
-  bool pair = false;
-  if (units > 0) {
-    bool big = true;
-    int64_t pt = 0;
-    for (int i = 0; i < count; ++i) {
-      big = big && as[i].M >= 256;
-      const int64_t t = ((as[i].M + 255) / 256) * ((as[i].N + BN - 1) / BN);
-      pt += as[i].lower ? t / 2 : t;
-    }
-    const int ov = as[0].form > 0 ? as[0].form - 1 : pair_override();
-    pair = big && (ov >= 0 ? ov > 0 : pt >= units);
-  }
-  const int tm = pair ? Shape<true>::TM : Shape<false>::TM;
+  const int units = pair_units(dev), sms = sm_count(dev);
+  const Form form = leaf_form(as, count, units, sms);
+  const bool pair = form == kPair;
+  const int tm = form_tm(form), tn = form_tn(form);
 
   Params *P = new Params;
   std::memset(P, 0, sizeof(Params));
@@ -1229,8 +1275,7 @@ cudaError_t launch_leaf_tc_multi(const TcLeafArgs *as, int count, const ModP &m,
     const TcLeafArgs &a = as[i];
     MultiProb &b = P->mp[i];
     if ((e = encode_planes(&b.tmx, a.x, BM)) != cudaSuccess ||
-        (e = encode_planes(&b.tmy, a.y, pair ? Shape<true>::YROWS : Shape<false>::YROWS)) !=
-            cudaSuccess) {
+        (e = encode_planes(&b.tmy, a.y, pair ? Shape<true>::YROWS : tn)) != cudaSuccess) {
       delete P;
       return e;
     }
@@ -1276,7 +1321,7 @@ cudaError_t launch_leaf_tc_multi(const TcLeafArgs *as, int count, const ModP &m,
   std::stable_sort(order.begin(), order.end(), [&](int u, int v) { return cost[u] > cost[v]; });
   int4 *tiles = nullptr;
   int nt = 0;
-  if ((e = get_multi_tiles(dev, as, order.data(), count, tm, &tiles, &nt)) != cudaSuccess) {
+  if ((e = get_multi_tiles(dev, as, order.data(), count, tm, tn, &tiles, &nt)) != cudaSuccess) {
     delete P;
     return e;
   }
@@ -1289,6 +1334,9 @@ cudaError_t launch_leaf_tc_multi(const TcLeafArgs *as, int count, const ModP &m,
     if ((e = cudaFuncSetAttribute(leaf_tc_kernel<kMulti, false, kEwLeaf>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)Shape<false, kEwLeaf>::SMEM)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(leaf_tc_kernel<kMulti, false, kEwLeaf, kTnNarrow>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)Shape<false, kEwLeaf, kTnNarrow>::SMEM)) != cudaSuccess ||
         (e = cudaFuncSetAttribute(leaf_tc_kernel<kMulti, true, kEwLeaf>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)Shape<true, kEwLeaf>::SMEM)) != cudaSuccess) {
@@ -1297,8 +1345,6 @@ cudaError_t launch_leaf_tc_multi(const TcLeafArgs *as, int count, const ModP &m,
     }
     attr[dev] = true;
   }
-  int sms = 148;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (nt > 0) {
     ProfScope prof(AAT_K_LEAF_TC, st, work);
     if (pair) {
@@ -1319,6 +1365,10 @@ cudaError_t launch_leaf_tc_multi(const TcLeafArgs *as, int count, const ModP &m,
         delete P;
         return e;
       }
+    } else if (form == kNarrow) {
+      leaf_tc_kernel<kMulti, false, kEwLeaf, kTnNarrow>
+          <<<std::max(1, std::min(nt, sms)), Shape<false, kEwLeaf, kTnNarrow>::THREADS,
+             Shape<false, kEwLeaf, kTnNarrow>::SMEM, st>>>(*P);
     } else {
       leaf_tc_kernel<kMulti, false, kEwLeaf>
           <<<std::max(1, std::min(nt, sms)), Shape<false, kEwLeaf>::THREADS,

@@ -58,3 +58,30 @@ def test_split_of_ragged_and_unaligned_rows(lib, p, rows, cols, off):
     pairs = [(i, j) for i in range(L) for j in range(i + 1, L)][:ns]
     for q, (i, j) in enumerate(pairs):
         assert np.array_equal(d[L + q], d[i] + d[j])
+
+
+@pytest.mark.parametrize("lower", [False, True])
+@pytest.mark.parametrize("p", [65521, 131071, 2**31 - 1])
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (128, 64, 64), (129, 65, 65), (127, 63, 63),
+                                   (200, 191, 130), (260, 260, 1030)])
+def test_narrow_leaf_tiles(lib, M, N, K, p, lower):
+    """64-column tiles at their edges, stored and accumulated, with rows that
+    are and are not 16-byte aligned."""
+    import torch
+    from paper_2101_01025_gb300 import testing as T
+    if lower and M != N:
+        N = M
+    X = synth.residues(M + K, (M, K), p, balanced=True)
+    Y = X if lower else synth.residues(N + 3 * K, (N, K), p, balanced=True)
+    ref = (X.astype(object) @ Y.astype(object).T) % p
+    Xd, Yd = torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda()
+    for ld in (N, (N + 3) // 4 * 4):
+        old = synth.residues(5, (M, ld), p)
+        for acc in (False, True):
+            C = torch.from_numpy(old.copy()).cuda()
+            T.leaf(Xd, Xd if lower else Yd, p, C=C[:, :N], lower=lower, accumulate=acc)
+            want = old.astype(object)
+            new = (ref + (want[:, :N] if acc else 0)) % p
+            mask = np.tril(np.ones((M, N), bool)) if lower else np.ones((M, N), bool)
+            want[:, :N][mask] = new[mask]
+            assert np.array_equal(C.cpu().numpy().astype(object), want)
