@@ -333,7 +333,8 @@ __global__ void __launch_bounds__(Shape<PAIR, EW, TN>::THREADS, 1)
   }
   const bool leader = (rank == 0);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // the shuffles tell the compiler that warp and tmem are the same in a warp
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(FULL(s), 1);
@@ -369,11 +370,17 @@ __global__ void __launch_bounds__(Shape<PAIR, EW, TN>::THREADS, 1)
   // reaches them
   if constexpr (PAIR) cluster_sync();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   if (warp == 0) {
     // ---------------------------------------------------------- producer
-    if (lane == 0) {
+    // the whole warp runs the loop in uniform control flow, as the MMA issuer
+    // does, and one elected lane issues the copies.  A loop run by one
+    // divergent lane needed ~500 cycles per K block (its operands moved to the
+    // uniform datapath one by one), which bounded the narrow form: 1001 x 1001
+    // x 3001 mod 2^31 - 1 went 127 -> 69 us, 2500 x 4001 x 3003 (pairs) 20 us
+    // less of 490
+    {
       int stage = 0;
       uint32_t ph = 0;
       int issued = 0;
@@ -387,21 +394,25 @@ __global__ void __launch_bounds__(Shape<PAIR, EW, TN>::THREADS, 1)
         for (int gi = 0; gi < v.ng && ok; ++gi) {
           const Group g = v.g[gi];
           for (int kb = g.kb0; kb < g.kb1; ++kb) {
-            if (!wait_bounded<PAIR>(EMPTY(stage), ph ^ 1u, abort_flag, P.status)) {
+            if (!__all_sync(0xffffffffu, wait_bounded<PAIR>(EMPTY(stage), ph ^ 1u, abort_flag,
+                                                            P.status))) {
               ok = false;
               break;
             }
             const uint32_t sa = sbase + (uint32_t)(stage * S::STAGE_BYTES);
             const uint32_t fb = full0 + 8u * (uint32_t)stage;
-            if constexpr (PAIR) {
-              if (leader) mbar_expect_tx(FULL(stage), (uint32_t)(2 * S::STAGE_BYTES));
-              tma_load_3d_pair(sa, v.tmx, fb, kb * BK, rowx, g.xp);
-              tma_load_3d_pair(sa + S::A_BYTES, v.tmy, fb, kb * BK, rowy, g.yp);
-            } else {
-              mbar_expect_tx(FULL(stage), (uint32_t)S::STAGE_BYTES);
-              tma_load_3d(sa, v.tmx, fb, kb * BK, rowx, g.xp);
-              tma_load_3d(sa + S::A_BYTES, v.tmy, fb, kb * BK, rowy, g.yp);
+            if (elect_one()) {
+              if constexpr (PAIR) {
+                if (leader) mbar_expect_tx(FULL(stage), (uint32_t)(2 * S::STAGE_BYTES));
+                tma_load_3d_pair(sa, v.tmx, fb, kb * BK, rowx, g.xp);
+                tma_load_3d_pair(sa + S::A_BYTES, v.tmy, fb, kb * BK, rowy, g.yp);
+              } else {
+                mbar_expect_tx(FULL(stage), (uint32_t)S::STAGE_BYTES);
+                tma_load_3d(sa, v.tmx, fb, kb * BK, rowx, g.xp);
+                tma_load_3d(sa + S::A_BYTES, v.tmy, fb, kb * BK, rowy, g.yp);
+              }
             }
+            __syncwarp();
             ++issued;
             if (++stage == STAGES) {
               stage = 0;
@@ -439,6 +450,9 @@ __global__ void __launch_bounds__(Shape<PAIR, EW, TN>::THREADS, 1)
       int stage = 0;
       uint32_t ph = 0, chunk = 0;
       bool ok = true;
+      // stage and K step move a shared-memory descriptor's start-address field
+      // (16-byte units) only, so descriptors are formed by adds
+      const uint64_t da0 = sw128_desc(sbase);
       for (int t = (int)unit0; t < P.ntiles && ok; t += (int)nunits) {
         const int ng = tile_ng<MODE>(P, t);
         for (int gi = 0; gi < ng && ok; ++gi) {
@@ -459,16 +473,16 @@ __global__ void __launch_bounds__(Shape<PAIR, EW, TN>::THREADS, 1)
                 break;
               }
               tc_fence_after();
-              const uint32_t sa = sbase + (uint32_t)(stage * S::STAGE_BYTES);
-              const uint32_t sb = sa + S::A_BYTES;
+              const uint64_t da = da0 + (uint64_t)((uint32_t)(stage * S::STAGE_BYTES) >> 4);
+              const uint64_t db = da + (uint64_t)(S::A_BYTES >> 4);
               if (elect_one()) {
 #pragma unroll
                 for (int s = 0; s < BK / 16; ++s) {
                   const uint32_t acc = (k > kb || s > 0) ? 1u : 0u;
                   if constexpr (PAIR)
-                    tc_mma_pair(dt, sw128_desc(sa + 32u * s), sw128_desc(sb + 32u * s), S::IDESC, acc);
+                    tc_mma_pair(dt, da + 2u * s, db + 2u * s, S::IDESC, acc);
                   else
-                    tc_mma(dt, sw128_desc(sa + 32u * s), sw128_desc(sb + 32u * s), S::IDESC, acc);
+                    tc_mma(dt, da + 2u * s, db + 2u * s, S::IDESC, acc);
                 }
                 if constexpr (PAIR)
                   tc_commit_pair(EMPTY(stage), 3);
@@ -1071,9 +1085,10 @@ int term_count(const TcLeafArgs &a) {
 // 512 cycles wide and ~200 narrow; per plane product a Horner step and a
 // drain, 4600 wide and 1150 narrow; prologue, fill and store).  Measured at
 // 1001 x 1001 x 3001
-// (lower) mod 2^31 - 1, 20 wide or 72 narrow tiles: 178 -> 127 us; the four and
-// the one product of 512 x 512 mod 131071 with one level, 23.5 -> 11.8 and
-// 38.1 -> 14.0 us.
+// (lower) mod 2^31 - 1, 20 wide or 72 narrow tiles: 178 -> 69 us; the four and
+// the one product of 512 x 512 mod 131071 with one level, 23.5 -> 10.4 and
+// 38.1 -> 12.0 us; 2048 x 2048 x 1500 (lower) mod 65521, 72 wide or 272
+// narrow tiles: 40.8 -> 31 us.
 Form leaf_form(const TcLeafArgs *as, int count, int units, int sms) {
   const int ov = as[0].form > 0 ? as[0].form - 1 : pair_override();
   if (units > 0) {
