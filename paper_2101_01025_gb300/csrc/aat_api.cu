@@ -1176,7 +1176,7 @@ static size_t choose_schedule(Ctx &c, const int32_t *A, int64_t n, int64_t k, in
 // M M^H mod p for the quaternion matrix M = A + B i + C j + D k (Sec. 6.2,
 // the 6-multiplication algorithm): U1 = A + B, U2 = C + D; five general
 // products Q1 = C A^T, Q2 = D B^T, Q3 = U2 U1^T, Q4 = A B^T, Q5 = C D^T on the
-// exact leaf (digit planes of A, B, C, D, U1, U2 split once and shared);
+// exact leaf (digit planes of every operand written once and shared);
 // Q6 = Low((U1 + U2)(U1 + U2)^T) by Algorithm 1 into H1; then the closing
 // additions into Low(H1..H4).
 static size_t quat_plan(Ctx &c, const int32_t *const M[4], int64_t n, int64_t k, int64_t lda,
@@ -1185,38 +1185,67 @@ static size_t quat_plan(Ctx &c, const int32_t *const M[4], int64_t n, int64_t k,
   c.ar.dry = dry;
   c.ar.base = ws;
   const bool tc = (c.leaf == AAT_LEAF_TC);
-  int32_t *U = (int32_t *)c.ar.get((size_t)3 * n * k * 4);
-  int32_t *U1 = U, *U2 = U + n * k, *U12 = U + 2 * n * k;
+  // Q6 straight from the digit planes of U1 + U2 when it is one leaf with the
+  // digit form of the other five (no recursion, no plane passes, nothing tuned)
+  TuneVal tv;
+  const bool q6_leaf =
+      tc && !c.passes && prepare_levels(n, k, c.m.p, flags) == 0 &&
+      ((flags & AAT_LEVELS_MASK) || !tune_find(n, k, c.m.p, &tv));
+  int32_t *U1 = nullptr, *U2 = nullptr, *U12 = nullptr;
+  if (!q6_leaf) U12 = (int32_t *)c.ar.get((size_t)n * k * 4);
+  if (!tc) {
+    U1 = (int32_t *)c.ar.get((size_t)n * k * 4);
+    U2 = (int32_t *)c.ar.get((size_t)n * k * 4);
+  }
   int32_t *Q = (int32_t *)c.ar.get((size_t)5 * n * n * 4);
-  if (!dry)
+  Operand o[7] = {{M[0], lda, no_planes()}, {M[1], lda, no_planes()}, {M[2], lda, no_planes()},
+                  {M[3], lda, no_planes()}, {U1, k, no_planes()},   {U2, k, no_planes()},
+                  {U12, k, no_planes()}};
+  if (tc) {
+    // the sums and every operand's planes in one pass over A, B, C, D
+    Planes pl[7];
+    for (int q = 0; q < 7; ++q) pl[q] = o[q].pl = q < 6 || q6_leaf ? planes_alloc(c, n, k) : no_planes();
+    if (!dry)
+      check(c, launch_quat_split(M[0], M[1], M[2], M[3], lda, n, k, pl, U12, k, c.m, c.ds.b, c.st),
+            "quaternion sums and splits");
+  } else if (!dry) {
     check(c, launch_quat_sums(M[0], M[1], M[2], M[3], lda, n, k, U1, U2, U12, k, c.m, c.st),
           "quaternion sums");
-  Operand o[6] = {{M[0], lda, no_planes()}, {M[1], lda, no_planes()}, {M[2], lda, no_planes()},
-                  {M[3], lda, no_planes()}, {U1, k, no_planes()},   {U2, k, no_planes()}};
-  if (tc)
-    for (Operand &x : o) {
-      x.pl = planes_alloc(c, n, k);
-      if (!dry) check(c, launch_split(x.x, x.ld, n, k, c.m, c.ds.b, x.pl, c.st), "split");
-    }
-  const Operand &oA = o[0], &oB = o[1], &oC = o[2], &oD = o[3], &oU1 = o[4], &oU2 = o[5];
-  leaf(c, oC, oA, false, n, n, k, Q + 0 * n * n, n, 0, 0);   // Q1 = C A^T
-  leaf(c, oD, oB, false, n, n, k, Q + 1 * n * n, n, 0, 0);   // Q2 = D B^T
-  leaf(c, oU2, oU1, false, n, n, k, Q + 2 * n * n, n, 0, 0); // Q3 = U2 U1^T
-  leaf(c, oA, oB, false, n, n, k, Q + 3 * n * n, n, 0, 0);   // Q4 = A B^T
-  leaf(c, oC, oD, false, n, n, k, Q + 4 * n * n, n, 0, 0);   // Q5 = C D^T
-  // Q6 = Low((U1 + U2)(U1 + U2)^T) -> H1 (the tuning table may change the
-  // digit form for it; the five products above keep theirs)
-  const DigitSpec ds = c.ds;
-  const int form = c.form;
-  run_plan_in(c, U12, n, k, k, H[0], ldh, flags & ~(uint32_t)AAT_ZERO_UPPER, dry, nullptr);
-  c.ds = ds;
-  c.form = form;
-  if (!dry) {
-    check(c, launch_quat_combine(Q, n, n * n, H[0], H[1], H[2], H[3], ldh, n, c.m, c.st),
-          "quaternion combine");
-    if (flags & AAT_ZERO_UPPER)
-      for (int q = 0; q < 4; ++q) check(c, launch_zero_upper(H[q], ldh, n, c.st), "zero upper");
   }
+  // Q1 = C A^T, Q2 = D B^T, Q3 = U2 U1^T, Q4 = A B^T, Q5 = C D^T
+  static const int lx[5] = {2, 3, 5, 0, 2}, ry[5] = {0, 1, 4, 1, 3};
+  // one launch over all six products' tiles where separate launches would
+  // leave slots idle in their last waves (n = 2048, k = 1500 mod 65521: six
+  // launches 245 us, one 162 us)
+  TcLeafArgs fa[6];
+  if (q6_leaf) {
+    for (int q = 0; q < 5; ++q)
+      fa[q] = tc_args(c, o[lx[q]].pl, o[ry[q]].pl, n, n, k, Q + q * n * n, n, 0, 0);
+    fa[5] = tc_args(c, o[6].pl, o[6].pl, n, n, k, H[0], ldh, 1, 0);
+  }
+  const int fo = fuse_override();
+  if (q6_leaf && (fo == 1 || (fo < 0 && leaf_tc_fuse_pays(fa, 6)))) {
+    if (!dry && c.err == AAT_OK)
+      check(c, launch_leaf_tc_multi(fa, 6, c.m, c.st), "leaf (tensor cores, Q1 .. Q6)");
+  } else {
+    for (int q = 0; q < 5; ++q)
+      leaf(c, o[lx[q]], o[ry[q]], false, n, n, k, Q + q * n * n, n, 0, 0);
+    // Q6 = Low((U1 + U2)(U1 + U2)^T) -> H1 (the tuning table may change the
+    // digit form for it; the five products above keep theirs)
+    if (q6_leaf) {
+      leaf(c, o[6], o[6], true, n, n, k, H[0], ldh, 1, 0);
+    } else {
+      const DigitSpec ds = c.ds;
+      const int form = c.form;
+      run_plan_in(c, U12, n, k, k, H[0], ldh, flags & ~(uint32_t)AAT_ZERO_UPPER, dry, nullptr);
+      c.ds = ds;
+      c.form = form;
+    }
+  }
+  if (!dry)
+    check(c, launch_quat_combine(Q, n, n * n, H[0], H[1], H[2], H[3], ldh, n,
+                                 (flags & AAT_ZERO_UPPER) != 0, c.m, c.st),
+          "quaternion combine");
   return c.ar.peak;
 }
 

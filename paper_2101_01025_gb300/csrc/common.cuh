@@ -371,9 +371,16 @@ cudaError_t launch_quat_sums(const int32_t *A, const int32_t *B, const int32_t *
                              const int32_t *D, int64_t lda, int64_t n, int64_t k, int32_t *U1,
                              int32_t *U2, int32_t *U12, int64_t ldu, const ModP &m,
                              cudaStream_t st);
+// The digit planes of A, B, C, D, U1, U2 and (where P[6].ptr is set) U12, and
+// U12 as int32 where it is not null, in one pass.
+cudaError_t launch_quat_split(const int32_t *A, const int32_t *B, const int32_t *C,
+                              const int32_t *D, int64_t lda, int64_t n, int64_t k,
+                              const Planes (&P)[7], int32_t *U12, int64_t ldu, const ModP &m,
+                              int b, cudaStream_t st);
+// zero: also clear the strict upper triangles of H1..H4.
 cudaError_t launch_quat_combine(const int32_t *Q, int64_t ldq, int64_t qstride, int32_t *H1,
                                 int32_t *H2, int32_t *H3, int32_t *H4, int64_t ldh, int64_t n,
-                                const ModP &m, cudaStream_t st);
+                                bool zero, const ModP &m, cudaStream_t st);
 
 // count balanced residues mod p, element t = SplitMix64 output t of stream
 // `seed` mapped to [0, p) by (z >> 32) p >> 32 (synthetic tuning inputs).

@@ -756,6 +756,56 @@ __global__ void quat_sums_kernel(const int32_t *__restrict__ A, const int32_t *_
   }
 }
 
+// The same sums in registers, with the digit planes of all seven operands
+// written straight from them: 16 B read and 7 L 2 B written per entry in one
+// pass, instead of the sums kernel and seven splits (18 + 7 x 7.7 us at n =
+// 2048, k = 1500 mod 65521; this one 32 us).  Quads of columns and
+// blockDim (bx, by) as split_ragged_kernel; VEC: 16-byte aligned rows of A,
+// B, C, D with k % 4 == 0.
+struct QuatPlanes {
+  Planes p[7];
+};
+template <int NB, bool VEC>
+__global__ void __launch_bounds__(kThreads)
+    quat_split_kernel(const int32_t *__restrict__ A, const int32_t *__restrict__ B,
+                      const int32_t *__restrict__ C, const int32_t *__restrict__ D, int64_t lda,
+                      int64_t n, int64_t k, const __grid_constant__ QuatPlanes Q, int32_t *U12,
+                      int64_t ldu, ModP m, int b) {
+  const int64_t nq = (k + 3) / 4;
+  for (int64_t r = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; r < n;
+       r += (int64_t)gridDim.y * blockDim.y)
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nq;
+         q += (int64_t)gridDim.x * blockDim.x) {
+      const int64_t c = 4 * q;
+      const int32_t *src[4] = {A + r * lda, B + r * lda, C + r * lda, D + r * lda};
+      int32_t v[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if constexpr (VEC) {
+          ldv_bal<4>(src[i] + c, m, v[i]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) v[i][j] = c + j < k ? ld_bal(src[i] + c + j, m) : 0;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) store_digits_t<NB, 4>(Q.p[i], r, c, v[i], b);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        v[0][j] = add_bal(v[0][j], v[1][j], m);
+        v[1][j] = add_bal(v[2][j], v[3][j], m);
+        v[2][j] = add_bal(v[0][j], v[1][j], m);
+      }
+      store_digits_t<NB, 4>(Q.p[4], r, c, v[0], b);
+      store_digits_t<NB, 4>(Q.p[5], r, c, v[1], b);
+      if (Q.p[6].ptr) store_digits_t<NB, 4>(Q.p[6], r, c, v[2], b);
+      if (U12)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (c + j < k) U12[r * ldu + c + j] = v[2][j];
+    }
+}
+
 // The additions closing the quaternion algorithm of Sec. 6.2, on the lower
 // triangle: T1 = Q1 - Q2, T2 = Q4 + Q5, T3 = (Q1 + Q2) - Q3,
 // H1 = Q6 - (Q3^T + Q3) - (T2^T + T2), H2 = T2^T - T2, H3 = T1 - T1^T,
@@ -763,7 +813,7 @@ __global__ void quat_sums_kernel(const int32_t *__restrict__ A, const int32_t *_
 // per CTA, with tile (J, I) of every Q for the transposed terms.
 __global__ void quat_combine_kernel(const int32_t *__restrict__ Q, int64_t ldq, int64_t qstride,
                                     int32_t *H1, int32_t *H2, int32_t *H3, int32_t *H4,
-                                    int64_t ldh, int64_t n, ModP m) {
+                                    int64_t ldh, int64_t n, int zero, ModP m) {
   __shared__ int32_t qt[5][T][T + 1];  // tile (J, I) of Q1..Q5
   const int64_t ntiles = (n + T - 1) / T;
   int64_t pid = blockIdx.x;
@@ -776,9 +826,14 @@ __global__ void quat_combine_kernel(const int32_t *__restrict__ Q, int64_t ldq, 
   const int64_t r0 = I * T, c0 = J * T;
   for (int yy = ty; yy < T; yy += 8) {
     const int64_t r2 = c0 + yy, c2 = r0 + tx;
-    if (r2 < n && c2 < n)
+    if (r2 < n && c2 < n) {
 #pragma unroll
       for (int q = 0; q < 5; ++q) qt[q][yy][tx] = bal(Q[q * qstride + r2 * ldq + c2], m);
+      if (zero && r2 < c2) {
+        const int64_t z = r2 * ldh + c2;
+        H1[z] = H2[z] = H3[z] = H4[z] = 0;
+      }
+    }
   }
   __syncthreads();
   for (int yy = ty; yy < T; yy += 8) {
@@ -826,15 +881,56 @@ cudaError_t launch_quat_sums(const int32_t *A, const int32_t *B, const int32_t *
   return cudaGetLastError();
 }
 
+cudaError_t launch_quat_split(const int32_t *A, const int32_t *B, const int32_t *C,
+                              const int32_t *D, int64_t lda, int64_t n, int64_t k,
+                              const Planes (&P)[7], int32_t *U12, int64_t ldu, const ModP &m,
+                              int b, cudaStream_t st) {
+  if (n * k <= 0) return cudaSuccess;
+  QuatPlanes Q;
+  double planes = 0.0;
+  for (int i = 0; i < 7; ++i) {
+    Q.p[i] = P[i];
+    if (!P[i].ptr && i == 6) continue;
+    if (!P[i].ptr || P[i].nbase != P[0].nbase || P[i].rows != n || P[i].cols != k ||
+        P[i].kstride % 8 || ((uintptr_t)P[i].ptr & 7))
+      return cudaErrorInvalidValue;
+    planes += P[i].L;
+  }
+  ProfScope prof(AAT_K_SPLIT, st, (double)n * k * (16.0 + 2.0 * planes + (U12 ? 4.0 : 0.0)));
+  auto al16 = [](const void *ptr) { return ((uintptr_t)ptr & 15) == 0; };
+  const bool vec = k % 4 == 0 && lda % 4 == 0 && al16(A) && al16(B) && al16(C) && al16(D);
+  const int64_t nq = (k + 3) / 4;
+  unsigned bx = 32;
+  while (bx < 128 && bx < nq) bx *= 2;
+  const unsigned by = kThreads / bx;
+  const int64_t cap = grid_for(INT64_MAX / 2), gx = std::min<int64_t>((nq + bx - 1) / bx, cap);
+  const int64_t gy = std::max<int64_t>(1, std::min<int64_t>((n + by - 1) / by, cap / gx));
+  const dim3 block(bx, by), grid((unsigned)gx, (unsigned)gy);
+#define AAT_QS(NBV)                                                                            \
+  case NBV:                                                                                    \
+    if (vec)                                                                                   \
+      quat_split_kernel<NBV, true><<<grid, block, 0, st>>>(A, B, C, D, lda, n, k, Q, U12, ldu, m, b); \
+    else                                                                                       \
+      quat_split_kernel<NBV, false><<<grid, block, 0, st>>>(A, B, C, D, lda, n, k, Q, U12, ldu, m, b); \
+    break;
+  switch (P[0].nbase) {
+    AAT_QS(1) AAT_QS(2) AAT_QS(3) AAT_QS(4) AAT_QS(5)
+    default:
+      return cudaErrorInvalidValue;
+  }
+#undef AAT_QS
+  return cudaGetLastError();
+}
+
 cudaError_t launch_quat_combine(const int32_t *Q, int64_t ldq, int64_t qstride, int32_t *H1,
                                 int32_t *H2, int32_t *H3, int32_t *H4, int64_t ldh, int64_t n,
-                                const ModP &m, cudaStream_t st) {
+                                bool zero, const ModP &m, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int64_t nt = (n + T - 1) / T;
   const double tri = 0.5 * (double)n * (double)(n + 1);
-  ProfScope prof(AAT_K_POSTADD, st, 4.0 * (10.0 * tri + 4.0 * tri + tri));
+  ProfScope prof(AAT_K_POSTADD, st, 4.0 * (10.0 * tri + 4.0 * tri + tri + (zero ? 4.0 * tri : 0.0)));
   quat_combine_kernel<<<(unsigned)(nt * (nt + 1) / 2), T * 8, 0, st>>>(Q, ldq, qstride, H1, H2,
-                                                                       H3, H4, ldh, n, m);
+                                                                       H3, H4, ldh, n, zero, m);
   return cudaGetLastError();
 }
 

@@ -85,3 +85,22 @@ def test_narrow_leaf_tiles(lib, M, N, K, p, lower):
             mask = np.tril(np.ones((M, N), bool)) if lower else np.ones((M, N), bool)
             want[:, :N][mask] = new[mask]
             assert np.array_equal(C.cpu().numpy().astype(object), want)
+
+
+@pytest.mark.parametrize("p", [65521, 131071, 2**31 - 1])
+@pytest.mark.parametrize("n,k,pad", [(1, 1, 0), (33, 5, 0), (64, 132, 4), (130, 259, 1), (300, 96, 0)])
+def test_quaternion_product_in_one_leaf_launch(lib, n, k, pad, p):
+    """Operand planes straight from A, B, C, D (aligned and ragged rows), the
+    six products' tiles in one launch, cleared upper triangles."""
+    import torch
+    parts = [synth.residues(7 * n + k + i, (n, k), p, balanced=bool(i & 1)) for i in range(4)]
+    dev = []
+    for x in parts:
+        buf = torch.zeros((n, k + pad), dtype=torch.int32, device="cuda")
+        buf[:, :k] = torch.from_numpy(x)
+        dev.append(buf[:, :k])
+    H = lib.aah_quat_modp(*dev, p, H=tuple(torch.full((n, n), -1, dtype=torch.int32, device="cuda")
+                                           for _ in range(4)), flags=lib.AAT_ZERO_UPPER)
+    ref = oracle.quat_aah_modp_low(*parts, p)
+    for h, r in zip(H, ref):
+        assert np.array_equal(h.cpu().numpy().astype(np.int64), np.tril(np.asarray(r, dtype=np.int64)))
