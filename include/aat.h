@@ -247,8 +247,11 @@ AAT_API int aat_gemm_modp_noalloc(const int32_t *X, int64_t ldx, const int32_t *
  * values split into BF16 pieces (x = x0 + x1 + x2, x0 = bf16(x),
  * x1 = bf16(x - x0), ...), piece products of weight >= 2^-16 kept, FP32
  * accumulation.  The precision flags name the accuracy class:
- *   AAT_C_FP32    FP32-accurate: 3 pieces, 6 piece products per real
- *                 product (relative Frobenius error <= 1e-5)
+ *   AAT_C_FP32    FP32-accurate (relative Frobenius error <= 1e-5): 2M on
+ *                 FP16 pieces of power-of-two scaled rows, 2 pieces and 3
+ *                 piece products per real product; on 3 BF16 pieces and 6
+ *                 piece products where a row's values spread too far for
+ *                 FP16 (decided on the device) and in Algorithm 1's levels
  *   AAT_C_BF16X3  2 pieces, 3 piece products (<= 1e-4)
  *   AAT_C_BF16    plain BF16 (<= 3e-3): one piece per input value; the 2M
  *                 form's sum operand (Ar + Ai or Ar - Ai) keeps 2 pieces (3
@@ -282,8 +285,9 @@ AAT_API int aat_complex_2m(const void *A, int64_t n, int64_t k, int64_t lda, voi
  * Y = i I (Sec. 4.1: multiplying by Y swaps real and imaginary parts with one
  * sign flip).  The general products P3, P4 use 3 real products (3M), the
  * recursion ends in Algorithm 2 (eps = -1).  flags: AAT_C_* precision, and
- * AAT_LEVELS(l) (no level bits: one level once n/2 >= 4096, k/2 >= 2048; no
- * level with AAT_C_BF16, which refuses AAT_LEVELS(l >= 1) with
+ * AAT_LEVELS(l) (no level bits: with AAT_C_BF16X3 one level once n/2 >= 4096,
+ * k/2 >= 2048; no level with AAT_C_FP32, where 2M is faster, nor with
+ * AAT_C_BF16, which refuses AAT_LEVELS(l >= 1) with
  * AAT_EUNSUPPORTED). */
 AAT_API int aat_complex(const void *A, int64_t n, int64_t k, void *C, void *stream);
 AAT_API int aat_complex_ex(const void *A, int64_t n, int64_t k, int64_t lda, void *C,

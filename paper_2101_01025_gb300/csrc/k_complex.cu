@@ -18,8 +18,24 @@
 // 8 K blocks into FP32 registers (round to nearest) while the next chunk
 // accumulates in the other TMEM buffer.  The Hermitian diagonal sum_l |a_il|^2 is
 // computed in FP64 (real and >= 0).
+//
+// FP16 pieces (2M in the FP32 class).  An FP16 piece carries 11 significant
+// bits where a BF16 piece carries 8, so two of them hold an FP32 value to
+// 2^-23 of itself and THREE piece products (x0y0, x0y1, x1y0; the dropped
+// x1y1 is below 2^-22 of the product) replace six, at the same tensor rate.
+// FP16's exponent range is the price: every row is scaled by a power of two
+// that brings its largest value into [2^13, 2^14) (row_stats_kernel; undone
+// exactly in the combine), and a value keeps full precision down to 2^-16 of
+// its row's largest.  The choice is made on the device, per product: when a
+// row's values lie on average (of their exponents) more than 2^8 below its
+// largest, or the row holds an Inf, a NaN or values near the ends of FP32's
+// range, the whole product runs on the six BF16 products instead
+// (`wide` != 0).  Relative Frobenius error against 64 bits at n = k = 8192,
+// N(0, 1): A A^H 1.8e-7 (3.4e-7 by the six BF16 products), A A^T by 2M 3.1e-7
+// (5.9e-7); 6.1 -> 3.5 ms, of it the leaf 5.4 -> 2.9 ms.
 #include <cuda.h>
 #include <cudaTypedefs.h>
+#include <cuda_fp16.h>
 
 #include <algorithm>
 #include <cstdint>
@@ -61,6 +77,7 @@ struct alignas(64) FJobDesc {
   float *out;
   int64_t ldo, M, N;
   int lower, kblocks, goff, ng;  // its groups: gtab[goff .. goff + ng)
+  const int32_t *wide;  // null: BF16 pieces; else FP16 pieces while *wide == 0
 };
 
 struct FParams {
@@ -88,9 +105,43 @@ struct FJob {
   const CUtensorMap *tmx, *tmy;
   const FGroup *g;
   int ng, kblocks, lower, I, J;
+  bool half;  // FP16 pieces: the first three groups only
   float *out;
   int64_t ldo, M, N;
+  // K blocks of the whole sum (all groups in turn), and the end of the chunk
+  // of one TMEM accumulation that starts at block q0
+  __device__ __forceinline__ int total() const { return ng * kblocks; }
+  __device__ __forceinline__ int chunk_end(int q0, int kchunk) const;
+  __device__ __forceinline__ int chunks(int kchunk) const;
+  // group gi of the sum
+  __device__ __forceinline__ const FGroup &group(int gi) const;
 };
+
+// FP16 pieces: x0y1 and x1y0 come first and x0y0, whose sums are 2^11 times
+// larger, last, so that the FP32 register that collects the chunks rounds at
+// full size only while x0y0 is added.  The tensor core truncates what falls
+// below an accumulator's last bit (x0y0 has 22 bits, where a BF16 product's
+// 16 bits fit), which short chunks keep small; the small terms take long ones.
+// Measured at n = k = 8192 (A A^H, every entry), x0y0 in chunks of 4 / 3 / 2 /
+// 1 K blocks: N(0, 1) parts 2.3 / 2.0 / 1.8 / 1.9e-7 (BF16: 3.4e-7), parts
+// uniform in [0, 1) 10 / 7.8 / 4.4 / 3.6e-7 (BF16: 4.4e-7), 3.44 / 3.49 / 3.54 /
+// 3.73 ms.
+constexpr int kHalfTerms = 3, kHalfSmall = 16, kHalfBig = 2;
+
+__device__ __forceinline__ int FJob::chunk_end(int q0, int kchunk) const {
+  if (!half) return min(q0 + kchunk, total());
+  const int small = (kHalfTerms - 1) * kblocks;
+  return q0 < small ? min(q0 + kHalfSmall, small) : min(q0 + kHalfBig, total());
+}
+__device__ __forceinline__ int FJob::chunks(int kchunk) const {
+  if (!half) return (total() + kchunk - 1) / kchunk;
+  const int small = (kHalfTerms - 1) * kblocks;
+  return (small + kHalfSmall - 1) / kHalfSmall + (total() - small + kHalfBig - 1) / kHalfBig;
+}
+__device__ __forceinline__ const FGroup &FJob::group(int gi) const {
+  return g[half ? (gi == kHalfTerms - 1 ? 0 : gi + 1) : gi];
+}
+
 
 template <bool BATCH>
 __device__ __forceinline__ FJob fjob(const FParams &P, int t) {
@@ -101,7 +152,8 @@ __device__ __forceinline__ FJob fjob(const FParams &P, int t) {
     j.tmx = &d.tmx;
     j.tmy = &d.tmy;
     j.g = P.gtab + d.goff;
-    j.ng = d.ng;
+    j.half = d.wide && *d.wide == 0;
+    j.ng = j.half ? kHalfTerms : d.ng;
     j.kblocks = d.kblocks;
     j.lower = d.lower;
     j.out = d.out;
@@ -116,6 +168,7 @@ __device__ __forceinline__ FJob fjob(const FParams &P, int t) {
     j.tmy = &P.tmy;
     j.g = P.g;
     j.ng = P.ng;
+    j.half = false;
     j.kblocks = P.kblocks;
     j.lower = P.lower;
     j.out = P.out;
@@ -149,8 +202,10 @@ struct FShape {
   static constexpr size_t XS_BYTES = (size_t)EPI_WARPS * 32 * 17 * 4;
   static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES + 256 + XS_BYTES;
   // kind::f16, FP32 accumulator, BF16 A and B, K-major, N = 256, M = TM
-  static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) |
-                                    ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+  // (IDESC_H: FP16 A and B)
+  static constexpr uint32_t IDESC_H =
+      (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+  static constexpr uint32_t IDESC = IDESC_H | (1u << 7) | (1u << 10);
 };
 
 template <bool PAIR, bool BATCH>
@@ -225,7 +280,7 @@ __global__ void __launch_bounds__(THREADS, 1) leaf_f32_kernel(const __grid_const
         const int rowx = jb.I * S::TM + (int)rank * BM;
         const int rowy = jb.J * BN + (int)rank * S::YROWS;
         for (int gi = 0; gi < jb.ng && ok; ++gi) {
-          const FGroup g = jb.g[gi];
+          const FGroup g = jb.group(gi);
           for (int kb = 0; kb < jb.kblocks; ++kb) {
             if (!wait_bounded<PAIR>(EMPTY(stage), ph ^ 1u, abort_flag, P.status)) {
               ok = false;
@@ -282,11 +337,12 @@ __global__ void __launch_bounds__(THREADS, 1) leaf_f32_kernel(const __grid_const
         const FJob jb = fjob<BATCH>(P, t);
         // chunks of kchunk K blocks over the flattened (group, K block)
         // sequence: a chunk may span two groups (one FP32 sum)
-        const int total = jb.ng * jb.kblocks;
+        const int total = jb.total();
         int gi = 0, kbi = 0;
-        uint32_t idesc = S::IDESC | ((jb.ng > 0 && jb.g[0].neg) ? NEG_A : 0u);
-        for (int q0 = 0; q0 < total && ok; q0 += P.kchunk) {
-          const int q1 = min(q0 + P.kchunk, total);
+        const uint32_t idesc0 = jb.half ? S::IDESC_H : S::IDESC;
+        uint32_t idesc = idesc0 | ((jb.ng > 0 && jb.group(0).neg) ? NEG_A : 0u);
+        for (int q0 = 0, q1; q0 < total && ok; q0 = q1) {
+          q1 = jb.chunk_end(q0, P.kchunk);
           const uint32_t buf = chunk & 1u, use = chunk >> 1;
           if (!__all_sync(0xffffffffu, wait_bounded<PAIR>(AEMPTY(buf), (use & 1u) ^ 1u, abort_flag,
                                                           P.status))) {
@@ -324,7 +380,7 @@ __global__ void __launch_bounds__(THREADS, 1) leaf_f32_kernel(const __grid_const
             }
             if (++kbi == jb.kblocks) {
               kbi = 0;
-              if (++gi < jb.ng) idesc = S::IDESC | (jb.g[gi].neg ? NEG_A : 0u);
+              if (++gi < jb.ng) idesc = idesc0 | (jb.group(gi).neg ? NEG_A : 0u);
             }
           }
           if (!ok) break;
@@ -359,7 +415,7 @@ __global__ void __launch_bounds__(THREADS, 1) leaf_f32_kernel(const __grid_const
     bool ok = true;
     for (int t = (int)unit0; t < P.ntiles && ok; t += (int)nunits) {
       const FJob jb = fjob<BATCH>(P, t);
-      const int nchunks = (jb.ng * jb.kblocks + P.kchunk - 1) / P.kchunk;
+      const int nchunks = jb.chunks(P.kchunk);
       float acc[128];
 #pragma unroll
       for (int i = 0; i < 128; ++i) acc[i] = 0.0f;
@@ -484,8 +540,9 @@ __device__ __forceinline__ void cload4(const float2 *__restrict__ a_row, int64_t
 // The pieces of 4 consecutive values a[0..nv) of row r, columns c0.., into
 // every plane set of o: one 8-byte store per plane (kstride is a multiple of
 // 8); a ragged last quad stores element by element.
+// sc != 0: two FP16 pieces of the values times sc (a power of two).
 __device__ __forceinline__ void csplit_store(const float2 (&a)[4], int64_t r, int64_t c0, int nv,
-                                             int np, const CSplitOut &o) {
+                                             int np, const CSplitOut &o, float sc = 0.0f) {
   const Planes *outs[4] = {&o.re, &o.im, &o.s, &o.d};
 #pragma unroll
   for (int w = 0; w < 4; ++w) {
@@ -498,53 +555,97 @@ __device__ __forceinline__ void csplit_store(const float2 (&a)[4], int64_t r, in
     // pieces of two values per conversion instruction (round to nearest),
     // the rest carried in FP32 (exact: each rest is an FP32 difference of a
     // value and its BF16 rounding)
-    __nv_bfloat162 lo[3], hi[3];
+    uint2 pc[3];  // piece q of the four values, 16 bits each
+    const int nq = sc != 0.0f ? 2 : np;
+    if (sc != 0.0f) {
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      if (q < np) {
-        lo[q] = __floats2bfloat162_rn(x[0], x[1]);
-        hi[q] = __floats2bfloat162_rn(x[2], x[3]);
-        const float2 fl = __bfloat1622float2(lo[q]), fh = __bfloat1622float2(hi[q]);
+      for (int v = 0; v < 4; ++v) x[v] *= sc;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        __half2 lo = __floats2half2_rn(x[0], x[1]), hi = __floats2half2_rn(x[2], x[3]);
+        pc[q].x = *reinterpret_cast<uint32_t *>(&lo);
+        pc[q].y = *reinterpret_cast<uint32_t *>(&hi);
+        const float2 fl = __half22float2(lo), fh = __half22float2(hi);
         x[0] -= fl.x;
         x[1] -= fl.y;
         x[2] -= fh.x;
         x[3] -= fh.y;
       }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        if (q < np) {
+          __nv_bfloat162 lo = __floats2bfloat162_rn(x[0], x[1]);
+          __nv_bfloat162 hi = __floats2bfloat162_rn(x[2], x[3]);
+          pc[q].x = *reinterpret_cast<uint32_t *>(&lo);
+          pc[q].y = *reinterpret_cast<uint32_t *>(&hi);
+          const float2 fl = __bfloat1622float2(lo), fh = __bfloat1622float2(hi);
+          x[0] -= fl.x;
+          x[1] -= fl.y;
+          x[2] -= fh.x;
+          x[3] -= fh.y;
+        }
+      }
     }
     const int64_t plane = P.rows * P.kstride;
-    __nv_bfloat16 *dst = P.ptr + r * P.kstride + c0;
-    for (int q = 0; q < np; ++q) {
+    uint16_t *dst = reinterpret_cast<uint16_t *>(P.ptr) + r * P.kstride + c0;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      if (q >= nq) break;
       if (nv == 4) {
-        uint2 u;
-        u.x = *reinterpret_cast<uint32_t *>(&lo[q]);
-        u.y = *reinterpret_cast<uint32_t *>(&hi[q]);
-        *reinterpret_cast<uint2 *>(dst + q * plane) = u;
+        *reinterpret_cast<uint2 *>(dst + q * plane) = pc[q];
       } else {
-        const __nv_bfloat16 pv[4] = {lo[q].x, lo[q].y, hi[q].x, hi[q].y};
+        const uint16_t pv[4] = {(uint16_t)pc[q].x, (uint16_t)(pc[q].x >> 16), (uint16_t)pc[q].y,
+                                (uint16_t)(pc[q].y >> 16)};
         for (int v = 0; v < nv; ++v) dst[q * plane + v] = pv[v];
       }
     }
   }
 }
 
+// What the FP16 form of a product keeps per row: the scale's exponent e (the
+// row is stored times 2^-e), the exact diagonal entry (A A^H), and one flag
+// for the whole product.  e == null: BF16 pieces.
+struct RowScale {
+  int32_t *e;
+  float *diag;
+  int32_t *wide;
+};
+
+__device__ __forceinline__ float exp2i(int e) { return __int_as_float((e + 127) << 23); }
+
+// 2^-e of row r, or 0 when the product runs on BF16 pieces.
+__device__ __forceinline__ float row_scale(const RowScale &s, int64_t r) {
+  return (s.e && *s.wide == 0) ? exp2i(-s.e[r]) : 0.0f;
+}
+
+// v 2^(ei + ej) with the exponent applied in two halves of one sign.
+__device__ __forceinline__ float unscale(float v, int ei, int ej) {
+  const int t = ei + ej, h = t / 2;
+  return v * exp2i(h) * exp2i(t - h);
+}
+
 // One thread per 4 consecutive columns of a row (rows over blockIdx.y, a
 // grid-stride loop over column quads).
 __device__ __forceinline__ void csplit_quad(const float2 *__restrict__ a_row, int64_t r,
-                                            int64_t q4, int64_t cols, int np, const CSplitOut &o) {
+                                            int64_t q4, int64_t cols, int np, const CSplitOut &o,
+                                            float sc) {
   const int64_t c0 = 4 * q4;
   const int nv = (int)min((int64_t)4, cols - c0);
   float2 a[4];
   cload4(a_row, c0, nv, a);
-  csplit_store(a, r, c0, nv, np, o);
+  csplit_store(a, r, c0, nv, np, o, sc);
 }
 
 __global__ void csplit_kernel(const float2 *__restrict__ A, int64_t lda, int64_t rows, int64_t cols,
-                              int np, CSplitOut o) {
+                              int np, CSplitOut o, RowScale rs) {
   const int64_t cq = (cols + 3) / 4;
-  for (int64_t r = blockIdx.y; r < rows; r += gridDim.y)
+  for (int64_t r = blockIdx.y; r < rows; r += gridDim.y) {
+    const float sc = row_scale(rs, r);
     for (int64_t q4 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q4 < cq;
          q4 += (int64_t)gridDim.x * blockDim.x)
-      csplit_quad(A + r * lda, r, q4, cols, np, o);
+      csplit_quad(A + r * lda, r, q4, cols, np, o, sc);
+  }
 }
 
 // ------------------------------------------------ batched A A^H / A A^T (2M)
@@ -560,6 +661,7 @@ struct CBProb {
   float *H, *G;
   float2 *C;
   int64_t ldc;
+  RowScale rs;
   int split_first, comb_first, diag_first;
 };
 
@@ -588,8 +690,9 @@ __global__ void csplit_batch_kernel(const CBProb *__restrict__ pr, int count) {
   for (uint32_t t = threadIdx.x; t < nr * cq; t += blockDim.x) {
     const uint32_t ri = t / cq;
     const int64_t r = r0 + ri, q4 = t - ri * cq;
-    csplit_quad(q.A + r * q.lda, r, q4, q.k, q.np, q.ox);
-    csplit_quad(q.A + r * q.lda, r, q4, q.k, q.np, q.oy);
+    const float sc = row_scale(q.rs, r);
+    csplit_quad(q.A + r * q.lda, r, q4, q.k, q.np, q.ox, sc);
+    csplit_quad(q.A + r * q.lda, r, q4, q.k, q.np, q.oy, sc);
   }
 }
 
@@ -600,7 +703,8 @@ constexpr int T = 32;
 __device__ __forceinline__ void combine2m_tile(const float *__restrict__ G,
                                                const float *__restrict__ H, int64_t ldw,
                                                int64_t n, float2 *C, int64_t ldc, int herm,
-                                               int64_t pid, float (&hij)[T][T + 1],
+                                               const RowScale &rs, int64_t pid,
+                                               float (&hij)[T][T + 1],
                                                float (&hji)[T][T + 1]) {
   const int64_t ntiles = (n + T - 1) / T;
   int64_t I, J;
@@ -608,6 +712,7 @@ __device__ __forceinline__ void combine2m_tile(const float *__restrict__ G,
   if (I >= ntiles) return;
   const int tx = threadIdx.x % T, ty = threadIdx.x / T;
   const int64_t r0 = I * T, c0 = J * T;
+  const bool half = rs.e && *rs.wide == 0;
   for (int yy = ty; yy < T; yy += 8) {
     int64_t r = r0 + yy, c = c0 + tx;
     if (r < n && c < n) hij[yy][tx] = H[r * ldw + c];
@@ -627,24 +732,31 @@ __device__ __forceinline__ void combine2m_tile(const float *__restrict__ G,
         v.x = g + h - ht;
         v.y = h + ht;
       }
+      if (half) {
+        const int ei = rs.e[r], ej = rs.e[c];
+        v.x = unscale(v.x, ei, ej);
+        v.y = unscale(v.y, ei, ej);
+      }
+      if (rs.diag && r == c) v = make_float2(rs.diag[r], 0.0f);
       C[r * ldc + c] = v;
     }
   }
 }
 
 __global__ void combine2m_kernel(const float *__restrict__ G, const float *__restrict__ H,
-                                 int64_t ldw, int64_t n, float2 *C, int64_t ldc, int herm) {
+                                 int64_t ldw, int64_t n, float2 *C, int64_t ldc, int herm,
+                                 RowScale rs) {
   __shared__ float hij[T][T + 1];
   __shared__ float hji[T][T + 1];
-  combine2m_tile(G, H, ldw, n, C, ldc, herm, blockIdx.x, hij, hji);
+  combine2m_tile(G, H, ldw, n, C, ldc, herm, rs, blockIdx.x, hij, hji);
 }
 
 __global__ void combine2m_batch_kernel(const CBProb *__restrict__ pr, int count) {
   __shared__ float hij[T][T + 1];
   __shared__ float hji[T][T + 1];
   const CBProb &q = pr[cb_find(pr, count, blockIdx.x, 1)];
-  combine2m_tile(q.G, q.H, q.n, q.n, q.C, q.ldc, q.herm, (int64_t)(blockIdx.x - q.comb_first),
-                 hij, hji);
+  combine2m_tile(q.G, q.H, q.n, q.n, q.C, q.ldc, q.herm, q.rs,
+                 (int64_t)(blockIdx.x - q.comb_first), hij, hji);
 }
 
 // x·x added to the unevaluated float pair hi + lo without rounding error:
@@ -661,20 +773,42 @@ __device__ __forceinline__ void sq_acc(float x, float &hi, float &lo) {
   lo = __fadd_rn(lo, __fadd_rn(err, e));
 }
 
-// Re C[row][row] = Σ_l |a_l|², one warp per row.  Each lane sums its
-// columns' squares as a float pair (about 48 significant bits: the only
-// rounding is in lo, whose terms are each below ulp(hi)), two pairs per lane
-// for the real and imaginary parts so the two dependency chains overlap;
-// the lanes' pairs are added in FP64.  This part's FP64 pipe is a small
-// fraction of its FP32 pipe: an FP64 multiply-add per square (and two
-// conversions) held the kernel far below the memory rate.
-__device__ __forceinline__ void herm_diag_row(const float2 *__restrict__ A, int64_t lda,
-                                              int64_t n, int64_t k, float2 *C, int64_t ldc,
-                                              int64_t row) {
+// What one lane has seen of its row: the squares' sum as two float pairs
+// (about 48 significant bits: the only rounding is in the low words, whose
+// terms are each below an ulp of the high ones; one pair each for the real
+// and imaginary parts so the two dependency chains overlap), the largest
+// magnitude's bits, and the biased exponents' sum over the nonzero values.
+struct RowAcc {
+  float h0, l0, h1, l1;
+  uint32_t mx, esum, nz;
+};
+
+template <bool DIAG, bool SCALE>
+__device__ __forceinline__ void row_acc(float2 v, RowAcc &a) {
+  if constexpr (DIAG) {
+    sq_acc(v.x, a.h0, a.l0);
+    sq_acc(v.y, a.h1, a.l1);
+  }
+  if constexpr (SCALE) {
+    const uint32_t x = __float_as_uint(v.x) & 0x7fffffffu, y = __float_as_uint(v.y) & 0x7fffffffu;
+    a.mx = max(a.mx, max(x, y));
+    a.esum += (x >> 23) + (y >> 23);  // a lane sees fewer than 2^23 values
+    a.nz += (x != 0u) + (y != 0u);
+  }
+}
+
+// One warp per row.  DIAG: Σ_l |a_l|², the lanes' pairs added in FP64 (this
+// part's FP64 pipe is a small fraction of its FP32 pipe: an FP64 multiply-add
+// per square held the kernel far below the memory rate).  SCALE: the row's
+// scale exponent, and the product's `wide` flag when the row needs BF16's
+// exponent range.  The diagonal goes to rs.diag.
+template <bool DIAG, bool SCALE>
+__device__ __forceinline__ void row_stats(const float2 *__restrict__ A, int64_t lda, int64_t n,
+                                          int64_t k, const RowScale &rs, int64_t row) {
   const int lane = threadIdx.x & 31;
   if (row >= n) return;
   const float2 *a_row = A + row * lda;
-  float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
+  RowAcc a = {0.f, 0.f, 0.f, 0.f, 0u, 0u, 0u};
   int64_t l = 0;
   if ((reinterpret_cast<uintptr_t>(a_row) & 15) == 0) {
     // two complex values per lane per 16-byte load, four loads in flight
@@ -682,38 +816,67 @@ __device__ __forceinline__ void herm_diag_row(const float2 *__restrict__ A, int6
     const int64_t k2 = k / 2;
     int64_t q = lane;
     for (; q + 96 < k2; q += 128) {
-      const float4 v0 = a4[q], v1 = a4[q + 32], v2 = a4[q + 64], v3 = a4[q + 96];
-      sq_acc(v0.x, h0, l0); sq_acc(v0.y, h1, l1); sq_acc(v0.z, h0, l0); sq_acc(v0.w, h1, l1);
-      sq_acc(v1.x, h0, l0); sq_acc(v1.y, h1, l1); sq_acc(v1.z, h0, l0); sq_acc(v1.w, h1, l1);
-      sq_acc(v2.x, h0, l0); sq_acc(v2.y, h1, l1); sq_acc(v2.z, h0, l0); sq_acc(v2.w, h1, l1);
-      sq_acc(v3.x, h0, l0); sq_acc(v3.y, h1, l1); sq_acc(v3.z, h0, l0); sq_acc(v3.w, h1, l1);
+      float4 v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = a4[q + 32 * i];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        row_acc<DIAG, SCALE>(make_float2(v[i].x, v[i].y), a);
+        row_acc<DIAG, SCALE>(make_float2(v[i].z, v[i].w), a);
+      }
     }
     for (; q < k2; q += 32) {
       const float4 v = a4[q];
-      sq_acc(v.x, h0, l0); sq_acc(v.y, h1, l1); sq_acc(v.z, h0, l0); sq_acc(v.w, h1, l1);
+      row_acc<DIAG, SCALE>(make_float2(v.x, v.y), a);
+      row_acc<DIAG, SCALE>(make_float2(v.z, v.w), a);
     }
     l = 2 * k2;  // an odd last column is left to the loop below
   }
-  for (l += lane; l < k; l += 32) {
-    const float2 a = a_row[l];
-    sq_acc(a.x, h0, l0);
-    sq_acc(a.y, h1, l1);
+  for (l += lane; l < k; l += 32) row_acc<DIAG, SCALE>(a_row[l], a);
+  if constexpr (DIAG) {
+    double s = ((double)a.h0 + (double)a.l0) + ((double)a.h1 + (double)a.l1);
+    for (int off = 16; off; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+    if (lane == 0) rs.diag[row] = (float)s;
   }
-  double s = ((double)h0 + (double)l0) + ((double)h1 + (double)l1);
-  for (int off = 16; off; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-  if (lane == 0) C[row * ldc + row] = make_float2((float)s, 0.0f);
+  if constexpr (SCALE) {
+    const uint32_t mx = __reduce_max_sync(0xffffffffu, a.mx);
+    unsigned long long es = a.esum, nz = a.nz;
+    for (int off = 16; off; off >>= 1) {
+      es += __shfl_down_sync(0xffffffffu, es, off);
+      nz += __shfl_down_sync(0xffffffffu, nz, off);
+    }
+    if (lane == 0) {
+      const int E = (int)(mx >> 23);
+      const bool zero = mx == 0u;
+      // average exponent of the nonzero values against the largest one's
+      const bool spread = (unsigned long long)E * nz > es + 8ull * nz;
+      if (!zero && (E < 24 || E > 230 || spread)) atomicOr(rs.wide, 1);
+      rs.e[row] = zero ? 0 : min(max(E - 127 - 13, -120), 120);
+    }
+  }
 }
 
-__global__ void herm_diag_kernel(const float2 *__restrict__ A, int64_t lda, int64_t n, int64_t k,
-                                 float2 *C, int64_t ldc) {
-  herm_diag_row(A, lda, n, k, C, ldc, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32);
+__global__ void row_stats_kernel(const float2 *__restrict__ A, int64_t lda, int64_t n, int64_t k,
+                                 RowScale rs) {
+  const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
+  if (rs.diag && rs.e)
+    row_stats<true, true>(A, lda, n, k, rs, row);
+  else if (rs.diag)
+    row_stats<true, false>(A, lda, n, k, rs, row);
+  else
+    row_stats<false, true>(A, lda, n, k, rs, row);
 }
 
-// one warp per row, kDiagRows rows of one Hermitian problem per block
-__global__ void herm_diag_batch_kernel(const CBProb *__restrict__ pr, int count) {
+// one warp per row, kDiagRows rows of one problem per block
+__global__ void row_stats_batch_kernel(const CBProb *__restrict__ pr, int count) {
   const CBProb &q = pr[cb_find(pr, count, blockIdx.x, 2)];
   const int64_t row = (int64_t)(blockIdx.x - q.diag_first) * kDiagRows + threadIdx.x / 32;
-  herm_diag_row(q.A, q.lda, q.n, q.k, q.C, q.ldc, row);
+  if (q.rs.diag && q.rs.e)
+    row_stats<true, true>(q.A, q.lda, q.n, q.k, q.rs, row);
+  else if (q.rs.diag)
+    row_stats<true, false>(q.A, q.lda, q.n, q.k, q.rs, row);
+  else if (q.rs.e)
+    row_stats<false, true>(q.A, q.lda, q.n, q.k, q.rs, row);
 }
 
 // ------------------------------------------------------------------ host
@@ -991,8 +1154,10 @@ std::map<int, bool> g_fattr[2];
 // the tiles fill every co-resident pair), so that no product's last wave
 // leaves SMs idle.  table_mem: fused_table_bytes() of device memory, 256-byte
 // aligned, for the job table.
+// wide: the products' FP16 / BF16 flag (null: BF16).
 static cudaError_t launch_leaf_f32_fused(const std::vector<FusedJob> &jobs, int np, int64_t K,
-                                         void *table_mem, cudaStream_t st) {
+                                         void *table_mem, cudaStream_t st,
+                                         const int32_t *wide = nullptr) {
   const int nj = (int)jobs.size();
   if (nj < 1 || nj > MAX_FUSED || K <= 0) return cudaErrorInvalidValue;
   std::lock_guard<std::mutex> lock(g_mu_c);
@@ -1027,6 +1192,7 @@ static cudaError_t launch_leaf_f32_fused(const std::vector<FusedJob> &jobs, int 
     d.N = j.N;
     d.lower = j.lower;
     d.kblocks = kblocks;
+    d.wide = wide;
     d.goff = T->ng;
     int pairs[6][2];
     const int npairs = piece_pairs(std::min(j.keep, np), pairs);
@@ -1370,7 +1536,7 @@ static Planes subset(const Planes &P, int set, int np) {
 }
 
 static void csplit(CCtx &c, const float2 *A, int64_t lda, int64_t rows, int64_t cols,
-                   const CSplitOut &o) {
+                   const CSplitOut &o, const RowScale &rs = RowScale{}) {
   if (c.ar.dry) return;
   int nsets = (o.re.ptr != nullptr) + (o.im.ptr != nullptr) + (o.s.ptr != nullptr) +
               (o.d.ptr != nullptr);
@@ -1378,7 +1544,7 @@ static void csplit(CCtx &c, const float2 *A, int64_t lda, int64_t rows, int64_t 
   const int64_t cq = (cols + 3) / 4;
   const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>((cq + 255) / 256, 64)),
                   (unsigned)std::max<int64_t>(1, std::min<int64_t>(rows, 65535)));
-  csplit_kernel<<<grid, 256, 0, c.st>>>(A, lda, rows, cols, c.np, o);
+  csplit_kernel<<<grid, 256, 0, c.st>>>(A, lda, rows, cols, c.np, o, rs);
   cchk(c, cudaGetLastError(), "complex split");
 }
 
@@ -1394,7 +1560,20 @@ static void c_two_m(CCtx &c, const float2 *A, int64_t lda, int64_t n, int64_t k,
   float *H = (float *)c.ar.get((size_t)n * n * 4);
   float *G = (float *)c.ar.get((size_t)n * n * 4);
   void *table = c.ar.get(fused_table_bytes());
+  // FP32 class (three pieces): FP16 pieces, decided on the device
+  RowScale rs = {};
+  if (c.np == 3) {
+    rs.e = (int32_t *)c.ar.get((size_t)(n + 1) * 4);
+    rs.wide = rs.e + n;
+  }
+  if (herm) rs.diag = (float *)c.ar.get((size_t)n * 4);
   if (!c.ar.dry) {
+    if (rs.e || rs.diag) {
+      if (rs.e) cchk(c, cudaMemsetAsync(rs.wide, 0, 4, c.st), "row flag");
+      ProfScope prof(AAT_K_COPY, c.st, (double)n * k * 8.0);
+      row_stats_kernel<<<(unsigned)((n * 32 + 255) / 256), 256, 0, c.st>>>(A, lda, n, k, rs);
+      cchk(c, cudaGetLastError(), "row scales and diagonal");
+    }
     // every piece set in one pass over A
     CSplitOut o;
     std::memset(&o, 0, sizeof(o));
@@ -1402,26 +1581,21 @@ static void c_two_m(CCtx &c, const float2 *A, int64_t lda, int64_t n, int64_t k,
     o.s = Xs;
     o.im = Yi;
     if (!herm) o.d = Ysd;
-    csplit(c, A, lda, n, k, o);
+    csplit(c, A, lda, n, k, o, rs);
     // H = Ar Ai^T (all entries) and G = (Ar + Ai)(Ar +- Ai)^T (lower tiles)
     // in one launch; G's sum operands keep every stored piece
     if (c.err == AAT_OK) {
       const std::vector<FusedJob> jobs = {
           FusedJob{&X, &Y, 0, 0, c.keep, H, n, n, n, 0},
           FusedJob{&X, herm ? &X : &Y, 1, 1, c.np, G, n, n, n, 1}};
-      cchk(c, launch_leaf_f32_fused(jobs, c.np, k, table, c.st), "2M H and G");
+      cchk(c, launch_leaf_f32_fused(jobs, c.np, k, table, c.st, rs.wide), "2M H and G");
     }
     if (c.err == AAT_OK) {
       const int64_t nt = (n + T - 1) / T;
       ProfScope prof(AAT_K_POSTADD, c.st, (double)n * n * (4.0 * 1.5 + 8.0 * 0.5));
       combine2m_kernel<<<(unsigned)(nt * (nt + 1) / 2), T * 8, 0, c.st>>>(G, H, n, n, C, ldc,
-                                                                           herm);
+                                                                           herm, rs);
       cchk(c, cudaGetLastError(), "2M combine");
-    }
-    if (herm && c.err == AAT_OK) {
-      ProfScope prof(AAT_K_COPY, c.st, (double)n * k * 8.0);
-      herm_diag_kernel<<<(unsigned)((n * 32 + 255) / 256), 256, 0, c.st>>>(A, lda, n, k, C, ldc);
-      cchk(c, cudaGetLastError(), "Hermitian diagonal");
     }
   }
   c.ar.used = mark;
@@ -1556,9 +1730,9 @@ static void c_last_level_fused(CCtx &c, const float2 *A, int64_t lda, int64_t n,
     if (c.err == AAT_OK) {
       ProfScope prof(AAT_K_POSTADD, c.st, 2.0 * (double)h * h * (4.0 * 1.5 + 8.0 * 0.5));
       combine2m_kernel<<<(unsigned)(nt * (nt + 1) / 2), T * 8, 0, c.st>>>(Gb[0], Hb[0], h, h, C12,
-                                                                          ldc, 0);
+                                                                          ldc, 0, RowScale{});
       combine2m_kernel<<<(unsigned)(nt * (nt + 1) / 2), T * 8, 0, c.st>>>(Gb[1], Hb[1], h, h, C11,
-                                                                          ldc, 0);
+                                                                          ldc, 0, RowScale{});
       cchk(c, cudaGetLastError(), "2M combine");
     }
     if (c.err == AAT_OK) {  // U4 -> C21, Low(U5) -> C22
@@ -1570,7 +1744,7 @@ static void c_last_level_fused(CCtx &c, const float2 *A, int64_t lda, int64_t n,
     if (c.err == AAT_OK) {  // P2 -> C12, Low(U3) = Low(P1 + P2) -> C11
       ProfScope prof(AAT_K_POSTADD, c.st, (double)h * h * (4.0 * 1.5 + 8.0 * 0.5));
       combine2m_kernel<<<(unsigned)(nt * (nt + 1) / 2), T * 8, 0, c.st>>>(Gb[2], Hb[2], h, h, C12,
-                                                                          ldc, 0);
+                                                                          ldc, 0, RowScale{});
       cchk(c, cudaGetLastError(), "2M combine");
     }
     if (c.err == AAT_OK) {
@@ -1682,6 +1856,9 @@ static int complex_levels(int64_t n, int64_t k, uint32_t flags) {
   const uint32_t lv = (flags & AAT_LEVELS_MASK) >> 8;
   if (lv) return (int)lv - 1;
   if ((flags & AAT_C_PREC_MASK) == AAT_C_BF16) return 0;  // see bf16_levels_ok
+  // FP32 class: 2M's three FP16 products take less than a level's BF16 ones
+  // (n = k = 8192: 3.5 against 5.8 ms), with a smaller error (3.1e-7, 9.7e-7)
+  if ((flags & AAT_C_PREC_MASK) == AAT_C_FP32) return 0;
   int levels = 0;  // one level pays off once the leaves stay large
   while (levels < 4 && (n >> (levels + 1)) >= 4096 && (k >> (levels + 1)) >= 2048) ++levels;
   return levels;
@@ -1695,6 +1872,7 @@ struct CBatchImpl {
   FGroup *gtab = nullptr;
   int4 *tiles = nullptr;
   int count = 0, ntiles = 0;
+  int32_t *flags = nullptr;  // one FP16 / BF16 flag per problem (workspace)
   int split_blocks = 0, comb_blocks = 0, diag_blocks = 0;
   double leaf_work = 0.0, split_bytes = 0.0, comb_bytes = 0.0, diag_bytes = 0.0;
 };
@@ -1706,10 +1884,11 @@ static size_t cb_planes_bytes(int64_t n, int64_t k, int np) {
 }
 
 size_t cbatch_workspace(const CBInput *in, int count) {
-  size_t total = 0;
+  size_t total = r256c((size_t)count * 4);
   for (int i = 0; i < count; ++i) {
     const int np = pieces_for(in[i].flags);
-    total += 2 * cb_planes_bytes(in[i].n, in[i].k, np) + 2 * r256c((size_t)in[i].n * in[i].n * 4);
+    total += 2 * cb_planes_bytes(in[i].n, in[i].k, np) +
+             2 * r256c((size_t)in[i].n * in[i].n * 4) + 2 * r256c((size_t)in[i].n * 4);
   }
   return total;
 }
@@ -1735,6 +1914,8 @@ cudaError_t cbatch_build(const CBInput *in, int count, char *ws, CBatch *out) {
   CBatchImpl *L = new CBatchImpl;
   L->count = count;
   char *w = ws;
+  L->flags = (int32_t *)w;
+  w += r256c((size_t)count * 4);
   int sb = 0, cbk = 0, db = 0;
   for (int i = 0; i < count; ++i) {
     const CBInput &q = in[i];
@@ -1756,6 +1937,13 @@ cudaError_t cbatch_build(const CBInput *in, int count, char *ws, CBatch *out) {
     w += r256c((size_t)q.n * q.n * 4);
     b.G = (float *)w;
     w += r256c((size_t)q.n * q.n * 4);
+    if (np == 3) {  // as c_two_m
+      b.rs.e = (int32_t *)w;
+      b.rs.wide = L->flags + i;
+    }
+    w += r256c((size_t)q.n * 4);
+    if (q.herm) b.rs.diag = (float *)w;
+    w += r256c((size_t)q.n * 4);
     b.A = q.A;
     b.lda = q.lda;
     b.n = q.n;
@@ -1774,10 +1962,10 @@ cudaError_t cbatch_build(const CBInput *in, int count, char *ws, CBatch *out) {
     b.comb_first = cbk;
     cbk += (int)(nt * (nt + 1) / 2);
     b.diag_first = db;
-    if (q.herm) db += (int)((q.n + kDiagRows - 1) / kDiagRows);
+    db += (int)((q.n + kDiagRows - 1) / kDiagRows);
     L->split_bytes += (double)q.n * q.k * (8.0 + 2.0 * np * (q.herm ? 3 : 4));
     L->comb_bytes += (double)q.n * q.n * (4.0 * 1.5 + 8.0 * 0.5);
-    if (q.herm) L->diag_bytes += (double)q.n * q.k * 8.0;
+    if (b.rs.e || b.rs.diag) L->diag_bytes += (double)q.n * q.k * 8.0;
     // two jobs: H = Ar Ai^T (all entries) from plane sets 0, G (lower) from
     // sets 1; G's sum operands keep every stored piece
     for (int jb = 0; jb < 2; ++jb) {
@@ -1801,6 +1989,7 @@ cudaError_t cbatch_build(const CBInput *in, int count, char *ws, CBatch *out) {
       d.M = d.N = q.n;
       d.lower = jb;
       d.kblocks = (int)((q.k + BK - 1) / BK);
+      d.wide = b.rs.wide;
       d.goff = (int)gtab.size();
       d.ng = npairs;
       for (int qq = 0; qq < npairs; ++qq) {
@@ -1863,6 +2052,12 @@ cudaError_t cbatch_launch(const CBatch &b, cudaStream_t st) {
   const CBatchImpl *L = (const CBatchImpl *)b.impl;
   if (!L || L->count == 0) return cudaSuccess;
   cudaError_t e;
+  if (L->diag_blocks > 0) {
+    if ((e = cudaMemsetAsync(L->flags, 0, (size_t)L->count * 4, st)) != cudaSuccess) return e;
+    ProfScope prof(AAT_K_COPY, st, L->diag_bytes);
+    row_stats_batch_kernel<<<(unsigned)L->diag_blocks, 256, 0, st>>>(L->probs, L->count);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
   if (L->split_blocks > 0) {
     ProfScope prof(AAT_K_SPLIT, st, L->split_bytes);
     csplit_batch_kernel<<<(unsigned)L->split_blocks, 256, 0, st>>>(L->probs, L->count);
@@ -1891,11 +2086,6 @@ cudaError_t cbatch_launch(const CBatch &b, cudaStream_t st) {
   if (L->comb_blocks > 0) {
     ProfScope prof(AAT_K_POSTADD, st, L->comb_bytes);
     combine2m_batch_kernel<<<(unsigned)L->comb_blocks, T * 8, 0, st>>>(L->probs, L->count);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  if (L->diag_blocks > 0) {
-    ProfScope prof(AAT_K_COPY, st, L->diag_bytes);
-    herm_diag_batch_kernel<<<(unsigned)L->diag_blocks, 256, 0, st>>>(L->probs, L->count);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;

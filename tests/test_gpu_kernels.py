@@ -104,3 +104,78 @@ def test_quaternion_product_in_one_leaf_launch(lib, n, k, pad, p):
     ref = oracle.quat_aah_modp_low(*parts, p)
     for h, r in zip(H, ref):
         assert np.array_equal(h.cpu().numpy().astype(np.int64), np.tril(np.asarray(r, dtype=np.int64)))
+
+
+def _row_relative(got, A, herm):
+    """Largest |error| of a lower entry against |a_i| |a_j| (FP64)."""
+    Z = A.astype(np.complex128)
+    ref = Z @ (Z.conj() if herm else Z).T
+    nrm = np.sqrt((np.abs(Z) ** 2).sum(1))
+    scale = np.outer(nrm, nrm)
+    scale[scale == 0] = 1
+    err = np.abs(np.tril(np.where(scale < 1e37, got - ref, 0)) / scale)  # finite in FP32
+    return err.max()
+
+
+def _complex_rows(n, k, kind):
+    rng = np.random.default_rng(n * 131 + k)
+    A = rng.standard_normal((n, k)) + 1j * rng.standard_normal((n, k))
+    if kind == "row_scales":    # one power of ten per row, 1e-15 .. 1e15
+        A *= 10.0 ** rng.uniform(-15, 15, (n, 1))
+    elif kind == "col_scales":  # every row spans 1e-6 .. 1e6
+        A *= 10.0 ** rng.uniform(-6, 6, (1, k))
+    elif kind == "zero_rows":
+        A[::3] = 0
+    elif kind == "huge_row":    # near the end of FP32's range
+        A[0] *= 1e32
+    return A.astype(np.complex64)
+
+
+# FP32 class: pieces of 2^-23, dropped products of 2^-22, and FP32 sums of at
+# most 512 products per drain, each a rounding of 2^-24 of a partial sum that
+# stays below |a_i| |a_j|: (2 + 2 + 4) 2^-23 at the outside of their random
+# sizes, 1e-6, taken twice
+@pytest.mark.parametrize("kind", ["normal", "row_scales", "col_scales", "zero_rows", "huge_row"])
+@pytest.mark.parametrize("n,k", [(1, 1), (5, 3), (33, 64), (130, 257), (300, 515)])
+def test_complex_fp32_class_rows_of_any_scale(lib, n, k, kind):
+    import torch
+    A = _complex_rows(n, k, kind)
+    Ad = torch.from_numpy(A).cuda()
+    for fn, herm in ((lib.aah_complex, True), (lib.aat_complex, False), (lib.aat_complex_2m, False)):
+        got = fn(Ad).cpu().numpy().astype(np.complex128)
+        assert _row_relative(got, A, herm) <= 2e-6, fn.__name__
+
+
+def test_complex_fp32_class_keeps_small_values_beside_an_outlier(lib):
+    """Rows whose one large value meets zeros in the other rows: the product
+    of their small values keeps FP32 accuracy (BF16 pieces)."""
+    import torch
+    n, k = 96, 200
+    A = _complex_rows(n, k, "normal")
+    A[: n // 2, 0] = 1e7
+    A[n // 2:, 0] = 0
+    for fn, conj in ((lib.aah_complex, True), (lib.aat_complex_2m, False)):
+        got = fn(torch.from_numpy(A).cuda()).cpu().numpy().astype(np.complex128)[n // 2:, :n // 2]
+        Z = A.astype(np.complex128)
+        ref = Z[n // 2:] @ (Z.conj() if conj else Z)[:n // 2].T
+        assert np.abs(got - ref).max() <= 1e-5 * k
+
+
+def test_plan_of_complex_products_mixes_fp16_and_bf16_rows(lib):
+    """Every problem of a plan chooses its own form, again on each execution."""
+    import torch
+    kinds = ["normal", "col_scales", "row_scales", "huge_row", "normal"]
+    mats = [_complex_rows(40 + 37 * i, 30 + 61 * i, kd) for i, kd in enumerate(kinds)]
+    xs = [torch.from_numpy(m).cuda() for m in mats]
+    cs = [torch.zeros((x.shape[0],) * 2, dtype=torch.complex64, device="cuda") for x in xs]
+    plan = lib.Plan([("aah", x, c, 0, lib.AAT_C_FP32) for x, c in zip(xs, cs)])
+    for swap in (False, True):
+        if swap:  # the forms change with the data
+            for i, x in enumerate(xs):
+                mats[i] = _complex_rows(*mats[i].shape, kinds[(i + 1) % len(kinds)])
+                x.copy_(torch.from_numpy(mats[i]))
+        plan.execute()
+        torch.cuda.synchronize()
+        for m, c in zip(mats, cs):
+            assert _row_relative(c.cpu().numpy().astype(np.complex128), m, True) <= 2e-6
+    plan.close()
