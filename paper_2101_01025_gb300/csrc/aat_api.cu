@@ -424,7 +424,17 @@ struct Ctx {
   // passes over windows of pass_w planes of its operands' plane sequence
   bool passes = false;
   int pass_w = 1;
+  // the entry point lets a small product without recursion levels run as one
+  // CUDA-core launch; zero_low: that launch clears the strict upper triangle
+  bool small_ok = false, zero_low = false;
 };
+
+// One CUDA-core launch for a whole product (leaf_small_pays), unless a form
+// was tuned or the low-memory schedule asked for.
+static bool small_product(const Ctx &c, int64_t M, int64_t N, int64_t K, int lower) {
+  return c.small_ok && c.leaf == AAT_LEAF_TC && c.form == 0 && !c.passes &&
+         leaf_small_pays(M, N, K, lower);
+}
 
 static Planes planes_for(const DigitSpec &ds, int64_t rows, int64_t cols) {
   Planes P;
@@ -524,6 +534,13 @@ static void leaf(Ctx &c, Operand X, Operand Y, bool same, int64_t M, int64_t N, 
                  int32_t *out, int64_t ldo, int lower, uint32_t beta) {
   const Lin lin = lin_of(c.alpha, beta, c.m.p);
   count_leaf(c, M, N, K, lower);
+  if (small_product(c, M, N, K, lower)) {
+    if (!c.ar.dry)
+      check(c, launch_leaf_small(X.x, X.ld, Y.x, Y.ld, M, N, K, out, ldo, lower, c.zero_low, lin,
+                                 c.m, c.st),
+            "leaf (CUDA cores, small)");
+    return;
+  }
   if (c.leaf == AAT_LEAF_SIMT) {
     if (!c.ar.dry)
       check(c, launch_leaf_simt(X.x, X.ld, Y.x, Y.ld, M, N, K, out, ldo, lower, lin, c.m,
@@ -1118,13 +1135,19 @@ static size_t run_plan_in(Ctx &c, const int32_t *A, int64_t n, int64_t k, int64_
   }
   c.top_levels = early ? pr.levels : -1;
   c.split_row = early ? pr.n_pad / 2 : n;
+  const bool small_ok = c.small_ok;
+  c.small_ok = small_ok && pr.levels == 0;
+  c.zero_low = small_product(c, n, n, k, 1) && (flags & AAT_ZERO_UPPER);
 
   if (beta)
     syrk_rec(c, Aw, ldaw, pr.n_pad, pr.k_pad, Cw, ldcw, pr.levels, *beta);
   else
     rec(c, Aw, ldaw, pr.n_pad, pr.k_pad, Cw, ldcw, pr.levels, no_planes());
   if (pr.padded && !dry) check(c, launch_copy_low(Cw, ldcw, C, ldc, n, c.st), "unpad");
-  if (!dry && (flags & AAT_ZERO_UPPER)) check(c, launch_zero_upper(C, ldc, n, c.st), "zero upper");
+  if (!dry && (flags & AAT_ZERO_UPPER) && !c.zero_low)
+    check(c, launch_zero_upper(C, ldc, n, c.st), "zero upper");
+  c.small_ok = small_ok;
+  c.zero_low = false;
   if (!dry && !early && c.split_ev && c.err == AAT_OK) cudaEventRecord(c.split_ev, c.st);
   c.in_a11 = in_a11;
   c.in_rest = in_rest;
@@ -1345,6 +1368,7 @@ static int modp_device(const int32_t *A, int64_t n, int64_t k, int64_t lda, uint
     return ce == cudaSuccess ? AAT_OK : cuda_fail(ce, "memset");
   }
   c.form = form;
+  c.small_ok = true;
   c.in_a11 = in_a11;
   c.in_rest = in_rest;
   c.in_bands = in_bands;
@@ -1837,6 +1861,7 @@ int aat_gemm_modp(const int32_t *X, int64_t ldx, const int32_t *Y, int64_t ldy, 
     return ce == cudaSuccess ? AAT_OK : cuda_fail(ce, "memset");
   }
   const bool same = (X == Y && ldx == ldy && m == n);
+  c.small_ok = true;
   size_t need = 0;
   for (int pass = 0; pass < 2; ++pass) {
     void *ws = nullptr;
@@ -1856,6 +1881,7 @@ int aat_gemm_modp(const int32_t *X, int64_t ldx, const int32_t *Y, int64_t ldy, 
 size_t aat_workspace_size(int64_t n, int64_t k, uint32_t p, uint32_t flags) {
   Ctx c;
   if (n <= 0 || k <= 0 || setup(c, p, flags, nullptr)) return 0;
+  c.small_ok = true;
   return choose_schedule(c, nullptr, n, k, k, nullptr, n, flags);
 }
 

@@ -393,6 +393,14 @@ cudaError_t launch_leaf_simt(const int32_t *X, int64_t ldx, const int32_t *Y, in
                              int64_t M, int64_t N, int64_t K, int32_t *out, int64_t ldo,
                              int lower, const Lin &lin, const ModP &m, cudaStream_t st);
 
+// The same for small products, in one launch; zero: the strict upper triangle
+// of out is cleared too (lower products).
+bool leaf_small_pays(int64_t M, int64_t N, int64_t K, int lower);
+cudaError_t launch_leaf_small(const int32_t *X, int64_t ldx, const int32_t *Y, int64_t ldy,
+                              int64_t M, int64_t N, int64_t K, int32_t *out, int64_t ldo,
+                              int lower, bool zero, const Lin &lin, const ModP &m,
+                              cudaStream_t st);
+
 // Warp-level mma.sync leaves (k_leaf_mma.cu): INT8 digits with exact INT32
 // accumulation (workspace: leaf_i8_workspace bytes), and FP64 (exact while
 // K ((p-1)/2)^2 < 2^53 per chunk).

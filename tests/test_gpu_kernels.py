@@ -179,3 +179,32 @@ def test_plan_of_complex_products_mixes_fp16_and_bf16_rows(lib):
         for m, c in zip(mats, cs):
             assert _row_relative(c.cpu().numpy().astype(np.complex128), m, True) <= 2e-6
     plan.close()
+
+
+@pytest.mark.parametrize("worst", [False, True])
+@pytest.mark.parametrize("p", [3, 65521, 1000003, 2147483587, 2**31 - 1])
+@pytest.mark.parametrize("n,k", [(1, 1), (15, 127), (16, 128), (17, 129), (33, 4), (96, 160), (50, 1024)])
+def test_small_products_in_one_launch(lib, n, k, p, worst):
+    """Low(A A^T) and X Y^T of small sizes, with entries at the ends of the
+    range (the int64 sums at their largest), strided rows, cleared and kept
+    upper triangles."""
+    import torch
+    if worst:  # squares all of one sign, and products of both signs
+        A = np.full((n, k), (p - 1) // 2, dtype=np.int32)
+        A[1::2] = -((p - 1) // 2)
+        A[::3] = p - 1
+    else:
+        A = synth.residues(n + k, (n, k), p, balanced=True)
+    buf = torch.zeros((n, k + 3), dtype=torch.int32, device="cuda")
+    X = buf[:, :k]
+    X.copy_(torch.from_numpy(A))
+    ref = (A.astype(object) @ A.astype(object).T) % p
+    for flags in (0, lib.AAT_ZERO_UPPER):
+        C = torch.full((n, n + 1), -5, dtype=torch.int32, device="cuda")
+        lib.aat_modp(X, p, C=C[:, :n], flags=flags)
+        want = np.tril(ref) + (0 if flags else np.triu(np.full((n, n), -5, dtype=object), 1))
+        got = C.cpu().numpy().astype(object)
+        assert np.array_equal(got[:, :n], want) and (got[:, n] == -5).all()
+    Y = torch.from_numpy(A[: max(1, n // 2)]).cuda()
+    got = lib.aat_gemm_modp(X, Y, p).cpu().numpy().astype(object)
+    assert np.array_equal(got, ref[:, : max(1, n // 2)])
