@@ -425,8 +425,11 @@ struct Ctx {
   bool passes = false;
   int pass_w = 1;
   // the entry point lets a small product without recursion levels run as one
-  // CUDA-core launch; zero_low: that launch clears the strict upper triangle
-  bool small_ok = false, zero_low = false;
+  // CUDA-core launch
+  bool small_ok = false;
+  // the product is one leaf whose launch may clear the strict upper triangle
+  // (want_zero), and did (zeroed)
+  bool want_zero = false, zeroed = false;
 };
 
 // One CUDA-core launch for a whole product (leaf_small_pays), unless a form
@@ -536,9 +539,10 @@ static void leaf(Ctx &c, Operand X, Operand Y, bool same, int64_t M, int64_t N, 
   count_leaf(c, M, N, K, lower);
   if (small_product(c, M, N, K, lower)) {
     if (!c.ar.dry)
-      check(c, launch_leaf_small(X.x, X.ld, Y.x, Y.ld, M, N, K, out, ldo, lower, c.zero_low, lin,
+      check(c, launch_leaf_small(X.x, X.ld, Y.x, Y.ld, M, N, K, out, ldo, lower, c.want_zero, lin,
                                  c.m, c.st),
             "leaf (CUDA cores, small)");
+    c.zeroed = c.want_zero;
     return;
   }
   if (c.leaf == AAT_LEAF_SIMT) {
@@ -603,9 +607,46 @@ static void leaf(Ctx &c, Operand X, Operand Y, bool same, int64_t M, int64_t N, 
     Y.pl = planes_alloc(c, N, K);
     if (!c.ar.dry) check(c, launch_split(Y.x, Y.ld, N, K, c.m, c.ds.b, Y.pl, c.st), "split");
   }
-  if (!c.ar.dry && c.err == AAT_OK)
-    check(c, launch_leaf_tc(tc_args(c, X.pl, Y.pl, M, N, K, out, ldo, lower, beta), c.m, c.st),
-          "leaf (tensor cores)");
+  TcLeafArgs a = tc_args(c, X.pl, Y.pl, M, N, K, out, ldo, lower, beta);
+  const LeafSplit sp = leaf_tc_split(a);
+  if (sp.window > 0) {
+    // every part a product of its own (scaled by alpha) into workspace
+    const bool sums = a.dx.nsum > 0;
+    const int64_t ldw = (N + 3) / 4 * 4, stride = M * ldw;
+    std::vector<TcLeafArgs> parts;
+    for (int q0 = 0; q0 < X.pl.L; q0 += sp.window)
+      for (int64_t k0 = 0; k0 < K; k0 += sp.slice_k) {
+        const int64_t kw = std::min(sp.slice_k, K - k0);
+        const int w = std::min(sp.window, X.pl.L - q0);
+        auto part = [&](const Planes &P, bool window) {
+          Planes Q = P;
+          if (window) {
+            Q.q0 = q0;
+            Q.L = w;
+          }
+          if (Q.ptr) Q.ptr += Q.q0 * Q.rows * Q.kstride + k0;
+          Q.cols = kw;
+          return Q;
+        };
+        TcLeafArgs b = tc_args(c, part(X.pl, true), part(Y.pl, sums), M, N, kw, nullptr, ldw, lower, 0);
+        if (c.ar.dry || leaf_tc_terms(b, c.m) > 0) parts.push_back(b);
+      }
+    int32_t *W = (int32_t *)c.ar.get(parts.size() * (size_t)stride * 4);
+    for (size_t q = 0; q < parts.size(); ++q) parts[q].out = c.ar.dry ? nullptr : W + q * stride;
+    if (!c.ar.dry && c.err == AAT_OK) {
+      if (!parts.empty())
+        check(c, launch_leaf_tc_multi(parts.data(), (int)parts.size(), c.m, c.st),
+              "leaf (tensor cores, parts)");
+      check(c, launch_partial_sum(W, ldw, stride, (int)parts.size(), out, ldo, M, N, lower,
+                                  c.want_zero, lin.beta, c.m, c.st),
+            "sum of parts");
+    }
+    c.zeroed = c.want_zero;
+    c.ar.used = mark;
+    return;
+  }
+
+  if (!c.ar.dry && c.err == AAT_OK) check(c, launch_leaf_tc(a, c.m, c.st), "leaf (tensor cores)");
   c.ar.used = mark;
 }
 
@@ -1137,17 +1178,18 @@ static size_t run_plan_in(Ctx &c, const int32_t *A, int64_t n, int64_t k, int64_
   c.split_row = early ? pr.n_pad / 2 : n;
   const bool small_ok = c.small_ok;
   c.small_ok = small_ok && pr.levels == 0;
-  c.zero_low = small_product(c, n, n, k, 1) && (flags & AAT_ZERO_UPPER);
+  c.want_zero = pr.levels == 0 && (flags & AAT_ZERO_UPPER);
+  c.zeroed = false;
 
   if (beta)
     syrk_rec(c, Aw, ldaw, pr.n_pad, pr.k_pad, Cw, ldcw, pr.levels, *beta);
   else
     rec(c, Aw, ldaw, pr.n_pad, pr.k_pad, Cw, ldcw, pr.levels, no_planes());
   if (pr.padded && !dry) check(c, launch_copy_low(Cw, ldcw, C, ldc, n, c.st), "unpad");
-  if (!dry && (flags & AAT_ZERO_UPPER) && !c.zero_low)
+  if (!dry && (flags & AAT_ZERO_UPPER) && !c.zeroed)
     check(c, launch_zero_upper(C, ldc, n, c.st), "zero upper");
   c.small_ok = small_ok;
-  c.zero_low = false;
+  c.want_zero = false;
   if (!dry && !early && c.split_ev && c.err == AAT_OK) cudaEventRecord(c.split_ev, c.st);
   c.in_a11 = in_a11;
   c.in_rest = in_rest;

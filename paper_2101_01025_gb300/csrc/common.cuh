@@ -432,6 +432,18 @@ cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st);
 // persistent launch (one tile list over all of them).
 cudaError_t launch_leaf_tc_multi(const TcLeafArgs *as, int count, const ModP &m,
                                  cudaStream_t st);
+// The parts of a product of few tiles: windows of `window` planes of X, and
+// `slices` slices of `slice_k` columns of K (window 0: not split).
+struct LeafSplit {
+  int window = 0, slices = 1;
+  int64_t slice_k = 0;
+};
+LeafSplit leaf_tc_split(const TcLeafArgs &a);
+// out <- sum of `parts` canonical M x N blocks W + q stride (row stride ldw)
+// + beta out mod p (lower: i >= j; zero: the strict upper triangle is cleared).
+cudaError_t launch_partial_sum(const int32_t *W, int64_t ldw, int64_t stride, int parts,
+                               int32_t *out, int64_t ldo, int64_t M, int64_t N, int lower,
+                               bool zero, const MulConst &beta, const ModP &m, cudaStream_t st);
 // Whether that one launch is expected to beat one launch per product (the
 // idle share of the separate launches' last waves).
 bool leaf_tc_fuse_pays(const TcLeafArgs *as, int count);

@@ -516,6 +516,50 @@ __global__ void zero_upper_kernel(int32_t *C, int64_t ldc, int64_t n) {
     }
 }
 
+// The parts of a split leaf product added mod p: one thread per four columns
+// of a row, parts read as 16-byte vectors (ldw and W are 16-byte aligned).
+// Bound by L2, where the leaf just wrote the parts.
+__global__ void __launch_bounds__(kThreads)
+    partial_sum_kernel(const int32_t *__restrict__ W, int64_t ldw, int64_t stride, int parts,
+                       int32_t *out, int64_t ldo, int64_t M, int64_t N, int lower, int zero,
+                       MulConst beta, ModP m) {
+  const int64_t c = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+  if (c >= N) return;
+  for (int64_t r = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; r < M;
+       r += (int64_t)gridDim.y * blockDim.y) {
+    int32_t *o = out + r * ldo + c;
+    const int lim = (int)min((int64_t)4, N - c);
+    int live = lim;  // columns of the quad that are summed
+    if (lower) live = (int)max((int64_t)0, min((int64_t)lim, r - c + 1));
+    uint64_t s[4] = {0, 0, 0, 0};
+    if (live > 0) {
+      const int32_t *w = W + r * ldw + c;
+#pragma unroll 4
+      for (int q = 0; q < parts; ++q) {
+        const int4 v = *reinterpret_cast<const int4 *>(w + q * stride);
+        s[0] += (uint32_t)v.x;
+        s[1] += (uint32_t)v.y;
+        s[2] += (uint32_t)v.z;
+        s[3] += (uint32_t)v.w;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (j < live) {
+        int32_t v = to_bal(red_u64(s[j], m), m);
+        if (beta.w) {
+          int32_t old = bal(o[j], m);
+          if (beta.w != 1u) old = mulmod_shoup(old, beta.w, beta.wsh, m);
+          v = add_bal(v, old, m);
+        }
+        o[j] = (int32_t)bal_to_canon(v, m);
+      } else if (zero && j < lim) {
+        o[j] = 0;
+      }
+    }
+  }
+}
+
 int grid_for(int64_t total) {
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
@@ -716,6 +760,22 @@ cudaError_t launch_add_low(int32_t *C11, int64_t ldc, const int32_t *S, int64_t 
   if (h <= 0) return cudaSuccess;
   ProfScope prof(AAT_K_ADD_LOW, st, 4.0 * 3.0 * 0.5 * (double)h * (double)(h + 1));
   add_low_kernel<<<grid_for(h * h), kThreads, 0, st>>>(C11, ldc, S, lds, h, m);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_partial_sum(const int32_t *W, int64_t ldw, int64_t stride, int parts,
+                               int32_t *out, int64_t ldo, int64_t M, int64_t N, int lower,
+                               bool zero, const MulConst &beta, const ModP &m, cudaStream_t st) {
+  if (M <= 0 || N <= 0) return cudaSuccess;
+  if (ldw % 4 || stride % 4 || ((uintptr_t)W & 15) || ldw < N) return cudaErrorInvalidValue;
+  const double n = lower ? 0.5 * (double)M * (double)(M + 1) : (double)M * N;
+  ProfScope prof(AAT_K_ADD_LOW, st, 4.0 * n * (parts + 1 + (beta.w ? 1 : 0)));
+  const int64_t nq = (N + 3) / 4;
+  const dim3 block(32, kThreads / 32);
+  const dim3 grid((unsigned)((nq + 31) / 32),
+                  (unsigned)std::min<int64_t>((M + block.y - 1) / block.y, 65535));
+  partial_sum_kernel<<<grid, block, 0, st>>>(W, ldw, stride, parts, out, ldo, M, N, lower, zero,
+                                             beta, m);
   return cudaGetLastError();
 }
 

@@ -1078,12 +1078,19 @@ int term_count(const TcLeafArgs &a) {
   return a.dx.nsum > 0 ? std::min(a.x.L, a.y.L) : a.x.L * a.y.L;
 }
 
+// Modelled SM cycles of one tile of a one-CTA form: per plane product its K
+// blocks, a Horner step and a drain; prologue, fill and store.  Fitted to
+// 1001 x 1001 x 3001 mod 2^31 - 1 on one wave (ten products wide 340 k cycles,
+// two 88 k; ten narrow 131 k) and to 256 x 256 x 256 mod 131071 (four narrow,
+// 15 k).
+double tile_cycles(int narrow, double kb, double terms) {
+  return narrow ? terms * (240.0 * kb + 1100.0) + 7000.0 : terms * (540.0 * kb + 4600.0) + 25000.0;
+}
+
 // The form of one launch over `count` products.  CTA pairs when their tiles
 // fill every co-resident pair (or AAT_LEAF_PAIR / TcLeafArgs::form says so).
 // Otherwise one CTA per tile, 256 or 64 columns wide, by the modelled length
-// of the longest CTA in SM cycles: waves of tiles times (K blocks of the MMA,
-// 512 cycles wide and ~200 narrow; per plane product a Horner step and a
-// drain, 4600 wide and 1150 narrow; prologue, fill and store).  Measured at
+// of the longest CTA in SM cycles: waves of tiles times tile_cycles.  Measured at
 // 1001 x 1001 x 3001
 // (lower) mod 2^31 - 1, 20 wide or 72 narrow tiles: 178 -> 69 us; the four and
 // the one product of 512 x 512 mod 131071 with one level, 23.5 -> 10.4 and
@@ -1108,8 +1115,7 @@ Form leaf_form(const TcLeafArgs *as, int count, int units, int sms) {
     for (int i = 0; i < count; ++i) {
       const TcLeafArgs &a = as[i];
       const int64_t t = tile_count(a.M, a.N, a.lower, BM, w ? kTnNarrow : BN);
-      const double kb = (double)((a.K + BK - 1) / BK), terms = term_count(a);
-      work += t * (w ? terms * (200.0 * kb + 1150.0) + 2500.0 : terms * (512.0 * kb + 4600.0) + 8000.0);
+      work += t * tile_cycles(w, (double)((a.K + BK - 1) / BK), term_count(a));
       tiles += t;
     }
     cost[w] = work / (double)tiles * (double)((tiles + sms - 1) / sms);
@@ -1250,6 +1256,57 @@ bool leaf_tc_fuse_pays(const TcLeafArgs *as, int count) {
     all += slots * kb;
   }
   return all > 0.0 && idle > 0.06 * all;
+}
+
+// Whether a product of few tiles runs as several parts in one launch, each
+// part a window of its plane products over a slice of K, whose canonical
+// results partial_sum_kernel adds mod p.  A product of 20 wide or 72 narrow
+// tiles leaves most of the 152 SMs idle while each tile runs through all ten
+// plane products of 2^31 - 1 over the whole of K.  The split with the shortest
+// modelled longest CTA, if that and the sum (6000 cycles, the launch, and the
+// partials once through L2) beat the whole product by 15 %.  Measured at 1001
+// x 1001 x 3001 (lower) mod 2^31 - 1: 72 narrow tiles 69 us; two parts of five
+// plane products, 144 units, 38 + 6 us; five parts of two on wide tiles, 100
+// units, 46 + 7 us.
+LeafSplit leaf_tc_split(const TcLeafArgs &a) {
+  LeafSplit best;
+  if (a.form != 0 || pair_override() >= 0 || a.x.q0 || a.y.q0) return best;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const int sms = sm_count(dev);
+  const int64_t kblocks = (a.K + BK - 1) / BK;
+  // windows of X's planes; a plane of X meets one plane of Y (pair sums) or all
+  const int planes = a.x.L, per = a.dx.nsum > 0 ? 1 : a.y.L;
+  const int64_t t256 = tile_count(a.M, a.N, a.lower, BM, BN);
+  if (2 * t256 > sms) return best;
+  auto model = [&](int t, int s, double *out) {
+    const int64_t parts = (int64_t)((planes + t - 1) / t) * s;
+    double c = 1e30;
+    for (int w = 0; w < 2; ++w) {
+      const int64_t units = parts * tile_count(a.M, a.N, a.lower, BM, w ? kTnNarrow : BN);
+      c = std::min(c, (double)((units + sms - 1) / sms) *
+                          tile_cycles(w, (double)((kblocks + s - 1) / s), (double)t * per));
+    }
+    if (parts > 1) c += 6000.0 + (double)parts * a.M * a.N * (a.lower ? 4.0 : 8.0) / 4000.0;
+    *out = c;
+    return parts;
+  };
+  double whole = 0.0, bc = 0.0;
+  model(planes, 1, &whole);
+  bc = 0.85 * whole;
+  for (int t = 1; t <= planes; ++t)
+    for (int s = 1; s <= MAX_MULTI; ++s) {
+      double c = 0.0;
+      const int64_t parts = model(t, s, &c);
+      if (parts > MAX_MULTI || s > kblocks) break;
+      if (parts > 1 && c < bc) {
+        bc = c;
+        best.window = t;
+        best.slices = s;
+        best.slice_k = (kblocks + s - 1) / s * BK;
+      }
+    }
+  return best;
 }
 
 // Several independent products of one modulus and digit base in one

@@ -208,3 +208,50 @@ def test_small_products_in_one_launch(lib, n, k, p, worst):
     Y = torch.from_numpy(A[: max(1, n // 2)]).cuda()
     got = lib.aat_gemm_modp(X, Y, p).cpu().numpy().astype(object)
     assert np.array_equal(got, ref[:, : max(1, n // 2)])
+
+
+@pytest.mark.parametrize("pad", [0, 1, 3])
+@pytest.mark.parametrize("n,k", [(1030, 300), (1100, 2100), (2900, 40), (4100, 70), (4352, 64)])
+def test_leaf_clears_the_upper_triangle(lib, n, k, pad):
+    """The tensor-core leaf's own clearing (narrow tiles, wide tiles, CTA
+    pairs; split products): every entry of C and nothing beside it."""
+    import torch
+    p = 65521
+    A = synth.residues(n + k, (n, k), p)
+    buf = torch.full((n, n + pad), -9, dtype=torch.int32, device="cuda")
+    lib.aat_modp(torch.from_numpy(A).cuda(), p, C=buf[:, :n], flags=lib.AAT_ZERO_UPPER, levels=0)
+    D = torch.from_numpy(A).cuda().double()     # products < 2^32, sums < 2^53
+    ref = torch.remainder((D @ D.T).to(torch.int64), p).tril()
+    assert torch.equal(buf[:, :n].to(torch.int64), ref)
+    assert bool((buf[:, n:] == -9).all())
+
+
+@pytest.mark.parametrize("p", [65521, 131071, 1000003, 2**31 - 1])
+@pytest.mark.parametrize("M,N,K", [(130, 130, 2500), (700, 300, 4097), (64, 1500, 9000),
+                                   (513, 513, 3001), (1001, 1001, 2100)])
+def test_leaf_split_into_parts(lib, M, N, K, p):
+    """Windows of the plane products and slices of K summed mod p: stored,
+    accumulated (beta) and lower, aligned and ragged rows of C."""
+    import torch
+    from paper_2101_01025_gb300 import testing as T
+    lower = M == N
+    X = synth.residues(M + K, (M, K), p, balanced=True)
+    Y = X if lower else synth.residues(N + 7 * K, (N, K), p, balanced=True)
+    Xd, Yd = torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda()
+
+    def dot(a, b):  # 16-bit halves: FP64 products and sums are exact integers
+        return torch.remainder((a @ b.T).to(torch.int64), p)
+    xl, yl = torch.remainder(Xd, 65536).double(), torch.remainder(Yd, 65536).double()
+    xh = torch.div(Xd - xl.int(), 65536, rounding_mode="floor").double()
+    yh = torch.div(Yd - yl.int(), 65536, rounding_mode="floor").double()
+    ref = torch.remainder(dot(xh, yh) * ((1 << 32) % p) + dot(xl, yl)
+                          + torch.remainder(dot(xl, yh) + dot(xh, yl), p) * 65536, p)
+    for ld in (N, (N + 7) // 4 * 4):
+        old = torch.from_numpy(synth.residues(3, (M, ld), p)).cuda()
+        for acc in (False, True):
+            C = old.clone()
+            T.leaf(Xd, Xd if lower else Yd, p, C=C[:, :N], lower=lower, accumulate=acc)
+            new = torch.remainder(ref + (old[:, :N].to(torch.int64) if acc else 0), p)
+            want = old.to(torch.int64)
+            want[:, :N] = torch.where(torch.ones_like(new).tril().bool(), new, want[:, :N]) if lower else new
+            assert torch.equal(C.to(torch.int64), want)
