@@ -302,6 +302,7 @@ struct Shape {
 // Epilogue warps of the single-problem launches and of the batched launch
 // (whose tiles are mostly short in K, so the per-tile epilogue dominates).
 constexpr int kEwLeaf = 8, kEwBatch = 16;
+constexpr int kTnNarrow = 64;  // tile columns of the narrow one-CTA form
 
 template <int MODE, bool PAIR, int EW, int TN = BN>
 __global__ void __launch_bounds__(Shape<PAIR, EW, TN>::THREADS, 1)
@@ -1053,6 +1054,21 @@ int pair_override() {
   return v;
 }
 
+// Shared-memory limits of every one-CTA form of the single-product kernel, set
+// together whichever entry point launches first (g_mu held).
+cudaError_t set_single_attrs(int dev) {
+  if (g_attr_set[dev]) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(leaf_tc_kernel<kSingle, false, kEwLeaf>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)Shape<false, kEwLeaf>::SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(leaf_tc_kernel<kSingle, false, kEwLeaf, kTnNarrow>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)Shape<false, kEwLeaf, kTnNarrow>::SMEM);
+  if (e == cudaSuccess) g_attr_set[dev] = true;
+  return e;
+}
+
 int sm_count(int dev) {
   int sms = 148;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1068,7 +1084,6 @@ int64_t tile_count(int64_t M, int64_t N, int lower, int tm, int tn) {
   return c;
 }
 
-constexpr int kTnNarrow = 64;
 enum Form { kCta = 1, kPair = 2, kNarrow = 3 };
 int form_tm(Form f) { return f == kPair ? 256 : 128; }
 int form_tn(Form f) { return f == kNarrow ? kTnNarrow : BN; }
@@ -1175,17 +1190,7 @@ cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) 
   }
   P->tiles = tiles;
   P->ntiles = nt;
-  if (!g_attr_set[dev]) {
-    e = cudaFuncSetAttribute(leaf_tc_kernel<kSingle, false, kEwLeaf>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)Shape<false, kEwLeaf>::SMEM);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(leaf_tc_kernel<kSingle, false, kEwLeaf, kTnNarrow>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)Shape<false, kEwLeaf, kTnNarrow>::SMEM);
-    if (e != cudaSuccess) { delete P; return e; }
-    g_attr_set[dev] = true;
-  }
+  if ((e = set_single_attrs(dev)) != cudaSuccess) { delete P; return e; }
   if (nt > 0) {
     // algorithmic tensor work: one BF16 product of the ring MACs per plane
     // product with a non-zero weight
@@ -1787,12 +1792,8 @@ extern "C" AAT_API int aat_gemm_modp_noalloc(const int32_t *X, int64_t ldx, cons
   P.status = nd.status;
   P.tiles = tiles_dev;
   P.ntiles = (int)(TI * TJ);
-  if (!g_attr_set[dev]) {
-    ce = cudaFuncSetAttribute(leaf_tc_kernel<kSingle, false, kEwLeaf>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)Shape<false, kEwLeaf>::SMEM);
-    if (ce != cudaSuccess) return report_error(AAT_ECUDA, cudaGetErrorString(ce));
-    g_attr_set[dev] = true;
-  }
+  if ((ce = set_single_attrs(dev)) != cudaSuccess)
+    return report_error(AAT_ECUDA, cudaGetErrorString(ce));
   int sms = 148;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int grid = std::max(1, std::min(P.ntiles, sms));

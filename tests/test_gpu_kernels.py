@@ -255,3 +255,31 @@ def test_leaf_split_into_parts(lib, M, N, K, p):
             want = old.to(torch.int64)
             want[:, :N] = torch.where(torch.ones_like(new).tril().bool(), new, want[:, :N]) if lower else new
             assert torch.equal(C.to(torch.int64), want)
+
+
+def test_every_leaf_form_runs_after_the_allocation_free_entry_point(lib):
+    """In a fresh process: the allocation-free product first, then products on
+    the other one-CTA form and on CTA pairs."""
+    import os
+    import subprocess
+    import sys
+    code = """
+import torch
+import paper_2101_01025_gb300 as aat
+from paper_2101_01025_gb300 import _native as nat
+p = 65521
+X = torch.randint(0, p, (300, 64), dtype=torch.int32, device="cuda")
+C = torch.zeros((300, 300), dtype=torch.int32, device="cuda")
+s = torch.cuda.current_stream().cuda_stream
+nat.check(nat.lib().aat_gemm_modp_noalloc(X.data_ptr(), 64, X.data_ptr(), 64, 300, 300, 64, p,
+                                          C.data_ptr(), 300, s))
+for n, k in ((700, 700), (4000, 64), (2500, 640)):
+    A = torch.randint(0, p, (n, k), dtype=torch.int32, device="cuda")
+    D = A.double()
+    assert torch.equal(aat.aat_gemm_modp(A, A, p).long(), torch.remainder((D @ D.T).long(), p))
+print("ok")
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
