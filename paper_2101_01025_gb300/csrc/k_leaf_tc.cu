@@ -280,7 +280,7 @@ struct Shape {
   static constexpr int XB = EW == 8 ? 16 : 8;     // staged store block width
   static constexpr int TM = PAIR ? 256 : 128;     // output tile rows
   static constexpr int YROWS = PAIR ? TN / 2 : TN;  // rows of Y per CTA and stage
-  static constexpr int STAGES = PAIR ? 6 : TN == 256 ? 4 : 8;
+  static constexpr int STAGES = TN == 256 ? (PAIR ? 6 : 4) : 8;
   static constexpr int A_BYTES = BM * BK * 2;
   static constexpr int B_BYTES = YROWS * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
@@ -302,7 +302,8 @@ struct Shape {
 // Epilogue warps of the single-problem launches and of the batched launch
 // (whose tiles are mostly short in K, so the per-tile epilogue dominates).
 constexpr int kEwLeaf = 8, kEwBatch = 16;
-constexpr int kTnNarrow = 64;  // tile columns of the narrow one-CTA form
+// tile columns of the narrow one-CTA form and of the half-width pair form
+constexpr int kTnNarrow = 64, kTnHalf = 128;
 
 template <int MODE, bool PAIR, int EW, int TN = BN>
 __global__ void __launch_bounds__(Shape<PAIR, EW, TN>::THREADS, 1)
@@ -1054,7 +1055,8 @@ int pair_override() {
   return v;
 }
 
-// Shared-memory limits of every one-CTA form of the single-product kernel, set
+// Shared-memory limits of the single-product kernel's forms (pair_units sets the
+// whole pair form's), set
 // together whichever entry point launches first (g_mu held).
 cudaError_t set_single_attrs(int dev) {
   if (g_attr_set[dev]) return cudaSuccess;
@@ -1065,6 +1067,10 @@ cudaError_t set_single_attrs(int dev) {
     e = cudaFuncSetAttribute(leaf_tc_kernel<kSingle, false, kEwLeaf, kTnNarrow>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)Shape<false, kEwLeaf, kTnNarrow>::SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(leaf_tc_kernel<kSingle, true, kEwLeaf, kTnHalf>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)Shape<true, kEwLeaf, kTnHalf>::SMEM);
   if (e == cudaSuccess) g_attr_set[dev] = true;
   return e;
 }
@@ -1084,9 +1090,12 @@ int64_t tile_count(int64_t M, int64_t N, int lower, int tm, int tn) {
   return c;
 }
 
-enum Form { kCta = 1, kPair = 2, kNarrow = 3 };
-int form_tm(Form f) { return f == kPair ? 256 : 128; }
-int form_tn(Form f) { return f == kNarrow ? kTnNarrow : BN; }
+enum Form { kCta = 1, kPair = 2, kNarrow = 3, kPairHalf = 4 };
+bool is_pair(Form f) { return f == kPair || f == kPairHalf; }
+int form_tm(Form f) { return is_pair(f) ? 256 : 128; }
+int form_tn(Form f) { return f == kNarrow ? kTnNarrow : f == kPairHalf ? kTnHalf : BN; }
+// rows of Y per CTA and stage
+int form_yrows(Form f) { return is_pair(f) ? form_tn(f) / 2 : form_tn(f); }
 
 // Plane products per ring multiply-add of a leaf.
 int term_count(const TcLeafArgs &a) {
@@ -1121,7 +1130,27 @@ Form leaf_form(const TcLeafArgs *as, int count, int units, int sms) {
       const int64_t t = ((as[i].M + 255) / 256) * ((as[i].N + BN - 1) / BN);
       pt += as[i].lower ? t / 2 : t;
     }
-    if (big && (ov >= 0 ? ov > 0 : pt >= units)) return kPair;
+    if (big && (ov >= 0 ? ov > 0 : pt >= units)) {
+      // 256 x 256 tiles, or 256 x 128 where their finer waves leave fewer
+      // pairs idle at the end (modelled as tile_cycles; a half tile takes 0.56
+      // of a whole one).  2500 x 4001 x 3003 mod 2^31 - 1: 160 tiles, 3 waves
+      // of 76 pairs, 470 us; 320 half tiles, 5 waves, 436 us.
+      double cost[2];
+      for (int w = 0; w < 2; ++w) {
+        double work = 0.0;
+        int64_t tiles = 0;
+        for (int i = 0; i < count; ++i) {
+          const TcLeafArgs &a = as[i];
+          const int64_t t = tile_count(a.M, a.N, a.lower, 256, w ? kTnHalf : BN);
+          const double kb = (double)((a.K + BK - 1) / BK), terms = term_count(a);
+          work += t * (w ? terms * (300.0 * kb + 2300.0) + 2000.0
+                         : terms * (520.0 * kb + 4600.0) + 8000.0);
+          tiles += t;
+        }
+        cost[w] = work / (double)tiles * (double)((tiles + units - 1) / units);
+      }
+      return cost[1] < 0.97 * cost[0] ? kPairHalf : kPair;
+    }
   }
   double cost[2];
   for (int w = 0; w < 2; ++w) {
@@ -1156,13 +1185,13 @@ cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) 
 
   const int units = pair_units(dev), sms = sm_count(dev);
   const Form form = leaf_form(&a, 1, units, sms);
-  const bool pair = form == kPair;
+  const bool pair = is_pair(form);
   const int tm = form_tm(form), tn = form_tn(form);
 
   Params *P = new Params;
   std::memset(P, 0, sizeof(Params));
   if ((e = encode_planes(&P->tmx, a.x, BM)) != cudaSuccess ||
-      (e = encode_planes(&P->tmy, a.y, pair ? Shape<true>::YROWS : tn)) != cudaSuccess) {
+      (e = encode_planes(&P->tmy, a.y, form_yrows(form))) != cudaSuccess) {
     delete P;
     return e;
   }
@@ -1206,11 +1235,14 @@ cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) 
       attr[0].val.clusterDim.z = 1;
       cfg.gridDim = dim3(2 * std::max(1, std::min(nt, units)), 1, 1);
       cfg.blockDim = dim3(Shape<true, kEwLeaf>::THREADS, 1, 1);
-      cfg.dynamicSmemBytes = Shape<true, kEwLeaf>::SMEM;
+      cfg.dynamicSmemBytes = form == kPairHalf ? Shape<true, kEwLeaf, kTnHalf>::SMEM
+                                               : Shape<true, kEwLeaf>::SMEM;
       cfg.stream = st;
       cfg.attrs = attr;
       cfg.numAttrs = 1;
-      e = cudaLaunchKernelEx(&cfg, leaf_tc_kernel<kSingle, true, kEwLeaf>, *P);
+      e = form == kPairHalf
+              ? cudaLaunchKernelEx(&cfg, leaf_tc_kernel<kSingle, true, kEwLeaf, kTnHalf>, *P)
+              : cudaLaunchKernelEx(&cfg, leaf_tc_kernel<kSingle, true, kEwLeaf>, *P);
       if (e != cudaSuccess) { delete P; return e; }
     } else if (form == kNarrow) {
       leaf_tc_kernel<kSingle, false, kEwLeaf, kTnNarrow>
@@ -1252,7 +1284,7 @@ bool leaf_tc_fuse_pays(const TcLeafArgs *as, int count) {
   double idle = 0.0, all = 0.0;
   for (int i = 0; i < count; ++i) {
     const TcLeafArgs &a = as[i];
-    const bool pair = leaf_form(&a, 1, units, sms) == kPair;
+    const bool pair = is_pair(leaf_form(&a, 1, units, sms));
     const int u = pair ? units : sms;
     const double nt = (double)tile_count(a.M, a.N, a.lower, pair ? 256 : 128, BN);
     const double slots = std::ceil(nt / u) * u;
@@ -1339,7 +1371,7 @@ cudaError_t launch_leaf_tc_multi(const TcLeafArgs *as, int count, const ModP &m,
 
   const int units = pair_units(dev), sms = sm_count(dev);
   const Form form = leaf_form(as, count, units, sms);
-  const bool pair = form == kPair;
+  const bool pair = is_pair(form);
   const int tm = form_tm(form), tn = form_tn(form);
 
   Params *P = new Params;
@@ -1352,7 +1384,7 @@ cudaError_t launch_leaf_tc_multi(const TcLeafArgs *as, int count, const ModP &m,
     const TcLeafArgs &a = as[i];
     MultiProb &b = P->mp[i];
     if ((e = encode_planes(&b.tmx, a.x, BM)) != cudaSuccess ||
-        (e = encode_planes(&b.tmy, a.y, pair ? Shape<true>::YROWS : tn)) != cudaSuccess) {
+        (e = encode_planes(&b.tmy, a.y, form_yrows(form))) != cudaSuccess) {
       delete P;
       return e;
     }
@@ -1414,6 +1446,9 @@ cudaError_t launch_leaf_tc_multi(const TcLeafArgs *as, int count, const ModP &m,
         (e = cudaFuncSetAttribute(leaf_tc_kernel<kMulti, false, kEwLeaf, kTnNarrow>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)Shape<false, kEwLeaf, kTnNarrow>::SMEM)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(leaf_tc_kernel<kMulti, true, kEwLeaf, kTnHalf>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)Shape<true, kEwLeaf, kTnHalf>::SMEM)) != cudaSuccess ||
         (e = cudaFuncSetAttribute(leaf_tc_kernel<kMulti, true, kEwLeaf>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)Shape<true, kEwLeaf>::SMEM)) != cudaSuccess) {
@@ -1433,11 +1468,14 @@ cudaError_t launch_leaf_tc_multi(const TcLeafArgs *as, int count, const ModP &m,
       attr1[0].val.clusterDim.z = 1;
       cfg.gridDim = dim3(2 * std::max(1, std::min(nt, units)), 1, 1);
       cfg.blockDim = dim3(Shape<true, kEwLeaf>::THREADS, 1, 1);
-      cfg.dynamicSmemBytes = Shape<true, kEwLeaf>::SMEM;
+      cfg.dynamicSmemBytes = form == kPairHalf ? Shape<true, kEwLeaf, kTnHalf>::SMEM
+                                               : Shape<true, kEwLeaf>::SMEM;
       cfg.stream = st;
       cfg.attrs = attr1;
       cfg.numAttrs = 1;
-      e = cudaLaunchKernelEx(&cfg, leaf_tc_kernel<kMulti, true, kEwLeaf>, *P);
+      e = form == kPairHalf
+              ? cudaLaunchKernelEx(&cfg, leaf_tc_kernel<kMulti, true, kEwLeaf, kTnHalf>, *P)
+              : cudaLaunchKernelEx(&cfg, leaf_tc_kernel<kMulti, true, kEwLeaf>, *P);
       if (e != cudaSuccess) {
         delete P;
         return e;

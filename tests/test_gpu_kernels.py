@@ -283,3 +283,16 @@ print("ok")
     r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True,
                        timeout=300)
     assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("p", [65521, 131071, 2**31 - 1])
+@pytest.mark.parametrize("M,N,K", [(2500, 4001, 130), (2304, 3970, 64), (2305, 3841, 65)])
+def test_half_width_pair_tiles(lib, M, N, K, p):
+    """256 x 128 tiles of CTA pairs at their edges (sampled rows, every column)."""
+    import torch
+    X = synth.residues(M + K, (M, K), p, balanced=True)
+    Y = synth.residues(N + 5 * K, (N, K), p, balanced=True)
+    got = lib.aat_gemm_modp(torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda(), p).cpu().numpy()
+    rows = sorted({0, 1, 127, 128, 255, 256, 257, 2047, 2048, M - 2, M - 1})
+    ref = (X[rows].astype(object) @ Y.astype(object).T) % p
+    assert np.array_equal(got[rows].astype(object), ref)
