@@ -189,11 +189,15 @@ __device__ __forceinline__ FJob fjob(const FParams &P, int t) {
 // M=256 MMAs, both CTAs' copies complete on its barrier, its commits
 // multicast to both, and the epilogues of both release a buffer on its
 // barrier).
-template <bool PAIR>
+// TN = 64 (kFNarrow): the one-CTA form with 64-column tiles and 8 stages of
+// 24 KB, for products of few tiles.
+constexpr int kFNarrow = 64;
+template <bool PAIR, int TN = BN>
 struct FShape {
   static constexpr int TM = PAIR ? 256 : 128;
-  static constexpr int YROWS = PAIR ? 128 : 256;
-  static constexpr int STAGES = PAIR ? 6 : 4;
+  static constexpr int YROWS = PAIR ? TN / 2 : TN;
+  static constexpr int VALS = TN / 2;  // accumulators per epilogue thread
+  static constexpr int STAGES = PAIR ? 6 : TN == 256 ? 4 : 8;
   static constexpr int A_BYTES = BM * BK * 2;
   static constexpr int B_BYTES = YROWS * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
@@ -204,14 +208,14 @@ struct FShape {
   // kind::f16, FP32 accumulator, BF16 A and B, K-major, N = 256, M = TM
   // (IDESC_H: FP16 A and B)
   static constexpr uint32_t IDESC_H =
-      (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+      (1u << 4) | ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
   static constexpr uint32_t IDESC = IDESC_H | (1u << 7) | (1u << 10);
 };
 
-template <bool PAIR, bool BATCH>
+template <bool PAIR, bool BATCH, int TN = BN>
 __global__ void __launch_bounds__(THREADS, 1) leaf_f32_kernel(const __grid_constant__ FParams P) {
-  using S = FShape<PAIR>;
-  constexpr int STAGES = S::STAGES;
+  using S = FShape<PAIR, TN>;
+  constexpr int STAGES = S::STAGES, VALS = S::VALS;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
@@ -233,7 +237,8 @@ __global__ void __launch_bounds__(THREADS, 1) leaf_f32_kernel(const __grid_const
   }
   const bool leader = (rank == 0);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // the shuffles tell the compiler that warp and tmem are the same in a warp
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(FULL(s), 1);
@@ -267,10 +272,10 @@ __global__ void __launch_bounds__(THREADS, 1) leaf_f32_kernel(const __grid_const
   __syncthreads();
   if constexpr (PAIR) cluster_sync();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   if (warp == 0) {
-    if (lane == 0) {  // TMA producer
+    {  // TMA producer: uniform control flow, one elected lane issues the copies
       int stage = 0, issued = 0;
       uint32_t ph = 0;
       bool ok = true;
@@ -278,25 +283,29 @@ __global__ void __launch_bounds__(THREADS, 1) leaf_f32_kernel(const __grid_const
       for (int t = (int)unit0; t < P.ntiles && ok; t += (int)nunits) {
         const FJob jb = fjob<BATCH>(P, t);
         const int rowx = jb.I * S::TM + (int)rank * BM;
-        const int rowy = jb.J * BN + (int)rank * S::YROWS;
+        const int rowy = jb.J * TN + (int)rank * S::YROWS;
         for (int gi = 0; gi < jb.ng && ok; ++gi) {
           const FGroup g = jb.group(gi);
           for (int kb = 0; kb < jb.kblocks; ++kb) {
-            if (!wait_bounded<PAIR>(EMPTY(stage), ph ^ 1u, abort_flag, P.status)) {
+            if (!__all_sync(0xffffffffu, wait_bounded<PAIR>(EMPTY(stage), ph ^ 1u, abort_flag,
+                                                            P.status))) {
               ok = false;
               break;
             }
             const uint32_t sa = sbase + (uint32_t)(stage * S::STAGE_BYTES);
             const uint32_t fb = full0 + 8u * (uint32_t)stage;
-            if constexpr (PAIR) {
-              if (leader) mbar_expect_tx(FULL(stage), (uint32_t)(2 * S::STAGE_BYTES));
-              tma_load_3d_pair(sa, jb.tmx, fb, kb * BK, rowx, g.xp);
-              tma_load_3d_pair(sa + S::A_BYTES, jb.tmy, fb, kb * BK, rowy, g.yp);
-            } else {
-              mbar_expect_tx(FULL(stage), (uint32_t)S::STAGE_BYTES);
-              tma_load_3d(sa, jb.tmx, fb, kb * BK, rowx, g.xp);
-              tma_load_3d(sa + S::A_BYTES, jb.tmy, fb, kb * BK, rowy, g.yp);
+            if (elect_one()) {
+              if constexpr (PAIR) {
+                if (leader) mbar_expect_tx(FULL(stage), (uint32_t)(2 * S::STAGE_BYTES));
+                tma_load_3d_pair(sa, jb.tmx, fb, kb * BK, rowx, g.xp);
+                tma_load_3d_pair(sa + S::A_BYTES, jb.tmy, fb, kb * BK, rowy, g.yp);
+              } else {
+                mbar_expect_tx(FULL(stage), (uint32_t)S::STAGE_BYTES);
+                tma_load_3d(sa, jb.tmx, fb, kb * BK, rowx, g.xp);
+                tma_load_3d(sa + S::A_BYTES, jb.tmy, fb, kb * BK, rowy, g.yp);
+              }
             }
+            __syncwarp();
             ++issued;
             if (++stage == STAGES) {
               stage = 0;
@@ -416,9 +425,9 @@ __global__ void __launch_bounds__(THREADS, 1) leaf_f32_kernel(const __grid_const
     for (int t = (int)unit0; t < P.ntiles && ok; t += (int)nunits) {
       const FJob jb = fjob<BATCH>(P, t);
       const int nchunks = jb.chunks(P.kchunk);
-      float acc[128];
+      float acc[VALS];
 #pragma unroll
-      for (int i = 0; i < 128; ++i) acc[i] = 0.0f;
+      for (int i = 0; i < VALS; ++i) acc[i] = 0.0f;
       for (int c = 0; c < nchunks; ++c) {
         const uint32_t buf = chunk & 1u, use = chunk >> 1;
         if (!wait_bounded<PAIR>(AFULL(buf), use & 1u, abort_flag, P.status)) {
@@ -426,15 +435,17 @@ __global__ void __launch_bounds__(THREADS, 1) leaf_f32_kernel(const __grid_const
           break;
         }
         tc_fence_after();
-        const uint32_t ta = tmem + lane_base + buf * ACC_COLS + (uint32_t)(chalf * 128);
+        const uint32_t ta = tmem + lane_base + buf * ACC_COLS + (uint32_t)(chalf * VALS);
         tmem_accum16f<0>(ta, acc);
         tmem_accum16f<16>(ta + 16u, acc);
-        tmem_accum16f<32>(ta + 32u, acc);
-        tmem_accum16f<48>(ta + 48u, acc);
-        tmem_accum16f<64>(ta + 64u, acc);
-        tmem_accum16f<80>(ta + 80u, acc);
-        tmem_accum16f<96>(ta + 96u, acc);
-        tmem_accum16f<112>(ta + 112u, acc);
+        if constexpr (VALS == 128) {
+          tmem_accum16f<32>(ta + 32u, acc);
+          tmem_accum16f<48>(ta + 48u, acc);
+          tmem_accum16f<64>(ta + 64u, acc);
+          tmem_accum16f<80>(ta + 80u, acc);
+          tmem_accum16f<96>(ta + 96u, acc);
+          tmem_accum16f<112>(ta + 112u, acc);
+        }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
@@ -447,7 +458,7 @@ __global__ void __launch_bounds__(THREADS, 1) leaf_f32_kernel(const __grid_const
       }
       if (!ok) break;
       const int64_t row = (int64_t)jb.I * S::TM + (int64_t)rank * BM + quarter * 32 + lane;
-      const int64_t col0 = (int64_t)jb.J * BN + chalf * 128;
+      const int64_t col0 = (int64_t)jb.J * TN + chalf * VALS;
       // rows 16-byte aligned: each thread stores its row segment with
       // 16-byte stores
       if (((reinterpret_cast<uintptr_t>(jb.out) | (uintptr_t)(jb.ldo * 4)) & 15) == 0) {
@@ -456,7 +467,7 @@ __global__ void __launch_bounds__(THREADS, 1) leaf_f32_kernel(const __grid_const
         if (row < jb.M && lim > 0) {
           float *orow = jb.out + row * jb.ldo + col0;
 #pragma unroll
-          for (int q = 0; q < 32; ++q) {
+          for (int q = 0; q < VALS / 4; ++q) {
             const int cc = 4 * q;
             if (cc + 4 <= lim) {
               *reinterpret_cast<float4 *>(orow + cc) =
@@ -475,12 +486,12 @@ __global__ void __launch_bounds__(THREADS, 1) leaf_f32_kernel(const __grid_const
       // 32 rows at a time, two contiguous 64-byte row segments per store
       const int64_t row0 = row - lane;
       const int mlim = (int)max((int64_t)0, min((int64_t)32, jb.M - row0));
-      const int nlim = (int)max((int64_t)0, min((int64_t)128, jb.N - col0));
+      const int nlim = (int)max((int64_t)0, min((int64_t)VALS, jb.N - col0));
       const int dl = jb.lower ? (int)max((int64_t)-256, min((int64_t)256, row0 - col0)) : 1 << 20;
       float *const base = jb.out + row0 * jb.ldo + col0;
       const int64_t ldo = jb.ldo;
 #pragma unroll
-      for (int cb = 0; cb < 128; cb += 16) {
+      for (int cb = 0; cb < VALS; cb += 16) {
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < 16; ++j) xs[lane * 17 + j] = acc[cb + j];
@@ -1138,7 +1149,8 @@ size_t fused_table_bytes() {
 namespace {
 
 __global__ void fused_table_kernel(const __grid_constant__ FusedTable T, FJobDesc *jobs,
-                                   FGroup *gtab) {
+                                   FGroup *gtab, int32_t *wide) {
+  if (wide && threadIdx.x == 0) *wide = 0;
   for (int i = threadIdx.x; i < T.njobs; i += blockDim.x) jobs[i] = T.jobs[i];
   for (int i = threadIdx.x; i < T.ng; i += blockDim.x) gtab[i] = T.g[i];
 }
@@ -1146,24 +1158,37 @@ __global__ void fused_table_kernel(const __grid_constant__ FusedTable T, FJobDes
 // Tile lists of fused launches, per device, tile height and job shapes: each
 // job's tiles in bands of 2048 rows swept column by column, jobs in order.
 std::map<std::vector<int64_t>, std::pair<int4 *, int>> g_ftiles;
-std::map<int, bool> g_fattr[2];
+std::map<int, bool> g_fattr;
+
+enum FForm { kFCta, kFPair, kFNarrowForm };
 
 }  // namespace
 
 // All jobs in one persistent launch of the FP32 leaf (tcgen05, CTA pairs when
 // the tiles fill every co-resident pair), so that no product's last wave
-// leaves SMs idle.  table_mem: fused_table_bytes() of device memory, 256-byte
-// aligned, for the job table.
-// wide: the products' FP16 / BF16 flag (null: BF16).
-static cudaError_t launch_leaf_f32_fused(const std::vector<FusedJob> &jobs, int np, int64_t K,
-                                         void *table_mem, cudaStream_t st,
-                                         const int32_t *wide = nullptr) {
+// leaves SMs idle.  fused_table writes the job table (and clears the products'
+// FP16 / BF16 flag `wide`, null: BF16) with one small kernel, fused_launch runs
+// the leaf from it; what sets the flag and the pieces runs between the two.
+// table_mem: fused_table_bytes() of device memory, 256-byte aligned.
+struct FusedLaunch {
+  FParams P;
+  double work = 0.0;
+  int units = 0, nt = 0;
+  FForm form = kFCta;
+};
+
+static cudaError_t fused_table(const std::vector<FusedJob> &jobs, int np, int64_t K,
+                               void *table_mem, cudaStream_t st, int32_t *wide,
+                               FusedLaunch *out) {
   const int nj = (int)jobs.size();
   if (nj < 1 || nj > MAX_FUSED || K <= 0) return cudaErrorInvalidValue;
   std::lock_guard<std::mutex> lock(g_mu_c);
   int dev = 0;
   cudaGetDevice(&dev);
   const int units = pair_units_c(dev);
+  int sms = 148;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int kblocks = (int)((K + BK - 1) / BK);
   bool pair = units > 0;
   int64_t pt = 0;
   for (const FusedJob &j : jobs) {
@@ -1173,18 +1198,36 @@ static cudaError_t launch_leaf_f32_fused(const std::vector<FusedJob> &jobs, int 
   }
   const char *ev = getenv("AAT_LEAF_PAIR");
   pair = ev ? (atoi(ev) > 0 && units > 0) : (pair && pt >= units);
-  const int tm = pair ? FShape<true>::TM : FShape<false>::TM;
+  FForm form = pair ? kFPair : kFCta;
+  if (!pair) {
+    // 64-column tiles when that shortens the longest CTA: waves of tiles times
+    // modelled SM cycles of a tile, 512 (wide) or 240 (narrow) per K block and
+    // piece product.  A A^H per call, FP32 class: 300 x 300 42 -> 30 us, 500 x
+    // 2000 104 -> 56 us, 100 x 5000 208 -> 99 us (half of it the FP16 pieces).
+    double cost[2];
+    for (int w = 0; w < 2; ++w) {
+      const int tn = w ? kFNarrow : BN;
+      int64_t tiles = 0;
+      for (const FusedJob &j : jobs)
+        for (int64_t i = 0; i < (j.M + BM - 1) / BM; ++i) {
+          const int64_t TJ = (j.N + tn - 1) / tn;
+          tiles += j.lower ? std::min(TJ, (i * BM + BM - 1) / tn + 1) : TJ;
+        }
+      cost[w] = (double)((tiles + sms - 1) / sms) *
+                (w ? 240.0 * 3.0 * kblocks + 5000.0 : 512.0 * 3.0 * kblocks + 14000.0);
+    }
+    if (cost[1] < cost[0]) form = kFNarrowForm;
+  }
+  const int tm = pair ? 256 : 128, tn = form == kFNarrowForm ? kFNarrow : BN;
   FusedTable *T = new FusedTable;
   std::memset(T, 0, sizeof(FusedTable));
   cudaError_t e = cudaSuccess;
   double work = 0.0;
-  const int kblocks = (int)((K + BK - 1) / BK);
   for (int i = 0; i < nj && e == cudaSuccess; ++i) {
     const FusedJob &j = jobs[i];
     FJobDesc &d = T->jobs[i];
     if ((e = encode_c(&d.tmx, *j.X, BM)) != cudaSuccess ||
-        (e = encode_c(&d.tmy, *j.Y, pair ? FShape<true>::YROWS : FShape<false>::YROWS)) !=
-            cudaSuccess)
+        (e = encode_c(&d.tmy, *j.Y, pair ? FShape<true>::YROWS : tn)) != cudaSuccess)
       break;
     d.out = j.out;
     d.ldo = j.ldo;
@@ -1208,7 +1251,7 @@ static cudaError_t launch_leaf_f32_fused(const std::vector<FusedJob> &jobs, int 
   }
   T->njobs = nj;
   // the tile list, cached per shape list
-  std::vector<int64_t> key = {dev, tm};
+  std::vector<int64_t> key = {dev, tm, tn};
   for (const FusedJob &j : jobs) key.insert(key.end(), {j.M, j.N, (int64_t)j.lower});
   int4 *tiles = nullptr;
   int nt = 0;
@@ -1221,12 +1264,12 @@ static cudaError_t launch_leaf_f32_fused(const std::vector<FusedJob> &jobs, int 
       std::vector<int4> v;
       for (int i = 0; i < nj; ++i) {
         const FusedJob &j = jobs[i];
-        const int64_t TI = (j.M + tm - 1) / tm, TJ = (j.N + BN - 1) / BN;
+        const int64_t TI = (j.M + tm - 1) / tm, TJ = (j.N + tn - 1) / tn;
         const int64_t band = std::max<int64_t>(1, 2048 / tm);
         for (int64_t bi = 0; bi < TI; bi += band)
           for (int64_t jj = 0; jj < TJ; ++jj)
             for (int64_t ii = bi; ii < std::min(TI, bi + band); ++ii) {
-              if (j.lower && jj * BN > ii * tm + tm - 1) continue;
+              if (j.lower && jj * tn > ii * tm + tm - 1) continue;
               v.push_back(make_int4(i, (int)ii, (int)jj, 0));
             }
       }
@@ -1238,14 +1281,17 @@ static cudaError_t launch_leaf_f32_fused(const std::vector<FusedJob> &jobs, int 
       }
     }
   }
-  if (e == cudaSuccess && !g_fattr[pair][dev]) {
-    e = pair ? cudaFuncSetAttribute(leaf_f32_kernel<true, true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)FShape<true>::SMEM)
-             : cudaFuncSetAttribute(leaf_f32_kernel<false, true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)FShape<false>::SMEM);
-    if (e == cudaSuccess) g_fattr[pair][dev] = true;
+  if (e == cudaSuccess && !g_fattr[dev]) {
+    if ((e = cudaFuncSetAttribute(leaf_f32_kernel<true, true>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)FShape<true>::SMEM)) == cudaSuccess &&
+        (e = cudaFuncSetAttribute(leaf_f32_kernel<false, true>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)FShape<false>::SMEM)) == cudaSuccess &&
+        (e = cudaFuncSetAttribute(leaf_f32_kernel<false, true, kFNarrow>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)FShape<false, kFNarrow>::SMEM)) == cudaSuccess)
+      g_fattr[dev] = true;
   }
   if (e != cudaSuccess) {
     delete T;
@@ -1254,43 +1300,49 @@ static cudaError_t launch_leaf_f32_fused(const std::vector<FusedJob> &jobs, int 
   FJobDesc *jobs_dev = (FJobDesc *)table_mem;
   FGroup *gtab_dev =
       (FGroup *)((char *)table_mem + ((sizeof(FJobDesc) * MAX_FUSED + 255) & ~(size_t)255));
-  fused_table_kernel<<<1, 64, 0, st>>>(*T, jobs_dev, gtab_dev);
+  fused_table_kernel<<<1, 64, 0, st>>>(*T, jobs_dev, gtab_dev, wide);
   delete T;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  FParams *P = new FParams;
-  std::memset(P, 0, sizeof(FParams));
-  P->kchunk = 8;  // as launch_leaf_f32
-  P->ntiles = nt;
-  P->status = device_status_ptr();
-  P->jobs = jobs_dev;
-  P->btiles = tiles;
-  P->gtab = gtab_dev;
-  int sms = 148;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (nt > 0) {
-    ProfScope prof(AAT_K_LEAF_F32, st, work);
-    if (pair) {
-      cudaLaunchConfig_t cfg = {};
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = 2;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      cfg.gridDim = dim3(2 * std::max(1, std::min(nt, units)), 1, 1);
-      cfg.blockDim = dim3(THREADS, 1, 1);
-      cfg.dynamicSmemBytes = FShape<true>::SMEM;
-      cfg.stream = st;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      e = cudaLaunchKernelEx(&cfg, leaf_f32_kernel<true, true>, *P);
-    } else {
-      leaf_f32_kernel<false, true><<<std::max(1, std::min(nt, sms)), THREADS, FShape<false>::SMEM,
-                                     st>>>(*P);
-      e = cudaGetLastError();
-    }
+  FParams &P = out->P;
+  std::memset(&P, 0, sizeof(FParams));
+  P.kchunk = 8;  // as launch_leaf_f32
+  P.ntiles = nt;
+  P.status = device_status_ptr();
+  P.jobs = jobs_dev;
+  P.btiles = tiles;
+  P.gtab = gtab_dev;
+  out->work = work;
+  out->units = pair ? units : sms;
+  out->nt = nt;
+  out->form = form;
+  return cudaSuccess;
+}
+
+static cudaError_t fused_launch(const FusedLaunch &L, cudaStream_t st) {
+  if (L.nt <= 0) return cudaSuccess;
+  ProfScope prof(AAT_K_LEAF_F32, st, L.work);
+  const int grid = std::max(1, std::min(L.nt, L.units));
+  if (L.form == kFPair) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(2 * grid, 1, 1);
+    cfg.blockDim = dim3(THREADS, 1, 1);
+    cfg.dynamicSmemBytes = FShape<true>::SMEM;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, leaf_f32_kernel<true, true>, L.P);
   }
-  delete P;
-  return e;
+  if (L.form == kFNarrowForm)
+    leaf_f32_kernel<false, true, kFNarrow>
+        <<<grid, THREADS, FShape<false, kFNarrow>::SMEM, st>>>(L.P);
+  else
+    leaf_f32_kernel<false, true><<<grid, THREADS, FShape<false>::SMEM, st>>>(L.P);
+  return cudaGetLastError();
 }
 
 void leaf_f32_release() {
@@ -1301,8 +1353,7 @@ void leaf_f32_release() {
   for (auto &kv : g_ftiles)
     if (kv.second.first) cudaFree(kv.second.first);
   g_ftiles.clear();
-  g_fattr[0].clear();
-  g_fattr[1].clear();
+  g_fattr.clear();
   g_attr_c.clear();
   g_pair_units_c.clear();
 }
@@ -1560,16 +1611,27 @@ static void c_two_m(CCtx &c, const float2 *A, int64_t lda, int64_t n, int64_t k,
   float *H = (float *)c.ar.get((size_t)n * n * 4);
   float *G = (float *)c.ar.get((size_t)n * n * 4);
   void *table = c.ar.get(fused_table_bytes());
-  // FP32 class (three pieces): FP16 pieces, decided on the device
+  // FP32 class (three pieces): FP16 pieces, decided on the device.  A A^H reads
+  // A for its diagonal anyway; A A^T pays a launch and a pass for the row
+  // scales, so only where the three products it saves take longer than that
+  // (~3 us).
   RowScale rs = {};
-  if (c.np == 3) {
+  const double saved = std::ceil(1.5 * (double)n * n / (BM * BN * 152.0)) *
+                       (double)((k + BK - 1) / BK) * 3.0 * 512.0;
+  if (c.np == 3 && (herm || saved > 6000.0)) {
     rs.e = (int32_t *)c.ar.get((size_t)(n + 1) * 4);
     rs.wide = rs.e + n;
   }
   if (herm) rs.diag = (float *)c.ar.get((size_t)n * 4);
   if (!c.ar.dry) {
-    if (rs.e || rs.diag) {
-      if (rs.e) cchk(c, cudaMemsetAsync(rs.wide, 0, 4, c.st), "row flag");
+    // H = Ar Ai^T (all entries) and G = (Ar + Ai)(Ar +- Ai)^T (lower tiles)
+    // in one launch; G's sum operands keep every stored piece
+    const std::vector<FusedJob> jobs = {
+        FusedJob{&X, &Y, 0, 0, c.keep, H, n, n, n, 0},
+        FusedJob{&X, herm ? &X : &Y, 1, 1, c.np, G, n, n, n, 1}};
+    FusedLaunch fl;
+    cchk(c, fused_table(jobs, c.np, k, table, c.st, rs.wide, &fl), "2M jobs");
+    if (c.err == AAT_OK && (rs.e || rs.diag)) {
       ProfScope prof(AAT_K_COPY, c.st, (double)n * k * 8.0);
       row_stats_kernel<<<(unsigned)((n * 32 + 255) / 256), 256, 0, c.st>>>(A, lda, n, k, rs);
       cchk(c, cudaGetLastError(), "row scales and diagonal");
@@ -1581,15 +1643,8 @@ static void c_two_m(CCtx &c, const float2 *A, int64_t lda, int64_t n, int64_t k,
     o.s = Xs;
     o.im = Yi;
     if (!herm) o.d = Ysd;
-    csplit(c, A, lda, n, k, o, rs);
-    // H = Ar Ai^T (all entries) and G = (Ar + Ai)(Ar +- Ai)^T (lower tiles)
-    // in one launch; G's sum operands keep every stored piece
-    if (c.err == AAT_OK) {
-      const std::vector<FusedJob> jobs = {
-          FusedJob{&X, &Y, 0, 0, c.keep, H, n, n, n, 0},
-          FusedJob{&X, herm ? &X : &Y, 1, 1, c.np, G, n, n, n, 1}};
-      cchk(c, launch_leaf_f32_fused(jobs, c.np, k, table, c.st, rs.wide), "2M H and G");
-    }
+    if (c.err == AAT_OK) csplit(c, A, lda, n, k, o, rs);
+    if (c.err == AAT_OK) cchk(c, fused_launch(fl, c.st), "2M H and G");
     if (c.err == AAT_OK) {
       const int64_t nt = (n + T - 1) / T;
       ProfScope prof(AAT_K_POSTADD, c.st, (double)n * n * (4.0 * 1.5 + 8.0 * 0.5));
@@ -1716,8 +1771,10 @@ static void c_last_level_fused(CCtx &c, const float2 *A, int64_t lda, int64_t n,
       jobs.push_back(FusedJob{&X2[q], &Y2[q], 0, 0, c.keep, Hb[q], h, h, h, 0});
       jobs.push_back(FusedJob{&X2[q], &Y2[q], 1, 1, c.np, Gb[q], h, h, h, 1});
     }
+    FusedLaunch fl;
     if (c.err == AAT_OK)
-      cchk(c, launch_leaf_f32_fused(jobs, c.np, kap, table, c.st), "fused complex leaves");
+      cchk(c, fused_table(jobs, c.np, kap, table, c.st, nullptr, &fl), "fused complex jobs");
+    if (c.err == AAT_OK) cchk(c, fused_launch(fl, c.st), "fused complex leaves");
     const int64_t nt = (h + T - 1) / T;
     if (c.err == AAT_OK) {
       ProfScope prof(AAT_K_POSTADD, c.st, (double)h * h * 2.0 * (12.0 + 8.0));

@@ -372,8 +372,8 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 // Add 16 consecutive FP32 TMEM columns of this thread's lane into the FP32
 // registers acc[B .. B+15] (round to nearest): load, wait and add in one
 // statement (half the temporaries of the 32-column form).
-template <int B>
-__device__ __forceinline__ void tmem_accum16f(uint32_t taddr, float (&acc)[128]) {
+template <int B, int N>
+__device__ __forceinline__ void tmem_accum16f(uint32_t taddr, float (&acc)[N]) {
   asm volatile(
       "{\n\t.reg .f32 t0, t1, t2, t3, t4, t5, t6, t7, t8, t9, t10, t11, t12, t13, t14, t15;\n\t"
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {t0, t1, t2, t3, t4, t5, t6, t7, t8, t9, t10, t11, t12, t13, t14, t15}, [%16];\n\t"
