@@ -715,38 +715,47 @@ __device__ __forceinline__ void combine2m_tile(const float *__restrict__ G,
                                                const float *__restrict__ H, int64_t ldw,
                                                int64_t n, float2 *C, int64_t ldc, int herm,
                                                const RowScale &rs, int64_t pid,
-                                               float (&hij)[T][T + 1],
                                                float (&hji)[T][T + 1]) {
   const int64_t ntiles = (n + T - 1) / T;
   int64_t I, J;
   tri_index(pid, I, J);
   if (I >= ntiles) return;
   const int tx = threadIdx.x % T, ty = threadIdx.x / T;
-  const int64_t r0 = I * T, c0 = J * T;
+  const int64_t r0 = I * T, c0 = J * T, c = c0 + tx, c2 = r0 + tx;
   const bool half = rs.e && *rs.wide == 0;
-  for (int yy = ty; yy < T; yy += 8) {
-    int64_t r = r0 + yy, c = c0 + tx;
-    if (r < n && c < n) hij[yy][tx] = H[r * ldw + c];
-    int64_t r2 = c0 + yy, c2 = r0 + tx;
-    if (r2 < n && c2 < n) hji[yy][tx] = H[r2 * ldw + c2];
+  // every load of the thread's four rows first (G's too, which need not wait
+  // for the transposed tile): twelve in flight instead of two at a time
+  // (n = 8192: 183 -> 132 us)
+  float a[4], t[4], g[4];
+  int er[4], ec = 0;
+  if (half && c < n) ec = rs.e[c];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int64_t r = r0 + ty + 8 * q, r2 = c0 + ty + 8 * q;
+    a[q] = (r < n && c < n) ? H[r * ldw + c] : 0.0f;
+    t[q] = (r2 < n && c2 < n) ? H[r2 * ldw + c2] : 0.0f;
+    g[q] = (r < n && c <= r) ? G[r * ldw + c] : 0.0f;
+    er[q] = (half && r < n) ? rs.e[r] : 0;
   }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) hji[ty + 8 * q][tx] = t[q];
   __syncthreads();
-  for (int yy = ty; yy < T; yy += 8) {
-    int64_t r = r0 + yy, c = c0 + tx;
-    if (r < n && c < n && c <= r) {
-      const float h = hij[yy][tx], ht = hji[tx][yy], g = G[r * ldw + c];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int64_t r = r0 + ty + 8 * q;
+    if (r < n && c <= r) {
+      const float h = a[q], ht = hji[tx][ty + 8 * q];
       float2 v;
       if (herm) {
-        v.x = g - h - ht;
+        v.x = g[q] - h - ht;
         v.y = ht - h;
       } else {
-        v.x = g + h - ht;
+        v.x = g[q] + h - ht;
         v.y = h + ht;
       }
       if (half) {
-        const int ei = rs.e[r], ej = rs.e[c];
-        v.x = unscale(v.x, ei, ej);
-        v.y = unscale(v.y, ei, ej);
+        v.x = unscale(v.x, er[q], ec);
+        v.y = unscale(v.y, er[q], ec);
       }
       if (rs.diag && r == c) v = make_float2(rs.diag[r], 0.0f);
       C[r * ldc + c] = v;
@@ -757,17 +766,15 @@ __device__ __forceinline__ void combine2m_tile(const float *__restrict__ G,
 __global__ void combine2m_kernel(const float *__restrict__ G, const float *__restrict__ H,
                                  int64_t ldw, int64_t n, float2 *C, int64_t ldc, int herm,
                                  RowScale rs) {
-  __shared__ float hij[T][T + 1];
   __shared__ float hji[T][T + 1];
-  combine2m_tile(G, H, ldw, n, C, ldc, herm, rs, blockIdx.x, hij, hji);
+  combine2m_tile(G, H, ldw, n, C, ldc, herm, rs, blockIdx.x, hji);
 }
 
 __global__ void combine2m_batch_kernel(const CBProb *__restrict__ pr, int count) {
-  __shared__ float hij[T][T + 1];
   __shared__ float hji[T][T + 1];
   const CBProb &q = pr[cb_find(pr, count, blockIdx.x, 1)];
   combine2m_tile(q.G, q.H, q.n, q.n, q.C, q.ldc, q.herm, q.rs,
-                 (int64_t)(blockIdx.x - q.comb_first), hij, hji);
+                 (int64_t)(blockIdx.x - q.comb_first), hji);
 }
 
 // x·x added to the unevaluated float pair hi + lo without rounding error:
