@@ -267,6 +267,31 @@ static DigitSpec make_digits(uint32_t p) {
   return best;
 }
 
+// The digit form the products run on.  A prime between 2^16 and 2^17 + 1 has
+// two digits, d_1 up to 256, whose balanced pair sum does not fit BF16's 256;
+// with digits of opposite signs (DigitSpec::opp) it does, and three plane
+// products replace the four digit pairs.  16384 x 4096 (lower) mod 131071: leaf
+// 2430 -> 2064 us (all three drained every 4 K blocks, the drains' pace).
+static DigitSpec product_digits(uint32_t p) {
+  DigitSpec d = make_digits(p);
+  if (d.L == 2 && d.nsum == 0 && d.b == 8 && (p - 1) / 2 <= 65536) {
+    d.opp = 1;
+    d.dmax[0] = 255;
+    d.dmax[1] = 256;
+    d.nsum = 1;
+    d.si[0] = 0;
+    d.sj[0] = 1;
+  }
+  return d;
+}
+
+// One product per digit pair.
+static DigitSpec plain_digits(uint32_t p) {
+  DigitSpec d = make_digits(p);
+  d.nsum = 0;
+  return d;
+}
+
 // ------------------------------------------------------- device state
 
 struct DeviceState {
@@ -404,6 +429,11 @@ struct Ctx {
   Arena ar;
   aatx_plan_stats_t *stats;  // optional counters
   int err = AAT_OK;
+  // the digit form of products (entry points; the single-step hooks keep
+  // make_digits' form)
+  void use_product_digits(uint32_t flags) {
+    if (!(flags & AAT_DIGITS_PLAIN)) ds = product_digits(m.p);
+  }
   // optional: recorded on `st` as soon as rows [split_row, n) of C are final
   // (after the top level's post-additions; at the end when C is padded)
   cudaEvent_t split_ev = nullptr;
@@ -448,6 +478,7 @@ static Planes planes_for(const DigitSpec &ds, int64_t rows, int64_t cols) {
   P.nbase = ds.L;
   P.nsum = ds.nsum;
   P.L = ds.L + ds.nsum;
+  P.opp = ds.opp;
   for (int q = 0; q < ds.nsum; ++q) {
     P.si[q] = (int8_t)ds.si[q];
     P.sj[q] = (int8_t)ds.sj[q];
@@ -1135,7 +1166,7 @@ static size_t run_plan_in(Ctx &c, const int32_t *A, int64_t n, int64_t k, int64_
   if (c.leaf == AAT_LEAF_TC && !(flags & AAT_LEVELS_MASK) && tune_find(n, k, c.m.p, &tv)) {
     flags |= AAT_LEVELS(tv.levels);
     c.form = tv.form;
-    if (tv.plain) c.ds.nsum = 0;
+    if (tv.plain) c.ds = plain_digits(c.m.p);
     if (tv.wino) c.wino = true;
   }
   Prepared pr = prepare(n, k, c.m.p, c.y, flags);
@@ -1346,13 +1377,12 @@ Planes planes_layout(const DigitSpec &ds, int64_t rows, int64_t cols) {
 }
 
 DigitSpec digits_for_problem(int64_t n, int64_t k, uint32_t p, uint32_t flags) {
-  DigitSpec d = make_digits(p);
   TuneVal tv;
-  if (flags & AAT_DIGITS_PLAIN) d.nsum = 0;
-  else if (!(flags & AAT_LEVELS_MASK) && (flags & AAT_LEAF_MASK) == AAT_LEAF_TC &&
-           tune_find(n, k, p, &tv) && tv.plain)
-    d.nsum = 0;
-  return d;
+  if ((flags & AAT_DIGITS_PLAIN) ||
+      (!(flags & AAT_LEVELS_MASK) && (flags & AAT_LEAF_MASK) == AAT_LEAF_TC &&
+       tune_find(n, k, p, &tv) && tv.plain))
+    return plain_digits(p);
+  return product_digits(p);
 }
 
 int modp_run(const int32_t *A, int64_t n, int64_t k, int64_t lda, uint32_t p, int32_t *C,
@@ -1360,6 +1390,7 @@ int modp_run(const int32_t *A, int64_t n, int64_t k, int64_t lda, uint32_t p, in
   Ctx c;
   int e = setup(c, p, flags, st);
   if (e) return e;
+  c.use_product_digits(flags);
   // the schedule as for a single call (fast, or low-memory by flag or limit)
   size_t peak = choose_schedule(c, A, n, k, lda, C, ldc, flags);
   if (!dry) peak = run_plan(c, A, n, k, lda, C, ldc, flags, false, ws);
@@ -1411,6 +1442,7 @@ static int modp_device(const int32_t *A, int64_t n, int64_t k, int64_t lda, uint
   }
   c.form = form;
   c.small_ok = true;
+  c.use_product_digits(flags);
   c.in_a11 = in_a11;
   c.in_rest = in_rest;
   c.in_bands = in_bands;
@@ -1484,6 +1516,7 @@ int aat_syrk_modp(uint32_t alpha, const int32_t *A, int64_t n, int64_t k, int64_
   if ((e = check_device())) return e;
   const MulConst b = mul_const(beta, p);
   c.alpha = mul_const(alpha, p).w;
+  c.use_product_digits(flags);
   cudaError_t ce = cudaSuccess;
   if (k == 0 || c.alpha == 0) {
     // Low(C) <- beta Low(C)
@@ -1536,6 +1569,7 @@ int aah_quat_modp(const int32_t *A, const int32_t *B, const int32_t *C, const in
     }
     return AAT_OK;
   }
+  c.use_product_digits(flags);
   const size_t need = quat_plan(c, M, n, k, lda, H, ldh, flags, true, nullptr);
   void *ws = nullptr;
   if ((e = ensure_workspace(need, &ws))) return e;
@@ -1717,7 +1751,7 @@ int aat_tune_modp(int64_t n, int64_t k, uint32_t p, uint32_t flags, int reps, vo
   cands.push_back({flags, -1, 0, 0, 1e300, 0});
   int maxl = 0;
   while (maxl < 3 && (n >> (maxl + 1)) >= 512 && (k >> (maxl + 1)) >= 128) ++maxl;
-  const bool sums = make_digits(p).nsum > 0;
+  const bool sums = product_digits(p).nsum > 0;
   for (int l = 0; l <= maxl; ++l)
     for (int form = 1; form <= 2; ++form) {
       if (form == 2 && (n >> l) < 256) continue;  // no leaf tall enough for a pair
@@ -1904,6 +1938,7 @@ int aat_gemm_modp(const int32_t *X, int64_t ldx, const int32_t *Y, int64_t ldy, 
   }
   const bool same = (X == Y && ldx == ldy && m == n);
   c.small_ok = true;
+  c.use_product_digits(flags);
   size_t need = 0;
   for (int pass = 0; pass < 2; ++pass) {
     void *ws = nullptr;
@@ -1924,6 +1959,7 @@ size_t aat_workspace_size(int64_t n, int64_t k, uint32_t p, uint32_t flags) {
   Ctx c;
   if (n <= 0 || k <= 0 || setup(c, p, flags, nullptr)) return 0;
   c.small_ok = true;
+  c.use_product_digits(flags);
   return choose_schedule(c, nullptr, n, k, k, nullptr, n, flags);
 }
 

@@ -206,6 +206,7 @@ struct Planes {
   int nsum;     // pair-sum planes of the sequence (after the digit planes)
   int8_t si[8], sj[8];  // pair of plane nbase + q (always (0,1), (0,2), ...)
   int q0;       // first stored plane (0 unless only a window of the planes is kept)
+  int opp;      // two digits of opposite signs (DigitSpec::opp)
 };
 
 struct DigitSpec {
@@ -214,6 +215,9 @@ struct DigitSpec {
   int dmax[8];    // bound on |digit| per position
   int nsum;       // pair-sum planes (0: every digit pair is its own product)
   int si[8], sj[8];
+  int opp;        // two base-256 digits of opposite signs: d_1 = x / 256 rounded
+                  // away from zero, so |d_0| <= 255, |d_1| <= 256 and their sum
+                  // lies between d_0 and d_1
 };
 
 __device__ __forceinline__ uint2 pack4(float a, float b, float c, float d) {
@@ -243,6 +247,13 @@ __device__ __forceinline__ void store_digits_t(const Planes &P, int64_t r, int64
 #pragma unroll
   for (int v = 0; v < V; ++v) {
     int32_t x = x0[v];
+    if constexpr (NB == 2) {
+      if (P.opp) {
+        dig[1][v] = (x + (x > 0 ? 255 : 0)) >> 8;
+        dig[0][v] = x - (dig[1][v] << 8);
+        continue;
+      }
+    }
 #pragma unroll
     for (int d = 0; d < NB - 1; ++d) {
       dig[d][v] = ((x + half) & mask) - half;

@@ -917,7 +917,8 @@ bool build_groups(const TcLeafArgs &a, const ModP &m, Group *out, int *ng_out, i
     }
     for (int q = 0; q < a.dx.nsum; ++q) {
       const int i = a.dx.si[q], j = a.dx.sj[q];
-      const int64_t bx = a.dx.dmax[i] + a.dx.dmax[j], by = a.dy.dmax[i] + a.dy.dmax[j];
+      const int64_t bx = a.dx.opp ? 256 : a.dx.dmax[i] + a.dx.dmax[j];
+      const int64_t by = a.dy.opp ? 256 : a.dy.dmax[i] + a.dy.dmax[j];
       terms.push_back({L + q, L + q, zp(i + j), bx * by});
     }
   } else {

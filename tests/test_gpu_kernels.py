@@ -296,3 +296,31 @@ def test_half_width_pair_tiles(lib, M, N, K, p):
     rows = sorted({0, 1, 127, 128, 255, 256, 257, 2047, 2048, M - 2, M - 1})
     ref = (X[rows].astype(object) @ Y.astype(object).T) % p
     assert np.array_equal(got[rows].astype(object), ref)
+
+
+@pytest.mark.parametrize("p", [65537, 65539, 131041, 131071])
+@pytest.mark.parametrize("worst", [False, True])
+@pytest.mark.parametrize("n,k", [(300, 2200), (1030, 600), (64, 5000)])
+def test_two_digits_of_opposite_signs(lib, n, k, p, worst):
+    """Primes whose two digits need opposite signs for their pair sum: random
+    residues, and sums of one sign at the digits' ends over all of K."""
+    import torch
+    half = (p - 1) // 2
+    if worst:
+        ends = np.array([half, -half, half - 255, 65280 if half >= 65280 else half - 1, 1, -1])
+        A = np.tile(ends[np.arange(n) % len(ends)][:, None], (1, k)).astype(np.int32)
+    else:
+        A = synth.residues(n + k, (n, k), p)
+    D = torch.from_numpy(A).cuda()
+    ref = torch.remainder((D.double() @ D.double().T).to(torch.int64), p)   # < 2^53
+    assert torch.equal(lib.aat_gemm_modp(D, D, p).long(), ref)
+    for levels in (0, 1, 2):
+        got = lib.aat_modp(D, p, levels=levels, flags=lib.AAT_ZERO_UPPER)
+        assert torch.equal(got.long(), ref.tril()), levels
+    low = lib.aat_modp(D, p, levels=1, flags=lib.AAT_ZERO_UPPER | lib.AAT_LOW_MEMORY)
+    assert torch.equal(low.long(), ref.tril())
+    C = torch.zeros((n, n), dtype=torch.int32, device="cuda")
+    plan = lib.Plan([("modp", D, C, p, 0)])
+    plan.execute()
+    assert torch.equal(C.long().tril(), ref.tril())
+    plan.close()
