@@ -676,7 +676,7 @@ static void leaf(Ctx &c, Operand X, Operand Y, bool same, int64_t M, int64_t N, 
     c.ar.used = mark;
     return;
   }
-
+  a.zero = c.zeroed = c.want_zero;
   if (!c.ar.dry && c.err == AAT_OK) check(c, launch_leaf_tc(a, c.m, c.st), "leaf (tensor cores)");
   c.ar.used = mark;
 }

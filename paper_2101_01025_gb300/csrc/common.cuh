@@ -437,6 +437,7 @@ struct TcLeafArgs {
   Lin lin;                // out <- alpha product + beta out
   int exact_bits;         // |partial FP32 sums| kept <= 2^exact_bits
   int form;               // kernel form: 0 chosen from the shape, 1 one CTA, 2 CTA pairs
+  bool zero = false;      // lower, launch_leaf_tc only: clear the strict upper triangle
 };
 cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st);
 // Up to 16 independent leaf products of one modulus and digit base in one

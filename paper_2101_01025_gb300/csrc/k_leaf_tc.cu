@@ -27,6 +27,8 @@
 //                 M=128 N=256 K=16 per instruction (CTA pair: M=256 across
 //                 the pair, issued by the leader), FP32 accumulator in one of
 //                 two 256-column TMEM buffers (double buffered per chunk)
+//   warp 10       (8 epilogue warps) clears the strict upper triangle of a
+//                 lower product, tile by tile, where that is asked for
 //   warps 2..9    epilogue: tcgen05.ld of the finished chunk, float -> int32,
 //                 accumulate; mod-p Horner step at digit-pair boundaries;
 //                 canonical store (lower triangle only for SYRK leaves)
@@ -113,6 +115,7 @@ struct Params {
   const int2 *tiles;
   int ntiles;
   int lower, accumulate;  // accumulate: out <- product + beta out
+  int zero;  // lower products: clear the strict upper triangle (single launches)
   uint32_t beta, beta_sh;
   ModP m;
   int32_t *status;
@@ -275,7 +278,8 @@ __device__ __forceinline__ OutView tile_out(const Params &P, int t) {
 template <bool PAIR, int EW = 8, int TN = 256>
 struct Shape {
   static constexpr int EPI_WARPS = EW;
-  static constexpr int THREADS = 64 + EW * 32;
+  // producer, MMA issuer, epilogue and (8 epilogue warps) the clearing warp
+  static constexpr int THREADS = 64 + EW * 32 + (EW == 8 ? 32 : 0);
   static constexpr int VALS = 4 * TN / EW;        // accumulators per thread
   static constexpr int XB = EW == 8 ? 16 : 8;     // staged store block width
   static constexpr int TM = PAIR ? 256 : 128;     // output tile rows
@@ -518,6 +522,36 @@ __global__ void __launch_bounds__(Shape<PAIR, EW, TN>::THREADS, 1)
         wait_quiet(DONE, 0);
       }
       __syncwarp();
+    }
+  } else if (EW == 8 && warp == 2 + EW) {
+    // ---------------------------------------------------- clearing the mirror
+    // P.zero: entry (c, r) for every entry (r, c) below the diagonal of this
+    // CTA's part of the tile, one row of 128 entries per 16-byte store of the
+    // warp.  A warp of its own, so that the stores' back-pressure delays nobody:
+    // a clearing kernel after the product took 81-155 us at n = 16384; the
+    // epilogue's warps took as long (their drains wait behind the stores).
+    // 16384 x 4096 mod 131071 with the clearing 2427 -> 2388 us, 8192^2 mod 65521
+    // 1098 -> 1092.
+    if constexpr (MODE == kSingle) {
+      const bool vec = ((reinterpret_cast<uintptr_t>(P.out) | (uintptr_t)(P.ldo * 4)) & 15) == 0;
+      for (int t = (int)unit0; P.zero && t < P.ntiles; t += (int)nunits) {
+        const int2 ij = P.tiles[t];
+        const int64_t r0 = (int64_t)ij.x * S::TM + (int64_t)rank * BM;
+        const int64_t c0 = (int64_t)ij.y * TN;
+        const int64_t c1 = min(min(c0 + TN, P.N), min(r0 + BM, P.M) - 1);
+        for (int64_t c = c0; c < c1; ++c) {
+          int32_t *z = P.out + c * P.ldo + r0;
+          if (vec && c < r0 && r0 + BM <= P.M) {
+            *reinterpret_cast<int4 *>(z + 4 * lane) = make_int4(0, 0, 0, 0);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const int64_t r = r0 + lane + 32 * j;
+              if (r > c && r < P.M) z[lane + 32 * j] = 0;
+            }
+          }
+        }
+      }
     }
   } else {
     // ---------------------------------------------------------- epilogue
@@ -1172,6 +1206,7 @@ Form leaf_form(const TcLeafArgs *as, int count, int units, int sms) {
 
 cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) {
   if (a.M <= 0 || a.N <= 0) return cudaSuccess;
+  if (a.zero && (!a.lower || a.M != a.N)) return cudaErrorInvalidValue;
   if (a.dx.b != a.dy.b || a.x.nbase != a.dx.L || a.y.nbase != a.dy.L || !window_ok(a.x) ||
       !window_ok(a.y))
     return cudaErrorInvalidValue;
@@ -1208,6 +1243,7 @@ cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) 
   P->N = a.N;
   P->lower = a.lower;
   P->accumulate = a.lin.beta.w != 0u;
+  P->zero = a.zero;
   P->beta = a.lin.beta.w;
   P->beta_sh = a.lin.beta.wsh;
   P->m = m;
