@@ -1582,6 +1582,109 @@ int aat_modp(const int32_t *A, int64_t n, int64_t k, uint32_t p, int32_t *C, voi
   return aat_modp_ex(A, n, k, k, p, C, n, 0u, stream);
 }
 
+// The end-to-end product without recursion levels in two row parts of about
+// equal work: rows [0, r1) of C need only rows [0, r1) of A, so the rest of A
+// comes in while they are computed, and they go back while the rows below,
+// C21 = A2 A1^T and Low(C22) = Low(A2 A2^T) in one launch, are computed.
+// Copies, product and copies one after the other took 2.85 ms at 6000 x 5000
+// mod 2^31 - 1 (0.6 + 1.5 + 0.7), two parts 2.49 ms; 8192 x 8192 5.9 -> 4.5 ms.
+// The row split with the shortest modelled sequence: the first rows in, both
+// launches (whole waves of tiles), the last rows out.  0: one part.
+static int64_t host_two_parts_rows(const Ctx &c, int64_t n, int64_t k, uint32_t flags) {
+  TuneVal tv;
+  if (c.leaf != AAT_LEAF_TC || c.passes || prepare_levels(n, k, c.m.p, flags) != 0 ||
+      (!(flags & AAT_LEVELS_MASK) && tune_find(n, k, c.m.p, &tv)))
+    return 0;
+  const double us_per_byte = 1e6 / 200e9;  // the host link, either way
+  const bool zero = (flags & AAT_ZERO_UPPER) != 0;
+  auto model = [&](int64_t r1) {
+    const Planes P1 = planes_for(c.ds, r1, k), P2 = planes_for(c.ds, n - r1, k);
+    const TcLeafArgs a = tc_args(c, P1, P1, r1, r1, k, nullptr, n, 1, 0);
+    double t = (double)r1 * k * 4.0 * us_per_byte + leaf_tc_model_us(&a, 1);
+    if (r1 == n) return t + (zero ? (double)n * n : 0.5 * (double)n * n) * 4.0 * us_per_byte;
+    const TcLeafArgs b[2] = {tc_args(c, P2, P1, n - r1, r1, k, nullptr, n, 0, 0),
+                             tc_args(c, P2, P2, n - r1, n - r1, k, nullptr, n, 1, 0)};
+    t += leaf_tc_model_us(b, 2);
+    return t + (double)(n - r1) * n * 4.0 * us_per_byte;
+  };
+  int64_t best = 0;
+  double bt = 0.9 * model(n);
+  // multiples of 512, as the bands in which the lower triangle goes back
+  for (int64_t r1 = 512; r1 + 512 <= n; r1 += 512) {
+    const double t = model(r1);
+    if (t < bt) {
+      bt = t;
+      best = r1;
+    }
+  }
+  return best;
+}
+
+static int host_two_parts(Ctx &c, const int32_t *A_host, int32_t *Ad, int64_t n, int64_t k,
+                          int32_t *C_host, int32_t *Cd, uint32_t flags, int64_t r1,
+                          DeviceState *s) {
+  cudaStream_t st = s->e2e_stream, s2 = s->e2e_stream2;
+  const bool zero = (flags & AAT_ZERO_UPPER) != 0;
+  const int64_t r2 = n - r1;
+  cudaError_t ce;
+  c.st = st;
+  void *ws = nullptr;
+  size_t need = 0;
+  for (int pass = 0; pass < 2; ++pass) {
+    c.ar = Arena();
+    c.ar.dry = pass == 0;
+    c.ar.base = (char *)ws;
+    const Planes P1 = planes_alloc(c, r1, k), P2 = planes_alloc(c, r2, k);
+    if (pass == 0) {
+      need = c.ar.peak;
+      int e = need > g_ws_limit.load() ? AAT_ENOMEM : ensure_workspace(need, &ws);
+      if (e) return e;  // the caller takes the one-part path
+      continue;
+    }
+    if ((ce = cudaMemcpyAsync(Ad, A_host, (size_t)r1 * k * 4, cudaMemcpyHostToDevice, s2)) !=
+            cudaSuccess ||
+        (ce = cudaEventRecord(s->e2e_a11, s2)) != cudaSuccess ||
+        (ce = cudaMemcpyAsync(Ad + r1 * k, A_host + r1 * k, (size_t)r2 * k * 4,
+                              cudaMemcpyHostToDevice, s2)) != cudaSuccess ||
+        (ce = cudaEventRecord(s->e2e_rest, s2)) != cudaSuccess)
+      return cuda_fail(ce, "copy A to the device");
+    // rows [0, r1)
+    cudaStreamWaitEvent(st, s->e2e_a11, 0);
+    if (zero && (ce = cudaMemset2DAsync(Cd + r1, (size_t)n * 4, 0, (size_t)r2 * 4, (size_t)r1, st)) !=
+                    cudaSuccess)
+      return cuda_fail(ce, "zero upper");
+    check(c, launch_split(Ad, k, r1, k, c.m, c.ds.b, P1, st), "split");
+    TcLeafArgs a = tc_args(c, P1, P1, r1, r1, k, Cd, n, 1, 0);
+    a.zero = zero;
+    if (c.err == AAT_OK) check(c, launch_leaf_tc(a, c.m, st), "leaf (tensor cores)");
+    if ((ce = cudaEventRecord(s->e2e_split, st)) != cudaSuccess) return cuda_fail(ce, "event");
+    // rows [r1, n)
+    cudaStreamWaitEvent(st, s->e2e_rest, 0);
+    int32_t *C21 = Cd + r1 * n, *C22 = C21 + r1;
+    check(c, launch_split(Ad + r1 * k, k, r2, k, c.m, c.ds.b, P2, st), "split");
+    const TcLeafArgs b[2] = {tc_args(c, P2, P1, r2, r1, k, C21, n, 0, 0),
+                             tc_args(c, P2, P2, r2, r2, k, C22, n, 1, 0)};
+    if (c.err == AAT_OK) check(c, launch_leaf_tc_multi(b, 2, c.m, st), "leaf (tensor cores, rows)");
+    if (zero) check(c, launch_zero_upper(C22, n, r2, st), "zero upper");
+    if (c.err != AAT_OK) {
+      cudaStreamSynchronize(s2);
+      cudaStreamSynchronize(st);
+      return c.err;
+    }
+    // the copies back are enqueued last: into pageable memory they block
+    if ((ce = cudaStreamWaitEvent(s2, s->e2e_split, 0)) != cudaSuccess ||
+        (ce = zero ? cudaMemcpyAsync(C_host, Cd, (size_t)r1 * n * 4, cudaMemcpyDeviceToHost, s2)
+                   : copy_low_bands(C_host, Cd, n, 0, r1, s2)) != cudaSuccess ||
+        (ce = zero ? cudaMemcpyAsync(C_host + r1 * n, C21, (size_t)r2 * n * 4,
+                                     cudaMemcpyDeviceToHost, st)
+                   : copy_low_bands(C_host, Cd, n, r1, n, st)) != cudaSuccess)
+      return cuda_fail(ce, "copy C to the host");
+    if ((ce = cudaStreamSynchronize(s2)) != cudaSuccess) return cuda_fail(ce, "synchronize");
+    if ((ce = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(ce, "synchronize");
+  }
+  return AAT_OK;
+}
+
 int aat_modp_host(const int32_t *A_host, int64_t n, int64_t k, uint32_t p, int32_t *C_host,
                   uint32_t flags) {
   g_last_error.clear();
@@ -1626,6 +1729,18 @@ int aat_modp_host(const int32_t *A_host, int64_t n, int64_t k, uint32_t p, int32
   cudaStream_t st = s->e2e_stream;
   cudaError_t ce;
   const int32_t *Cd = (const int32_t *)s->e2e_c;
+  if (k > 0) {
+    Ctx c;
+    if ((e = setup(c, p, flags, st))) return e;
+    c.use_product_digits(flags);
+    const int64_t r1 = host_two_parts_rows(c, n, k, flags);
+    if (r1 > 0) {
+      e = host_two_parts(c, A_host, (int32_t *)s->e2e_a, n, k, C_host, (int32_t *)s->e2e_c, flags,
+                         r1, s);
+      if (e != AAT_ENOMEM) return e;
+      g_last_error.clear();
+    }
+  }
   if (!(flags & AAT_ZERO_UPPER) && n >= 2 && k >= 2) {
     // A comes in on the second stream, its top-left block A11 (rows and
     // columns below n/2, k/2) first: when a recursion level runs, the

@@ -456,6 +456,8 @@ LeafSplit leaf_tc_split(const TcLeafArgs &a);
 cudaError_t launch_partial_sum(const int32_t *W, int64_t ldw, int64_t stride, int parts,
                                int32_t *out, int64_t ldo, int64_t M, int64_t N, int lower,
                                bool zero, const MulConst &beta, const ModP &m, cudaStream_t st);
+// Modelled time of one launch over `count` products.
+double leaf_tc_model_us(const TcLeafArgs *as, int count);
 // Whether that one launch is expected to beat one launch per product (the
 // idle share of the separate launches' last waves).
 bool leaf_tc_fuse_pays(const TcLeafArgs *as, int count);

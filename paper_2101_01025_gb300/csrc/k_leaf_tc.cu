@@ -1155,7 +1155,7 @@ double tile_cycles(int narrow, double kb, double terms) {
 // the one product of 512 x 512 mod 131071 with one level, 23.5 -> 10.4 and
 // 38.1 -> 12.0 us; 2048 x 2048 x 1500 (lower) mod 65521, 72 wide or 272
 // narrow tiles: 40.8 -> 31 us.
-Form leaf_form(const TcLeafArgs *as, int count, int units, int sms) {
+Form leaf_form(const TcLeafArgs *as, int count, int units, int sms, double *cycles = nullptr) {
   const int ov = as[0].form > 0 ? as[0].form - 1 : pair_override();
   if (units > 0) {
     bool big = true;
@@ -1184,7 +1184,9 @@ Form leaf_form(const TcLeafArgs *as, int count, int units, int sms) {
         }
         cost[w] = work / (double)tiles * (double)((tiles + units - 1) / units);
       }
-      return cost[1] < 0.97 * cost[0] ? kPairHalf : kPair;
+      const bool half = cost[1] < 0.97 * cost[0];
+      if (cycles) *cycles = cost[half];
+      return half ? kPairHalf : kPair;
     }
   }
   double cost[2];
@@ -1199,7 +1201,9 @@ Form leaf_form(const TcLeafArgs *as, int count, int units, int sms) {
     }
     cost[w] = work / (double)tiles * (double)((tiles + sms - 1) / sms);
   }
-  return cost[1] < cost[0] ? kNarrow : kCta;
+  const bool narrow = cost[1] < cost[0];
+  if (cycles) *cycles = cost[narrow];
+  return narrow ? kNarrow : kCta;
 }
 
 }  // namespace
@@ -1381,6 +1385,18 @@ LeafSplit leaf_tc_split(const TcLeafArgs &a) {
       }
     }
   return best;
+}
+
+double leaf_tc_model_us(const TcLeafArgs *as, int count) {
+  int dev = 0, units = 0;
+  cudaGetDevice(&dev);
+  {
+    std::lock_guard<std::mutex> lock(g_mu);
+    units = pair_units(dev);
+  }
+  double cycles = 0.0;
+  leaf_form(as, count, units, sm_count(dev), &cycles);
+  return cycles / 1.9e3;  // at 1.9 GHz
 }
 
 // Several independent products of one modulus and digit base in one

@@ -324,3 +324,30 @@ def test_two_digits_of_opposite_signs(lib, n, k, p, worst):
     plan.execute()
     assert torch.equal(C.long().tril(), ref.tril())
     plan.close()
+
+
+@pytest.mark.parametrize("zero", [False, True])
+@pytest.mark.parametrize("pinned", [False, True])
+@pytest.mark.parametrize("p,n,k", [(2**31 - 1, 5000, 2600), (65521, 6200, 4100), (131071, 4700, 1999)])
+def test_host_product_in_two_row_parts(lib, p, n, k, pinned, zero):
+    """From host memory without recursion levels: both row parts, sampled rows
+    against exact sums, cleared or untouched entries above the bands."""
+    import torch
+    A = torch.from_numpy(synth.residues(n + k, (n, k), p, balanced=True))
+    C = torch.full((n, n), -3, dtype=torch.int32)
+    if pinned:
+        A, C = A.pin_memory(), C.pin_memory()
+    for _ in range(2):  # a second call reuses every buffer and event
+        C.fill_(-3)
+        lib.aat_modp_host(A, p, C=C, flags=lib.AAT_ZERO_UPPER if zero else 0, levels=0)
+        rows = sorted({0, 1, 511, 512, n // 2, n - 513, n - 512, n - 2, n - 1} | set(range(2048, n, 517)))
+        X = A.numpy()
+        for r in rows:
+            lo, hi = X[r].astype(np.int64) & 0xffff, X[r].astype(np.int64) >> 16
+            Y = X[: r + 1].astype(np.int64)
+            ref = ((Y @ hi) % p * 65536 + Y @ lo) % p   # sums below 2^47 p's 2^31: exact in int64
+            assert np.array_equal(C[r, : r + 1].numpy().astype(np.int64), ref), r
+            if zero:
+                assert not C[r, r + 1:].any()
+            else:
+                assert bool((C[r, (r // 512 + 1) * 512:] == -3).all())
