@@ -488,6 +488,7 @@ static Planes planes_for(const DigitSpec &ds, int64_t rows, int64_t cols) {
 
 static Planes planes_alloc(Ctx &c, int64_t rows, int64_t cols) {
   Planes P = planes_for(c.ds, rows, cols);
+  P.kstride = plane_stride(cols);
   P.ptr = (__nv_bfloat16 *)c.ar.get((size_t)P.L * rows * P.kstride * 2);
   return P;
 }
@@ -511,6 +512,7 @@ static int plane_count(const Ctx &c) { return c.ds.L + c.ds.nsum; }
 // Planes q0 .. q0 + w - 1 of an r x c block, in the arena.
 static Planes planes_window(Ctx &c, int64_t rows, int64_t cols, int q0, int w) {
   Planes P = planes_for(c.ds, rows, cols);
+  P.kstride = plane_stride(cols);
   P.q0 = q0;
   P.L = w;
   P.ptr = (__nv_bfloat16 *)c.ar.get((size_t)w * rows * P.kstride * 2);
@@ -1373,7 +1375,9 @@ int modp_levels(int64_t n, int64_t k, uint32_t p, uint32_t flags) {
 }
 
 Planes planes_layout(const DigitSpec &ds, int64_t rows, int64_t cols) {
-  return planes_for(ds, rows, cols);
+  Planes P = planes_for(ds, rows, cols);
+  P.kstride = plane_stride(cols);
+  return P;
 }
 
 DigitSpec digits_for_problem(int64_t n, int64_t k, uint32_t p, uint32_t flags) {

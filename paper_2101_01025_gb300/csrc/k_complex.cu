@@ -1579,7 +1579,7 @@ static Planes cplanes(CCtx &c, int64_t rows, int64_t cols, int sets) {
   std::memset(&P, 0, sizeof(P));
   P.rows = rows;
   P.cols = cols;
-  P.kstride = (cols + 7) / 8 * 8;
+  P.kstride = plane_stride(cols);
   P.L = c.np * sets;
   P.nbase = P.L;
   P.ptr = (__nv_bfloat16 *)c.ar.get((size_t)P.L * rows * P.kstride * 2);
@@ -1944,7 +1944,7 @@ struct CBatchImpl {
 static size_t r256c(size_t x) { return (x + 255) & ~(size_t)255; }
 
 static size_t cb_planes_bytes(int64_t n, int64_t k, int np) {
-  return r256c((size_t)2 * np * n * ((k + 7) / 8 * 8) * 2);
+  return r256c((size_t)2 * np * n * plane_stride(k) * 2);
 }
 
 size_t cbatch_workspace(const CBInput *in, int count) {
@@ -1990,7 +1990,7 @@ cudaError_t cbatch_build(const CBInput *in, int count, char *ws, CBatch *out) {
     std::memset(&X, 0, sizeof(X));
     X.rows = q.n;
     X.cols = q.k;
-    X.kstride = (q.k + 7) / 8 * 8;
+    X.kstride = plane_stride(q.k);
     X.L = X.nbase = 2 * np;
     Y = X;
     X.ptr = (__nv_bfloat16 *)w;
