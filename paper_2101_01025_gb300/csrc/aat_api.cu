@@ -460,6 +460,7 @@ struct Ctx {
   // the product is one leaf whose launch may clear the strict upper triangle
   // (want_zero), and did (zeroed)
   bool want_zero = false, zeroed = false;
+  int zero_levels = 0;  // the depth of the call that may clear
 };
 
 // One CUDA-core launch for a whole product (leaf_small_pays), unless a form
@@ -575,7 +576,7 @@ static void leaf(Ctx &c, Operand X, Operand Y, bool same, int64_t M, int64_t N, 
       check(c, launch_leaf_small(X.x, X.ld, Y.x, Y.ld, M, N, K, out, ldo, lower, c.want_zero, lin,
                                  c.m, c.st),
             "leaf (CUDA cores, small)");
-    c.zeroed = c.want_zero;
+    c.zeroed = c.want_zero;  // small products have no levels
     return;
   }
   if (c.leaf == AAT_LEAF_SIMT) {
@@ -671,14 +672,14 @@ static void leaf(Ctx &c, Operand X, Operand Y, bool same, int64_t M, int64_t N, 
         check(c, launch_leaf_tc_multi(parts.data(), (int)parts.size(), c.m, c.st),
               "leaf (tensor cores, parts)");
       check(c, launch_partial_sum(W, ldw, stride, (int)parts.size(), out, ldo, M, N, lower,
-                                  c.want_zero, lin.beta, c.m, c.st),
+                                  c.want_zero && c.zero_levels == 0, lin.beta, c.m, c.st),
             "sum of parts");
     }
-    c.zeroed = c.want_zero;
+    if (c.want_zero && c.zero_levels == 0) c.zeroed = true;
     c.ar.used = mark;
     return;
   }
-  a.zero = c.zeroed = c.want_zero;
+  if (c.want_zero && c.zero_levels == 0) a.zero = c.zeroed = true;
   if (!c.ar.dry && c.err == AAT_OK) check(c, launch_leaf_tc(a, c.m, c.st), "leaf (tensor cores)");
   c.ar.used = mark;
 }
@@ -888,8 +889,9 @@ static void rec(Ctx &c, const int32_t *A, int64_t lda, int64_t n, int64_t k, int
   // 2-5 at the last level: P4^T, P5, P3 and P1 read only digit planes
   // written by step 1 and write four different blocks of C, so they may run
   // as one persistent launch over the tiles of all four
-  TcLeafArgs fa[4];
+  TcLeafArgs fa[5];
   int nfa = 0;
+  bool p2_done = false;
   if (last && c.leaf == AAT_LEAF_TC) {
     fa[nfa++] = tc_args(c, L.oS2.pl, L.oS1.pl, h, h, kap, C22, ldc, 0, 0);
     fa[nfa++] = tc_args(c, L.pS3, L.pS3, h, h, kap, C12, ldc, 1, 0);
@@ -901,9 +903,19 @@ static void rec(Ctx &c, const int32_t *A, int64_t lda, int64_t n, int64_t k, int
     const TcLeafArgs sym[2] = {fa[1], fa[nfa - 1]};  // P5, and P1 unless it ran first
     wino_products(c, L, A + h * lda + kap, lda, h, kap, C21, C22, ldc, sym, p1_first ? 1 : 2);
   } else if (nfa > 0 && (fo == 1 || (fo < 0 && leaf_tc_fuse_pays(fa, nfa)))) {
+    // P2 joins them, into workspace, and steps 6-8 become one kernel: the same
+    // traffic as P2 accumulating onto P1 in a launch of its own, one launch fewer
+    const int64_t ldp2 = (h + 3) / 4 * 4;
+    int32_t *P2 = (int32_t *)c.ar.get((size_t)h * ldp2 * 4);
+    fa[nfa++] = tc_args(c, L.pA12, L.pA12, h, h, kap, P2, ldp2, 1, 0);
     for (int q = 0; q < nfa; ++q) count_leaf(c, fa[q].M, fa[q].N, fa[q].K, fa[q].lower);
     if (!c.ar.dry && c.err == AAT_OK)
-      check(c, launch_leaf_tc_multi(fa, nfa, c.m, c.st), "leaf (tensor cores, P1 P3 P4 P5)");
+      check(c, launch_leaf_tc_multi(fa, nfa, c.m, c.st), "leaf (tensor cores, P1 .. P5)");
+    const bool zero = c.want_zero && levels == c.zero_levels;
+    if (!c.ar.dry && c.err == AAT_OK)
+      check(c, launch_postadd_p2(C11, P2, ldp2, C12, C21, C22, ldc, h, zero, c.m, c.st), "postadd");
+    if (zero) c.zeroed = true;
+    p2_done = true;
   } else {
     // 2. P4^T = S2 S1^T -> C22
     leaf(c, L.oS2, L.oS1, false, h, h, kap, C22, ldc, 0, 0);
@@ -913,6 +925,12 @@ static void rec(Ctx &c, const int32_t *A, int64_t lda, int64_t n, int64_t k, int
     leaf(c, L.oA22, L.oS4, false, h, h, kap, C21, ldc, 0, 0);
     // 5. P1 = Low(A11 A11^T) -> C11
     if (!p1_first) rec(c, A11, lda, h, kap, C11, ldc, levels - 1, L.pA11);
+  }
+  if (p2_done) {
+    if (c.split_ev && levels == c.top_levels && !c.ar.dry && c.err == AAT_OK)
+      cudaEventRecord(c.split_ev, c.st);
+    c.ar.used = mark;
+    return;
   }
   // 6. U1 = P1 + P5, U2 = U1 + P4, U4 = U2 + P3 -> C21, U5 = Low(U2 + P4^T) -> C22
   if (!c.ar.dry) check(c, launch_postadd(C11, ldc, C12, C21, C22, ldc, h, c.m, c.st), "postadd");
@@ -1211,7 +1229,10 @@ static size_t run_plan_in(Ctx &c, const int32_t *A, int64_t n, int64_t k, int64_
   c.split_row = early ? pr.n_pad / 2 : n;
   const bool small_ok = c.small_ok;
   c.small_ok = small_ok && pr.levels == 0;
-  c.want_zero = pr.levels == 0 && (flags & AAT_ZERO_UPPER);
+  // one level clears in its post-additions, no level in the leaf (the SYRK
+  // form's level in neither)
+  c.want_zero = !pr.padded && pr.levels <= (beta ? 0 : 1) && (flags & AAT_ZERO_UPPER);
+  c.zero_levels = pr.levels;
   c.zeroed = false;
 
   if (beta)

@@ -364,6 +364,13 @@ cudaError_t launch_postadd(const int32_t *P1, int64_t ldp, int32_t *C12, int32_t
                            int32_t *C22, int64_t ldc, int64_t h, const ModP &m, cudaStream_t st,
                            const SyrkSave *sv = nullptr);
 
+// The same with U3 = P1 + P2 -> Low(C11) as the closing step (P1 in C11, P2 =
+// Low at P2 with row stride ldp2); zero: also clears everything above the
+// diagonal (C12 and the strict upper triangles of C11 and C22).
+cudaError_t launch_postadd_p2(int32_t *C11, const int32_t *P2, int64_t ldp2, int32_t *C12,
+                              int32_t *C21, int32_t *C22, int64_t ldc, int64_t h, bool zero,
+                              const ModP &m, cudaStream_t st);
+
 // Up(C11) <- Low(C22)^T strictly, dg <- diag(C22) (SYRK, Table 4).
 cudaError_t launch_save_c22(int32_t *C11, const int32_t *C22, int64_t ldc, int64_t h, int32_t *dg,
                             cudaStream_t st);

@@ -418,6 +418,74 @@ __global__ void postadd_kernel(const int32_t *__restrict__ P1, int64_t ldp,
   }
 }
 
+// The post-additions of a last level whose five products ran as one launch:
+// postadd_kernel's steps and U3 = P1 + P2 (P2 in workspace), with every load of
+// the thread's four rows issued before the barrier (a tile pair's 28 loads: at
+// h = 256, where 36 blocks run, postadd_kernel's dependent loads took 12.3 us,
+// this one 5.6 us with the addition and the clearing that took two more
+// launches, 12.3 and 2.4 us).  zero: everything above the diagonal is cleared.
+__global__ void __launch_bounds__(T * 8)
+    postadd_p2_kernel(int32_t *C11, const int32_t *__restrict__ P2, int64_t ldp2, int32_t *C12,
+                      int32_t *C21, int32_t *C22, int64_t ldc, int64_t h, int zero, ModP m) {
+  __shared__ int32_t p4t_ij[T][T + 1];  // C22 tile (I, J) = P4^T block
+  __shared__ int32_t p4t_ji[T][T + 1];  // C22 tile (J, I)
+  __shared__ int32_t u1_ij[T][T + 1];   // U1 tile (I, J)
+  const int64_t ntiles = (h + T - 1) / T;
+  int64_t I, J;
+  tri_index(blockIdx.x, I, J);
+  if (I >= ntiles) return;
+  const int tx = threadIdx.x % T, ty = threadIdx.x / T;
+  const int64_t r0 = I * T, c0 = J * T, c = c0 + tx, c2 = r0 + tx;
+  int32_t a[4], b[4], p1[4], p5[4], p2[4], x[4], y[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int64_t r = r0 + ty + 8 * q, r2 = c0 + ty + 8 * q;
+    const bool in = r < h && c < h, in2 = r2 < h && c2 < h;
+    const int64_t lr = r >= c ? r : c, lc = r >= c ? c : r;  // U1 is symmetric
+    a[q] = in ? C22[r * ldc + c] : 0;
+    p1[q] = in ? C11[lr * ldc + lc] : 0;
+    p5[q] = in ? C12[lr * ldc + lc] : 0;
+    p2[q] = in && c <= r ? P2[r * ldp2 + c] : 0;
+    x[q] = in ? C21[r * ldc + c] : 0;
+    b[q] = in2 ? C22[r2 * ldc + c2] : 0;
+    y[q] = in2 && I != J ? C21[r2 * ldc + c2] : 0;
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int yy = ty + 8 * q;
+    a[q] = bal(a[q], m);
+    p1[q] = bal(p1[q], m);
+    p4t_ij[yy][tx] = a[q];
+    p4t_ji[yy][tx] = bal(b[q], m);
+    u1_ij[yy][tx] = p5[q] = add_bal(p1[q], bal(p5[q], m), m);
+  }
+  __syncthreads();  // every read of the pair's tiles is done
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int yy = ty + 8 * q;
+    const int64_t r = r0 + yy, r2 = c0 + yy;
+    if (r < h && c < h) {
+      const int32_t u2 = add_bal(p5[q], p4t_ji[tx][yy], m);  // P4(r, c) = P4^T(c, r)
+      C21[r * ldc + c] = (int32_t)bal_to_canon(add_bal(u2, bal(x[q], m), m), m);
+      if (c <= r) {
+        C22[r * ldc + c] = (int32_t)bal_to_canon(add_bal(u2, a[q], m), m);
+        C11[r * ldc + c] = (int32_t)bal_to_canon(add_bal(p1[q], bal(p2[q], m), m), m);
+      } else if (zero) {
+        C22[r * ldc + c] = C11[r * ldc + c] = 0;
+      }
+      if (zero) C12[r * ldc + c] = 0;
+    }
+    if (I != J && r2 < h && c2 < h) {  // tile (J, I): above the diagonal
+      const int32_t u2 = add_bal(u1_ij[tx][yy], p4t_ij[tx][yy], m);
+      C21[r2 * ldc + c2] = (int32_t)bal_to_canon(add_bal(u2, bal(y[q], m), m), m);
+      if (zero) {
+        const int64_t z = r2 * ldc + c2;
+        C11[z] = C12[z] = C22[z] = 0;
+      }
+    }
+  }
+}
+
 // The SYRK schedule's first step (Table 4): Up(C11) <- Low(C22)^T on the
 // strictly triangular parts (C11[c][r] = C22[r][c], r > c) and dg[r] =
 // C22[r][r], so that C22 can receive P4^T.  One T x T tile of Low(C22) per
@@ -735,6 +803,18 @@ cudaError_t launch_postadd(const int32_t *P1, int64_t ldp, int32_t *C12, int32_t
   else
     postadd_kernel<false><<<(unsigned)pairs, T * 8, 0, st>>>(P1, ldp, C12, C21, C22, ldc, h, m,
                                                             nullptr, nullptr, 0u, 0u);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_postadd_p2(int32_t *C11, const int32_t *P2, int64_t ldp2, int32_t *C12,
+                              int32_t *C21, int32_t *C22, int64_t ldc, int64_t h, bool zero,
+                              const ModP &m, cudaStream_t st) {
+  if (h <= 0) return cudaSuccess;
+  const int64_t nt = (h + T - 1) / T;
+  const double tri = 0.5 * (double)h * (double)(h + 1), sq = (double)h * h;
+  ProfScope prof(AAT_K_POSTADD, st, 4.0 * (5.0 * tri + 3.0 * sq + (zero ? 2.0 * sq : 0.0)));
+  postadd_p2_kernel<<<(unsigned)(nt * (nt + 1) / 2), T * 8, 0, st>>>(C11, P2, ldp2, C12, C21, C22,
+                                                                    ldc, h, zero, m);
   return cudaGetLastError();
 }
 

@@ -351,3 +351,19 @@ def test_host_product_in_two_row_parts(lib, p, n, k, pinned, zero):
                 assert not C[r, r + 1:].any()
             else:
                 assert bool((C[r, (r // 512 + 1) * 512:] == -3).all())
+
+
+@pytest.mark.parametrize("zero", [False, True])
+@pytest.mark.parametrize("p", [65521, 131071, 2**31 - 1])
+@pytest.mark.parametrize("n,k,pad", [(4, 8, 0), (66, 132, 0), (130, 64, 3), (512, 512, 0), (1300, 700, 1)])
+def test_one_level_in_one_leaf_launch(lib, n, k, pad, p, zero):
+    """The last level's five products in one launch and its closing kernel:
+    tiles at their edges, cleared and kept surroundings."""
+    import torch
+    A = torch.from_numpy(synth.residues(n + k, (n, k), p, balanced=True)).cuda()
+    buf = torch.full((n, n + pad), -4, dtype=torch.int32, device="cuda")
+    lib.aat_modp(A, p, C=buf[:, :n], levels=1, flags=lib.AAT_ZERO_UPPER if zero else 0)
+    ref = torch.tril(lib.aat_gemm_modp(A, A, p))   # the plain product (other tests' subject)
+    got = buf[:, :n] if zero else torch.tril(buf[:, :n])
+    assert torch.equal(got, ref)
+    assert bool((buf[:, n:] == -4).all())
