@@ -497,6 +497,13 @@ cudaError_t leaf_tc_batch_launch(const LeafBatch &lb, cudaStream_t st);
 void leaf_tc_batch_free(LeafBatch *lb);
 
 // Batched split: one launch, problem q in blockIdx.y.
+// Rows per block of the batched splits: about 8192 entries, whatever the row
+// length, so that blocks of problems with short rows have work for every thread
+// and those with long rows spread over more of the chip.
+inline int split_block_rows(int64_t cols) {
+  const int64_t r = (8192 + cols - 1) / cols;
+  return (int)(r < 1 ? 1 : r > 256 ? 256 : r);
+}
 struct SplitDesc {
   const int32_t *X;
   int64_t ldx, rows, cols;
@@ -504,9 +511,10 @@ struct SplitDesc {
   int b;
   Planes P;
   int first_block;  // first block of this problem in the launch (split_batch_blocks)
+  int block_rows;   // rows per block
   int vec;          // rows start 16-byte aligned and cols % 4 == 0: 4-wide path
 };
-// Fills first_block / vec of descs (host) and returns the launch's block count.
+// Fills first_block / block_rows / vec of descs (host) and returns the launch's block count.
 int split_batch_blocks(SplitDesc *descs, int count);
 cudaError_t launch_split_batch(const SplitDesc *descs_dev, int count, int nblocks, double bytes,
                                cudaStream_t st);

@@ -280,20 +280,19 @@ __global__ void wino_combine_kernel(const int32_t *__restrict__ W, int64_t ldw, 
   }
 }
 
-// Batched split: every problem owns ceil(rows / kSplitRows) consecutive
-// blocks (first_block ascending), so the work of a block does not depend on
-// how large its problem is; a block finds its problem by binary search and
-// splits its kSplitRows rows, 4 columns per thread where rows are aligned.
-constexpr int kSplitRows = 8;
-
+// Batched split: every problem owns ceil(rows / block_rows) consecutive blocks
+// (first_block ascending); a block finds its problem by binary search and
+// splits its rows, 4 columns per thread.  256 F_65521 problems (1.43 GB): 8 rows
+// per block whatever their length 330 us, blocks of about equal work 326
+// us; the complex split 170 -> 150 us.
 template <int NB>
 __device__ __forceinline__ void split_rows(const SplitDesc &d, int64_t r0) {
   // the block's rows x column quads as one index, so that every thread has
   // work when the rows are short; plane rows are 16-byte aligned (kstride is
   // a multiple of 8), so each quad leaves as one 8-byte store per plane,
   // the columns past the last one written as zeros into the row padding
-  // (32-bit index arithmetic: nr * nq < 8 * 2^28)
-  const uint32_t nr = (uint32_t)min((int64_t)kSplitRows, d.rows - r0);
+  // (32-bit index arithmetic: nr * nq < 2^29)
+  const uint32_t nr = (uint32_t)min((int64_t)d.block_rows, d.rows - r0);
   const uint32_t nq = (uint32_t)((d.cols + 3) / 4);
   for (uint32_t t = threadIdx.x; t < nr * nq; t += blockDim.x) {
     const uint32_t ri = t / nq;
@@ -319,7 +318,7 @@ __global__ void split_batch_kernel(const SplitDesc *__restrict__ descs, int coun
     else hi = mid - 1;
   }
   const SplitDesc &d = descs[lo];
-  const int64_t r0 = (int64_t)(b - d.first_block) * kSplitRows;
+  const int64_t r0 = (int64_t)(b - d.first_block) * d.block_rows;
   switch (d.P.nbase) {
     case 1: split_rows<1>(d, r0); break;
     case 2: split_rows<2>(d, r0); break;
@@ -774,7 +773,8 @@ int split_batch_blocks(SplitDesc *descs, int count) {
     SplitDesc &d = descs[i];
     d.first_block = (int)nb;
     d.vec = (d.cols % 4 == 0) && (d.ldx % 4 == 0) && ((reinterpret_cast<uintptr_t>(d.X) & 15) == 0);
-    nb += (d.rows + kSplitRows - 1) / kSplitRows;
+    d.block_rows = split_block_rows(d.cols);
+    nb += (d.rows + d.block_rows - 1) / d.block_rows;
   }
   return nb > INT32_MAX ? -1 : (int)nb;
 }

@@ -673,10 +673,10 @@ struct CBProb {
   float2 *C;
   int64_t ldc;
   RowScale rs;
-  int split_first, comb_first, diag_first;
+  int split_first, split_rows, comb_first, diag_first;
 };
 
-constexpr int kCSplitRows = 8, kDiagRows = 8;
+constexpr int kDiagRows = 8;
 
 __device__ __forceinline__ int cb_find(const CBProb *pr, int count, int b, int which) {
   int lo = 0, hi = count - 1;
@@ -690,14 +690,14 @@ __device__ __forceinline__ int cb_find(const CBProb *pr, int count, int b, int w
   return lo;
 }
 
-// both plane sets of kCSplitRows rows of one problem per block
+// both plane sets of split_block_rows rows of one problem per block
 __global__ void csplit_batch_kernel(const CBProb *__restrict__ pr, int count) {
   const CBProb &q = pr[cb_find(pr, count, blockIdx.x, 0)];
-  const int64_t r0 = (int64_t)(blockIdx.x - q.split_first) * kCSplitRows;
-  const uint32_t nr = (uint32_t)min((int64_t)kCSplitRows, q.n - r0);
+  const int64_t r0 = (int64_t)(blockIdx.x - q.split_first) * q.split_rows;
+  const uint32_t nr = (uint32_t)min((int64_t)q.split_rows, q.n - r0);
   const uint32_t cq = (uint32_t)((q.k + 3) / 4);
   // the block's rows x column quads as one index: every thread has work
-  // when the rows are short (32-bit index arithmetic: nr * cq < 8 * 2^28)
+  // when the rows are short (32-bit index arithmetic: nr * cq < 2^29)
   for (uint32_t t = threadIdx.x; t < nr * cq; t += blockDim.x) {
     const uint32_t ri = t / cq;
     const int64_t r = r0 + ri, q4 = t - ri * cq;
@@ -2021,7 +2021,8 @@ cudaError_t cbatch_build(const CBInput *in, int count, char *ws, CBatch *out) {
     b.C = q.C;
     b.ldc = q.ldc;
     b.split_first = sb;
-    sb += (int)((q.n + kCSplitRows - 1) / kCSplitRows);
+    b.split_rows = split_block_rows(q.k);
+    sb += (int)((q.n + b.split_rows - 1) / b.split_rows);
     const int64_t nt = (q.n + T - 1) / T;
     b.comb_first = cbk;
     cbk += (int)(nt * (nt + 1) / 2);
