@@ -69,6 +69,45 @@ __device__ __forceinline__ void sblocks_store(const SKernelOut &o, int64_t i, in
   if (has(o.a22)) store_digits_t<NB, V>(o.a22, i, j, a22, b);
 }
 
+// Columns c .. c + 3 of a row whose start is only 4-byte aligned, by the two
+// 16-byte words that hold them, the second one from the next lane of the row
+// (four 4-byte loads per lane touch the same sectors four times over).  sh: the
+// row start's offset in words from 16-byte alignment; every lane of the warp
+// takes part, `in` says whether its quad lies in the row (the lanes that do are
+// the warp's first, with consecutive quads).  Words that are not
+// wholly inside the row are put together from single loads, so nothing outside
+// [0, cols) is read.
+__device__ __forceinline__ void ld4_shifted(const int32_t *row, int64_t c, int64_t cols, int sh,
+                                            bool in, const ModP &m, int32_t (&v)[4]) {
+  int4 w = make_int4(0, 0, 0, 0);
+  const int64_t a = c - sh;  // the aligned word that holds column c
+  auto word = [&](int64_t s) {
+    int4 x = make_int4(0, 0, 0, 0);
+    if (s >= 0 && s + 4 <= cols) {
+      x = __ldg(reinterpret_cast<const int4 *>(row + s));
+    } else {
+      if (s >= 0 && s < cols) x.x = __ldg(row + s);
+      if (s + 1 >= 0 && s + 1 < cols) x.y = __ldg(row + s + 1);
+      if (s + 2 >= 0 && s + 2 < cols) x.z = __ldg(row + s + 2);
+      if (s + 3 >= 0 && s + 3 < cols) x.w = __ldg(row + s + 3);
+    }
+    return x;
+  };
+  if (in) w = word(a);
+  int4 n;
+  n.x = __shfl_down_sync(0xffffffffu, w.x, 1);
+  n.y = __shfl_down_sync(0xffffffffu, w.y, 1);
+  n.z = __shfl_down_sync(0xffffffffu, w.z, 1);
+  n.w = 0;
+  if (in && sh && ((threadIdx.x & 31) == 31 || c + 4 >= cols)) n = word(a + 4);
+  v[0] = sh == 0 ? w.x : sh == 1 ? w.y : sh == 2 ? w.z : w.w;
+  v[1] = sh == 0 ? w.y : sh == 1 ? w.z : sh == 2 ? w.w : n.x;
+  v[2] = sh == 0 ? w.z : sh == 1 ? w.w : sh == 2 ? n.x : n.y;
+  v[3] = sh == 0 ? w.w : sh == 1 ? n.x : sh == 2 ? n.y : n.z;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v[j] = in && c + j < cols ? bal(v[j], m) : 0;
+}
+
 template <int V>
 __device__ __forceinline__ void ldv_bal(const int32_t *p, const ModP &m, int32_t (&v)[V]) {
   if constexpr (V == 4) {
@@ -166,11 +205,11 @@ __global__ void split_kernel(const int32_t *__restrict__ X, int64_t ldx, int64_t
 // The same for any rows: plane rows are 16-byte aligned whatever X's are
 // (kstride is a multiple of 8), so a quad still leaves as one 8-byte store per
 // plane, the columns past the last one as zeros into the row padding; X comes
-// in by 4-byte loads, the quad's four in the same sectors.  blockDim (bx, by):
-// bx threads sweep a row's quads, by rows per block, so no thread divides.
-// Bound by HBM.  Before (one thread per entry, 2-byte stores, a 64-bit
-// division each) 2500 x 3003 and 4001 x 3003 residues mod 2^31 - 1, 24 bytes an
-// entry, took 61 and 104 us; now 36 and 55 (5.1-5.3 TB/s).
+// in by ld4_shifted.  blockDim (bx, by): bx threads sweep a row's quads, by rows
+// per block, so no thread divides.  Bound by HBM.  2500 x 3003 and 4001 x 3003
+// residues mod 2^31 - 1, 24 bytes an entry: one thread per entry with 2-byte
+// stores and a 64-bit division 61 and 104 us; quads with four 4-byte loads 36
+// and 55; now 31 and 48 (5.8-6.0 TB/s).
 template <int NB>
 __global__ void __launch_bounds__(kThreads)
     split_ragged_kernel(const int32_t *__restrict__ X, int64_t ldx, int64_t rows, int64_t cols,
@@ -179,13 +218,15 @@ __global__ void __launch_bounds__(kThreads)
   for (int64_t r = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; r < rows;
        r += (int64_t)gridDim.y * blockDim.y) {
     const int32_t *xr = X + r * ldx;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nq;
-         q += (int64_t)gridDim.x * blockDim.x) {
-      const int64_t c = 4 * q;
+    const int sh = (int)(reinterpret_cast<uintptr_t>(xr) >> 2) & 3;
+    // blockDim.x is a multiple of 32: a warp is 32 consecutive quads of one row,
+    // and the last quads' warp goes on with its lanes past the row's end idle
+    for (int64_t q0 = (int64_t)blockIdx.x * blockDim.x; q0 < nq;
+         q0 += (int64_t)gridDim.x * blockDim.x) {
+      const int64_t q = q0 + threadIdx.x, c = 4 * q;
       int32_t v[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = c + j < cols ? ld_bal(xr + c + j, m) : 0;
-      store_digits_t<NB, 4>(P, r, c, v, b);
+      ld4_shifted(xr, c, cols, sh, q < nq, m, v);
+      if (q < nq) store_digits_t<NB, 4>(P, r, c, v, b);
     }
   }
 }
