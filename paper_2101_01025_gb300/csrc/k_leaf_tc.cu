@@ -1377,6 +1377,11 @@ LeafSplit leaf_tc_split(const TcLeafArgs &a) {
       double c = 0.0;
       const int64_t parts = model(t, s, &c);
       if (parts > MAX_MULTI || s > kblocks) break;
+      // the launch's group table holds a list per window and slice length (two
+      // lengths): a group per plane product and K segment, and the multiplier
+      const int64_t seg = std::min(kseg_blocks(), 256);
+      const int64_t groups = (int64_t)t * per * (((kblocks + s - 1) / s + seg - 1) / seg) + 1;
+      if (((planes + t - 1) / t) * (s > 1 ? 2 : 1) * groups > MAX_GROUPS) continue;
       if (parts > 1 && c < bc) {
         bc = c;
         best.window = t;

@@ -367,3 +367,40 @@ def test_one_level_in_one_leaf_launch(lib, n, k, pad, p, zero):
     got = buf[:, :n] if zero else torch.tril(buf[:, :n])
     assert torch.equal(got, ref)
     assert bool((buf[:, n:] == -4).all())
+
+
+@pytest.mark.parametrize("off", [0, 1, 2, 3])
+@pytest.mark.parametrize("cols", [1, 3, 4, 5, 125, 126, 127, 128, 129, 130, 131, 132, 509, 1029])
+def test_split_reads_only_its_rows(lib, cols, off):
+    """Every offset of a row from 16 bytes with the row's end at every offset:
+    digits of the row itself, whatever stands before and behind it."""
+    import torch
+    from paper_2101_01025_gb300 import testing as T
+    p, rows = 2**31 - 1, 7
+    X = synth.residues(cols, (rows, cols), p, balanced=True)
+    ld = cols + 1 + (cols + off) % 3        # rows at changing offsets
+    buf = torch.full((off + rows * ld + 8,), 12345, dtype=torch.int32, device="cuda")
+    view = torch.as_strided(buf, (rows, cols), (ld, 1), off)
+    view.copy_(torch.from_numpy(X))
+    b, L, _, _ = T.digit_spec(p, with_sums=True)
+    got = T.split(view, p).float().cpu().numpy().astype(np.int64)
+    assert np.array_equal(sum(got[i, :, :cols] << (b * i) for i in range(L)), X.astype(np.int64))
+    assert not got[:, :, cols:].any()
+
+
+@pytest.mark.parametrize("p", [131071, 2**31 - 1])
+@pytest.mark.parametrize("k", [66000, 120000])
+def test_split_parts_of_long_sums(lib, p, k):
+    """Parts whose K segments fill the launch's group table."""
+    import torch
+    n = 200
+    A = torch.from_numpy(synth.residues(k, (n, k), p, balanced=True)).cuda()
+    got = torch.tril(lib.aat_gemm_modp(A, A, p))
+    low = lib.aat_modp(A, p, levels=0, flags=lib.AAT_ZERO_UPPER)
+    rows = [0, 1, 127, 128, n - 1]
+    X = A.cpu().numpy()
+    ref = (X[rows].astype(object) @ X.T.astype(object)) % p
+    for i, r in enumerate(rows):
+        want = ref[i, :r + 1].astype(np.int64)
+        assert np.array_equal(got[r, :r + 1].cpu().numpy().astype(np.int64), want)
+        assert np.array_equal(low[r, :r + 1].cpu().numpy().astype(np.int64), want)
