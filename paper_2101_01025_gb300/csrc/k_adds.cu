@@ -997,40 +997,48 @@ __global__ void quat_combine_kernel(const int32_t *__restrict__ Q, int64_t ldq, 
                                     int64_t ldh, int64_t n, int zero, ModP m) {
   __shared__ int32_t qt[5][T][T + 1];  // tile (J, I) of Q1..Q5
   const int64_t ntiles = (n + T - 1) / T;
-  int64_t pid = blockIdx.x;
-  int64_t I = (int64_t)((sqrt(8.0 * (double)pid + 1.0) - 1.0) * 0.5);
-  while (I * (I + 1) / 2 > pid) --I;
-  while ((I + 1) * (I + 2) / 2 <= pid) ++I;
-  const int64_t J = pid - I * (I + 1) / 2;
+  int64_t I, J;
+  tri_index(blockIdx.x, I, J);
   if (I >= ntiles) return;
   const int tx = threadIdx.x % T, ty = threadIdx.x / T;
-  const int64_t r0 = I * T, c0 = J * T;
-  for (int yy = ty; yy < T; yy += 8) {
-    const int64_t r2 = c0 + yy, c2 = r0 + tx;
-    if (r2 < n && c2 < n) {
+  const int64_t r0 = I * T, c0 = J * T, c = c0 + tx, c2 = r0 + tx;
+  // the four rows' loads before the barrier (n = 2048: 35 -> 29 us)
+  int32_t q[4][5], h[4];
 #pragma unroll
-      for (int q = 0; q < 5; ++q) qt[q][yy][tx] = bal(Q[q * qstride + r2 * ldq + c2], m);
-      if (zero && r2 < c2) {
-        const int64_t z = r2 * ldh + c2;
-        H1[z] = H2[z] = H3[z] = H4[z] = 0;
-      }
-    }
-  }
-  __syncthreads();
-  for (int yy = ty; yy < T; yy += 8) {
-    const int64_t r = r0 + yy, c = c0 + tx;
-    if (r >= n || c >= n || c > r) continue;
-    int32_t q[5], qT[5];
+  for (int y = 0; y < 4; ++y) {
+    const int64_t r = r0 + ty + 8 * y, r2 = c0 + ty + 8 * y;
+    const bool in = r < n && c <= r, in2 = r2 < n && c2 < n;
+    int32_t t[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-      q[i] = bal(Q[i * qstride + r * ldq + c], m);
+      t[i] = in2 ? Q[i * qstride + r2 * ldq + c2] : 0;
+      q[y][i] = in ? Q[i * qstride + r * ldq + c] : 0;
+    }
+    h[y] = in ? H1[r * ldh + c] : 0;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) qt[i][ty + 8 * y][tx] = bal(t[i], m);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int y = 0; y < 4; ++y) {
+    const int yy = ty + 8 * y;
+    const int64_t r = r0 + yy, r2 = c0 + yy;
+    if (zero && r2 < n && c2 < n && r2 < c2) {
+      const int64_t z = r2 * ldh + c2;
+      H1[z] = H2[z] = H3[z] = H4[z] = 0;
+    }
+    if (r >= n || c > r) continue;
+    int32_t qT[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      q[y][i] = bal(q[y][i], m);
       qT[i] = qt[i][tx][yy];  // Q_i(c, r)
     }
-    const int32_t t1 = sub_bal(q[0], q[1], m), t1T = sub_bal(qT[0], qT[1], m);
-    const int32_t t2 = add_bal(q[3], q[4], m), t2T = add_bal(qT[3], qT[4], m);
-    const int32_t t3 = sub_bal(add_bal(q[0], q[1], m), q[2], m);
+    const int32_t t1 = sub_bal(q[y][0], q[y][1], m), t1T = sub_bal(qT[0], qT[1], m);
+    const int32_t t2 = add_bal(q[y][3], q[y][4], m), t2T = add_bal(qT[3], qT[4], m);
+    const int32_t t3 = sub_bal(add_bal(q[y][0], q[y][1], m), q[y][2], m);
     const int32_t t3T = sub_bal(add_bal(qT[0], qT[1], m), qT[2], m);
-    int32_t h1 = sub_bal(bal(H1[r * ldh + c], m), add_bal(qT[2], q[2], m), m);
+    int32_t h1 = sub_bal(bal(h[y], m), add_bal(qT[2], q[y][2], m), m);
     h1 = sub_bal(h1, add_bal(t2T, t2, m), m);
     H1[r * ldh + c] = (int32_t)bal_to_canon(h1, m);
     H2[r * ldh + c] = (int32_t)bal_to_canon(sub_bal(t2T, t2, m), m);
