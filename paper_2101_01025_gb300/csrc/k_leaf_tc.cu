@@ -126,6 +126,9 @@ struct Params {
   const Group *gtab;
   // multi-problem launches: tile entries (problem, I, J, 0)
   const int4 *mtiles;
+  // pacing of the pairs (null: none): pace[s] counts the pairs that have begun
+  // their s-th group
+  uint32_t *pace;
   MultiProb mp[MAX_MULTI];
 };
 
@@ -303,6 +306,16 @@ struct Shape {
                                     ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
 };
 
+// Pacing: the pairs of a wave share their panels in L2 only while they are at the
+// same plane product and K position, and nothing but their equal speed keeps
+// them there.  At the start of each group a pair's producer counts itself and
+// waits for the others of its wave, at most kPaceNs: a hint, not a barrier, so
+// pairs that never run together only lose that time.  8192^3 mod 2^31 - 1: DRAM
+// reads 17-23 -> 11.4 GB, 5.9-6.25 -> 5.73 ms; 16384 x 16384 26.0-26.5 ->
+// 24.8 ms a pass under the power cap (limits of 3 and 10 us alike).
+constexpr uint32_t kPaceMax = 4096;
+constexpr unsigned long long kPaceNs = 5000;
+
 // Epilogue warps of the single-problem launches and of the batched launch
 // (whose tiles are mostly short in K, so the per-tile epilogue dominates).
 constexpr int kEwLeaf = 8, kEwBatch = 16;
@@ -385,29 +398,44 @@ __global__ void __launch_bounds__(Shape<PAIR, EW, TN>::THREADS, 1)
     // divergent lane needed ~500 cycles per K block (its operands moved to the
     // uniform datapath one by one), which bounded the narrow form: 1001 x 1001
     // x 3001 mod 2^31 - 1 went 127 -> 69 us, 2500 x 4001 x 3003 (pairs) 20 us
-    // less of 490
-    {
+    // less of 490.  kDiv: the 256 x 256 pair form keeps the divergent lane; it
+    // is fast enough there, and the uniform loop's pairs drift apart more
+    // (21-23 against 17-19 GB of DRAM reads per 8192^3 product unpaced; 16384 x
+    // 16384 26.5 against 26.0 ms).
+    constexpr bool kDiv = PAIR && TN == BN;
+    if (!kDiv || lane == 0) {
       int stage = 0;
       uint32_t ph = 0;
       int issued = 0;
       bool ok = true;
       // both CTAs' copies of a stage complete on the leader's FULL barrier
       const uint32_t full0 = PAIR ? map_to_rank(FULL(0), 0) : FULL(0);
+      uint32_t seq = 0;
       for (int t = (int)unit0; t < P.ntiles && ok; t += (int)nunits) {
         const TileView v = tile_view<MODE>(P, t);
         const int rowx = v.I * S::TM + (int)rank * BM;
         const int rowy = v.J * TN + (int)rank * S::YROWS;
         for (int gi = 0; gi < v.ng && ok; ++gi) {
           const Group g = v.g[gi];
+          if constexpr (kDiv && MODE != kBatch) {
+            if (P.pace && leader && seq < kPaceMax) {
+              const uint32_t all = (uint32_t)min((int)nunits, P.ntiles - (t - (int)unit0));
+              atomicAdd(P.pace + seq, 1u);
+              const unsigned long long t0 = gtimer();
+              while (*(volatile uint32_t *)(P.pace + seq) < all && gtimer() - t0 < kPaceNs) {
+              }
+            }
+            ++seq;
+          }
           for (int kb = g.kb0; kb < g.kb1; ++kb) {
-            if (!__all_sync(0xffffffffu, wait_bounded<PAIR>(EMPTY(stage), ph ^ 1u, abort_flag,
-                                                            P.status))) {
+            const bool got = wait_bounded<PAIR>(EMPTY(stage), ph ^ 1u, abort_flag, P.status);
+            if (kDiv ? !got : !__all_sync(0xffffffffu, got)) {
               ok = false;
               break;
             }
             const uint32_t sa = sbase + (uint32_t)(stage * S::STAGE_BYTES);
             const uint32_t fb = full0 + 8u * (uint32_t)stage;
-            if (elect_one()) {
+            if (kDiv || elect_one()) {
               if constexpr (PAIR) {
                 if (leader) mbar_expect_tx(FULL(stage), (uint32_t)(2 * S::STAGE_BYTES));
                 tma_load_3d_pair(sa, v.tmx, fb, kb * BK, rowx, g.xp);
@@ -418,7 +446,7 @@ __global__ void __launch_bounds__(Shape<PAIR, EW, TN>::THREADS, 1)
                 tma_load_3d(sa + S::A_BYTES, v.tmy, fb, kb * BK, rowy, g.yp);
               }
             }
-            __syncwarp();
+            if (!kDiv) __syncwarp();
             ++issued;
             if (++stage == STAGES) {
               stage = 0;
@@ -1090,6 +1118,9 @@ int pair_override() {
   return v;
 }
 
+// The pacing counters of the current device, cleared on `st`, for a launch whose
+// groups are long enough to drift apart in; null (no pacing) otherwise.
+std::map<int, uint32_t *> g_pace;
 // Shared-memory limits of the single-product kernel's forms (pair_units sets the
 // whole pair form's), set
 // together whichever entry point launches first (g_mu held).
@@ -1129,6 +1160,21 @@ enum Form { kCta = 1, kPair = 2, kNarrow = 3, kPairHalf = 4 };
 bool is_pair(Form f) { return f == kPair || f == kPairHalf; }
 int form_tm(Form f) { return is_pair(f) ? 256 : 128; }
 int form_tn(Form f) { return f == kNarrow ? kTnNarrow : f == kPairHalf ? kTnHalf : BN; }
+uint32_t *pace_for(int dev, Form f, int64_t K, int ntiles, int units, int ngroups,
+                   cudaStream_t st) {
+  if (f != kPair || K < 2048 || ntiles < 2 * units) return nullptr;
+  uint32_t *&p = g_pace[dev];
+  if (!p && cudaMalloc(&p, kPaceMax * sizeof(uint32_t)) != cudaSuccess) {
+    cudaGetLastError();
+    p = nullptr;
+  }
+  const int64_t n = std::min<int64_t>(kPaceMax, (int64_t)((ntiles + units - 1) / units) * ngroups);
+  if (!p || cudaMemsetAsync(p, 0, (size_t)n * 4, st) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return p;
+}
 // rows of Y per CTA and stage
 int form_yrows(Form f) { return is_pair(f) ? form_tn(f) / 2 : form_tn(f); }
 
@@ -1260,6 +1306,7 @@ cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) 
   }
   P->tiles = tiles;
   P->ntiles = nt;
+  P->pace = pace_for(dev, form, a.K, nt, units, ng, st);
   if ((e = set_single_attrs(dev)) != cudaSuccess) { delete P; return e; }
   if (nt > 0) {
     // algorithmic tensor work: one BF16 product of the ring MACs per plane
@@ -1688,6 +1735,9 @@ void leaf_tc_release() {
   for (auto &kv : g_mtiles)
     if (kv.second.first) cudaFree(kv.second.first);
   g_mtiles.clear();
+  for (auto &kv : g_pace)
+    if (kv.second) cudaFree(kv.second);
+  g_pace.clear();
   g_attr_set.clear();
   g_pair_units.clear();
 }
