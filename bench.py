@@ -47,8 +47,8 @@ P = 2**31 - 1
 SEED_OFFSET = 2
 # DRAM traffic of the dominant kernel from one ncu capture of three 8192^3
 # leaf products mod 2^31-1 (dram__bytes_read.sum + dram__bytes_write.sum:
-# 11.63, 11.63 and 11.63 GB for 10.995 TFLOP of algorithmic work each;
-# CTA-pair form, tiles in bands of 2048 rows), scaled to the average launch
+# 11.63, 11.63 and 11.63 GB for 10.995 TFLOP of algorithmic work each (11.37
+# GB read and 0.26 GB written); CTA-pair form, paced, tiles in bands of 2048 rows), scaled to the average launch
 # of the step by its algorithmic work.  None whenever the kernel has changed
 # since the counters were taken.
 LEAF_TC_BYTES_PER_FLOP = 11.63e9 / 10.995e12
@@ -323,7 +323,7 @@ def run_configs(peaks):
     Z = torch.view_as_complex(torch.randn((8192, 8192, 2), device="cuda", generator=gen))
     CZ = torch.empty((8192, 8192), dtype=torch.complex64, device="cuda")
     measure("complex8192_aah_2m_fp32", lambda: aat.aah_complex(Z, C=CZ), 8192.0**3, 5,
-            "Low(A A^H) by 2M, FP32-accurate (3 BF16 pieces)", "leaf_f32")
+            "Low(A A^H) by 2M, FP32-accurate (2 FP16 pieces, 3 piece products)", "leaf_f32")
     measure("complex8192_aat_alg1_fp32", lambda: aat.aat_complex(Z, C=CZ), 8192.0**3, 5,
             "Low(A A^T) by Algorithm 1 (Y = i I, default depth), FP32-accurate", "leaf_f32")
     del Z, CZ
@@ -343,13 +343,13 @@ def run_configs(peaks):
           for n, k in zip(cn, ck)]
     # algorithmic tensor FLOPs: mod 65521 three plane products (two digit
     # planes, one pair sum) of the lower triangle; complex A A^H (FP32 class)
-    # six piece products of H (all n^2 entries) and of G (lower triangle)
+    # three FP16 piece products of H (all n^2 entries) and of G (lower triangle)
     def flops(probs):
         f = 0.0
         for kind, Ap, _, _, _ in probs:
             n, k = float(Ap.shape[0]), float(Ap.shape[1])
             low = n * (n + 1) / 2 * k
-            f += 2 * 3 * low if kind == "modp" else 2 * 6 * (n * n * k + low)
+            f += 2 * 3 * low if kind == "modp" else 2 * 3 * (n * n * k + low)
         return f
     for name, probs, cls in (("batch256_p65521", fp, "leaf_tc"), ("batch64_complex_aah", cx,
                                                                    "leaf_f32"),

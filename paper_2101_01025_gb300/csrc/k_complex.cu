@@ -1254,7 +1254,8 @@ static cudaError_t fused_table(const std::vector<FusedJob> &jobs, int np, int64_
       g.neg = 0;
     }
     const double macs = j.lower ? 0.5 * (double)j.M * (double)(j.M + 1) * K : (double)j.M * j.N * K;
-    work += 2.0 * npairs * macs;
+    // the FP16 form's three piece products (the flag is set on the device)
+    work += 2.0 * (wide ? kHalfTerms : npairs) * macs;
   }
   T->njobs = nj;
   // the tile list, cached per shape list
@@ -2074,7 +2075,7 @@ cudaError_t cbatch_build(const CBInput *in, int count, char *ws, CBatch *out) {
           tiles.push_back({make_int4(jobi, (int)I, (int)J, 0), cost});
         }
       const double macs = jb == 1 ? 0.5 * (double)q.n * (q.n + 1) * q.k : (double)q.n * q.n * q.k;
-      L->leaf_work += 2.0 * npairs * macs;
+      L->leaf_work += 2.0 * (b.rs.wide ? kHalfTerms : npairs) * macs;
     }
   }
   std::stable_sort(tiles.begin(), tiles.end(),
