@@ -148,9 +148,12 @@ AAT_API int aah_quat_modp(const int32_t *A, const int32_t *B, const int32_t *C, 
  * copied back in bands of 512 rows, band [a, b) carrying columns [0, b).
  * When a recursion level runs, A's top-left block A11 is copied first and
  * the product P1 = Low(A11 A11^T) runs while the rest of A arrives, and the
- * rows below n/2 of C go back while the last product still computes.  With
- * AAT_ZERO_UPPER, A is copied whole first and the whole of C (upper
- * triangle zero) after the computation.
+ * rows below n/2 of C go back while the last product still computes.
+ * Without recursion levels a large product runs in two row parts, the rest
+ * of A arriving and the first rows of C going back beside the launches.  With
+ * AAT_ZERO_UPPER the whole of C (upper triangle zero) is copied back; with
+ * it and recursion levels, A is copied whole first and C after the
+ * computation.
  */
 AAT_API int aat_modp_host(const int32_t *A_host, int64_t n, int64_t k, uint32_t p,
                   int32_t *C_host, uint32_t flags);
@@ -243,10 +246,10 @@ AAT_API int aat_gemm_modp_noalloc(const int32_t *X, int64_t ldx, const int32_t *
 /* ------------------------------------------------------------------ C
  * Complex inputs and outputs are complex64, interleaved (re, im) floats,
  * row-major with strides in complex elements.  No product runs in FP32
- * arithmetic: every real product runs on the BF16 tensor cores with the FP32
- * values split into BF16 pieces (x = x0 + x1 + x2, x0 = bf16(x),
- * x1 = bf16(x - x0), ...), piece products of weight >= 2^-16 kept, FP32
- * accumulation.  The precision flags name the accuracy class:
+ * arithmetic: every real product runs on the 16-bit tensor cores with the
+ * FP32 values split into BF16 pieces (x = x0 + x1 + x2, x0 = bf16(x),
+ * x1 = bf16(x - x0), ...; piece products of weight >= 2^-16 kept) or into two
+ * FP16 pieces, FP32 accumulation.  The precision flags name the accuracy class:
  *   AAT_C_FP32    FP32-accurate (relative Frobenius error <= 1e-5): 2M on
  *                 FP16 pieces of power-of-two scaled rows, 2 pieces and 3
  *                 piece products per real product; on 3 BF16 pieces and 6
