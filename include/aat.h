@@ -253,8 +253,12 @@ AAT_API int aat_gemm_modp_noalloc(const int32_t *X, int64_t ldx, const int32_t *
  *   AAT_C_FP32    FP32-accurate (relative Frobenius error <= 1e-5): 2M on
  *                 FP16 pieces of power-of-two scaled rows, 2 pieces and 3
  *                 piece products per real product; on 3 BF16 pieces and 6
- *                 piece products where a row's values spread too far for
- *                 FP16 (decided on the device) and in Algorithm 1's levels
+ *                 piece products where a row has two values more than 2^28
+ *                 or one more than 2^33 below its largest, an Inf, a NaN or
+ *                 a largest value outside 2^-103 .. 2^103 (decided on the
+ *                 device), and in Algorithm 1's levels.  Either way a value
+ *                 enters with an error of at most 2^-22 of itself (2^-17 when
+ *                 it is the only one of its row below that 2^28)
  *   AAT_C_BF16X3  2 pieces, 3 piece products (<= 1e-4)
  *   AAT_C_BF16    plain BF16 (<= 3e-3): one piece per input value; the 2M
  *                 form's sum operand (Ar + Ai or Ar - Ai) keeps 2 pieces (3

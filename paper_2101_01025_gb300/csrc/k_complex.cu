@@ -25,12 +25,20 @@
 // x1y1 is below 2^-22 of the product) replace six, at the same tensor rate.
 // FP16's exponent range is the price: every row is scaled by a power of two
 // that brings its largest value into [2^13, 2^14) (row_stats_kernel; undone
-// exactly in the combine), and a value keeps full precision down to 2^-16 of
-// its row's largest.  The choice is made on the device, per product: when a
-// row's values lie on average (of their exponents) more than 2^8 below its
-// largest, or the row holds an Inf, a NaN or values near the ends of FP32's
-// range, the whole product runs on the six BF16 products instead
-// (`wide` != 0).  Relative Frobenius error against 64 bits at n = k = 8192,
+// exactly in the combine), and the second piece is stored times 2^12 (undone
+// in the leaf's registers between the small products and x0y0), so that it
+// does not leave FP16's range before the first one does: a value keeps 22 bits
+// down to 2^-28 of its row's largest, and an error of 2^-50 of the largest
+// below that.  The choice is made on the device, per product, by what
+// that cannot hold: when a row has two values more than 2^28 or one more than
+// 2^33 below its largest, or when it holds an Inf, a NaN or values near the
+// ends of FP32's range, the whole product runs on the six BF16 products instead
+// (`wide` != 0).  An entry made only of a row's small values (the other row
+// zero elsewhere) then keeps FP32's accuracy; with the second piece unscaled
+// and a limit of 2^8 on the average spread of a row, 15 % of the values 2^-26 below the rest came out 3.7e-4
+// wrong and 5 % at 2^-60 were lost.  N(0, 1) rows of 32768 values have a value
+// 2^-28 below the largest in one row of 2500, one at 2^-33 in one of 80000.
+// Relative Frobenius error against 64 bits at n = k = 8192,
 // N(0, 1): A A^H 1.8e-7 (3.4e-7 by the six BF16 products), A A^T by 2M 3.1e-7
 // (5.9e-7); 6.1 -> 3.5 ms, of it the leaf 5.4 -> 2.9 ms.
 #include <cuda.h>
@@ -112,14 +120,19 @@ struct FJob {
   // of one TMEM accumulation that starts at block q0
   __device__ __forceinline__ int total() const { return ng * kblocks; }
   __device__ __forceinline__ int chunk_end(int q0, int kchunk) const;
-  __device__ __forceinline__ int chunks(int kchunk) const;
+  // chunks of the sum, numbered from `first` up to (not including) the result:
+  // FP16 pieces' x0y0 begins with chunk 0, BF16 pieces have no chunk 0
+  __device__ __forceinline__ int chunks(int kchunk, int *first) const;
   // group gi of the sum
   __device__ __forceinline__ const FGroup &group(int gi) const;
 };
 
 // FP16 pieces: x0y1 and x1y0 come first and x0y0, whose sums are 2^11 times
 // larger, last, so that the FP32 register that collects the chunks rounds at
-// full size only while x0y0 is added.  The tensor core truncates what falls
+// full size only while x0y0 is added.  Before that it is multiplied by
+// 1 / kHalfUp, the power of two that second pieces are stored with: their
+// residues are at most 2^3 (|x| < 2^15), so 2^12 is the largest that keeps
+// them below FP16's end.  The tensor core truncates what falls
 // below an accumulator's last bit (x0y0 has 22 bits, where a BF16 product's
 // 16 bits fit), which short chunks keep small; the small terms take long ones.
 // Measured at n = k = 8192 (A A^H, every entry), x0y0 in chunks of 4 / 3 / 2 /
@@ -127,16 +140,16 @@ struct FJob {
 // uniform in [0, 1) 10 / 7.8 / 4.4 / 3.6e-7 (BF16: 4.4e-7), 3.44 / 3.49 / 3.54 /
 // 3.73 ms.
 constexpr int kHalfTerms = 3, kHalfSmall = 16, kHalfBig = 2;
+constexpr float kHalfUp = 4096.0f;
 
 __device__ __forceinline__ int FJob::chunk_end(int q0, int kchunk) const {
   if (!half) return min(q0 + kchunk, total());
   const int small = (kHalfTerms - 1) * kblocks;
   return q0 < small ? min(q0 + kHalfSmall, small) : min(q0 + kHalfBig, total());
 }
-__device__ __forceinline__ int FJob::chunks(int kchunk) const {
-  if (!half) return (total() + kchunk - 1) / kchunk;
-  const int small = (kHalfTerms - 1) * kblocks;
-  return (small + kHalfSmall - 1) / kHalfSmall + (total() - small + kHalfBig - 1) / kHalfBig;
+__device__ __forceinline__ int FJob::chunks(int kchunk, int *first) const {
+  *first = half ? -(((kHalfTerms - 1) * kblocks + kHalfSmall - 1) / kHalfSmall) : 1;
+  return half ? (kblocks + kHalfBig - 1) / kHalfBig : (total() + kchunk - 1) / kchunk + 1;
 }
 __device__ __forceinline__ const FGroup &FJob::group(int gi) const {
   return g[half ? (gi == kHalfTerms - 1 ? 0 : gi + 1) : gi];
@@ -424,12 +437,17 @@ __global__ void __launch_bounds__(THREADS, 1) leaf_f32_kernel(const __grid_const
     bool ok = true;
     for (int t = (int)unit0; t < P.ntiles && ok; t += (int)nunits) {
       const FJob jb = fjob<BATCH>(P, t);
-      const int nchunks = jb.chunks(P.kchunk);
+      int c;
+      const int cend = jb.chunks(P.kchunk, &c);
       float acc[VALS];
 #pragma unroll
       for (int i = 0; i < VALS; ++i) acc[i] = 0.0f;
-      for (int c = 0; c < nchunks; ++c) {
+      for (; c < cend; ++c) {
         const uint32_t buf = chunk & 1u, use = chunk >> 1;
+        if (c == 0) {
+#pragma unroll
+          for (int i = 0; i < VALS; ++i) acc[i] *= 1.0f / kHalfUp;
+        }
         if (!wait_bounded<PAIR>(AFULL(buf), use & 1u, abort_flag, P.status)) {
           ok = false;
           break;
@@ -551,7 +569,8 @@ __device__ __forceinline__ void cload4(const float2 *__restrict__ a_row, int64_t
 // The pieces of 4 consecutive values a[0..nv) of row r, columns c0.., into
 // every plane set of o: one 8-byte store per plane (kstride is a multiple of
 // 8); a ragged last quad stores element by element.
-// sc != 0: two FP16 pieces of the values times sc (a power of two).
+// sc != 0: two FP16 pieces of the values times sc (a power of two), the second
+// one times kHalfUp.
 __device__ __forceinline__ void csplit_store(const float2 (&a)[4], int64_t r, int64_t c0, int nv,
                                              int np, const CSplitOut &o, float sc = 0.0f) {
   const Planes *outs[4] = {&o.re, &o.im, &o.s, &o.d};
@@ -577,10 +596,10 @@ __device__ __forceinline__ void csplit_store(const float2 (&a)[4], int64_t r, in
         pc[q].x = *reinterpret_cast<uint32_t *>(&lo);
         pc[q].y = *reinterpret_cast<uint32_t *>(&hi);
         const float2 fl = __half22float2(lo), fh = __half22float2(hi);
-        x[0] -= fl.x;
-        x[1] -= fl.y;
-        x[2] -= fh.x;
-        x[3] -= fh.y;
+        x[0] = (x[0] - fl.x) * kHalfUp;
+        x[1] = (x[1] - fl.y) * kHalfUp;
+        x[2] = (x[2] - fh.x) * kHalfUp;
+        x[3] = (x[3] - fh.y) * kHalfUp;
       }
     } else {
 #pragma unroll
@@ -795,10 +814,10 @@ __device__ __forceinline__ void sq_acc(float x, float &hi, float &lo) {
 // (about 48 significant bits: the only rounding is in the low words, whose
 // terms are each below an ulp of the high ones; one pair each for the real
 // and imaginary parts so the two dependency chains overlap), the largest
-// magnitude's bits, and the biased exponents' sum over the nonzero values.
+// and the smallest nonzero magnitude's bits (the latter less one).
 struct RowAcc {
   float h0, l0, h1, l1;
-  uint32_t mx, esum, nz;
+  uint32_t mx, mn;
 };
 
 template <bool DIAG, bool SCALE>
@@ -810,23 +829,39 @@ __device__ __forceinline__ void row_acc(float2 v, RowAcc &a) {
   if constexpr (SCALE) {
     const uint32_t x = __float_as_uint(v.x) & 0x7fffffffu, y = __float_as_uint(v.y) & 0x7fffffffu;
     a.mx = max(a.mx, max(x, y));
-    a.esum += (x >> 23) + (y >> 23);  // a lane sees fewer than 2^23 values
-    a.nz += (x != 0u) + (y != 0u);
+    a.mn = min(a.mn, min(x - 1u, y - 1u));  // zeros wrap around to the largest
   }
+}
+
+// What the FP16 pieces cannot hold of a row: values this many powers of two
+// below the row's largest, more than one and any.
+constexpr int kHalfDeep = 28, kHalfDeepest = 33;
+
+// Nonzero values of a row with a biased exponent below `floor` (by the whole
+// warp; only rows whose smallest value lies there come here).
+__device__ __forceinline__ uint32_t count_below(const float2 *__restrict__ a_row, int64_t k,
+                                                uint32_t floor) {
+  uint32_t c = 0;
+  for (int64_t l = threadIdx.x & 31; l < k; l += 32) {
+    const float2 v = a_row[l];
+    const uint32_t x = __float_as_uint(v.x) & 0x7fffffffu, y = __float_as_uint(v.y) & 0x7fffffffu;
+    c += (x != 0u && (x >> 23) < floor) + (y != 0u && (y >> 23) < floor);
+  }
+  return __reduce_add_sync(0xffffffffu, c);
 }
 
 // One warp per row.  DIAG: Σ_l |a_l|², the lanes' pairs added in FP64 (this
 // part's FP64 pipe is a small fraction of its FP32 pipe: an FP64 multiply-add
 // per square held the kernel far below the memory rate).  SCALE: the row's
 // scale exponent, and the product's `wide` flag when the row needs BF16's
-// exponent range.  The diagonal goes to rs.diag.
+// exponent range.  The diagonal goes to rs.diag.  Bound by HBM.
 template <bool DIAG, bool SCALE>
 __device__ __forceinline__ void row_stats(const float2 *__restrict__ A, int64_t lda, int64_t n,
                                           int64_t k, const RowScale &rs, int64_t row) {
   const int lane = threadIdx.x & 31;
   if (row >= n) return;
   const float2 *a_row = A + row * lda;
-  RowAcc a = {0.f, 0.f, 0.f, 0.f, 0u, 0u, 0u};
+  RowAcc a = {0.f, 0.f, 0.f, 0.f, 0u, 0xffffffffu};
   int64_t l = 0;
   if ((reinterpret_cast<uintptr_t>(a_row) & 15) == 0) {
     // two complex values per lane per 16-byte load, four loads in flight
@@ -858,18 +893,14 @@ __device__ __forceinline__ void row_stats(const float2 *__restrict__ A, int64_t 
   }
   if constexpr (SCALE) {
     const uint32_t mx = __reduce_max_sync(0xffffffffu, a.mx);
-    unsigned long long es = a.esum, nz = a.nz;
-    for (int off = 16; off; off >>= 1) {
-      es += __shfl_down_sync(0xffffffffu, es, off);
-      nz += __shfl_down_sync(0xffffffffu, nz, off);
-    }
+    const int E = (int)(mx >> 23);
+    const int low = mx ? (int)((__reduce_min_sync(0xffffffffu, a.mn) + 1u) >> 23) : 0;
+    // a subnormal (exponent 0) counts as below either line
+    bool deep = mx && low < max(E - kHalfDeepest, 1);
+    if (mx && !deep && low < E - kHalfDeep) deep = count_below(a_row, k, E - kHalfDeep) > 1;
     if (lane == 0) {
-      const int E = (int)(mx >> 23);
-      const bool zero = mx == 0u;
-      // average exponent of the nonzero values against the largest one's
-      const bool spread = (unsigned long long)E * nz > es + 8ull * nz;
-      if (!zero && (E < 24 || E > 230 || spread)) atomicOr(rs.wide, 1);
-      rs.e[row] = zero ? 0 : min(max(E - 127 - 13, -120), 120);
+      if (mx && (E < 24 || E > 230 || deep)) atomicOr(rs.wide, 1);
+      rs.e[row] = mx ? min(max(E - 127 - 13, -120), 120) : 0;
     }
   }
 }

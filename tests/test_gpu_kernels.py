@@ -404,3 +404,37 @@ def test_split_parts_of_long_sums(lib, p, k):
         want = ref[i, :r + 1].astype(np.int64)
         assert np.array_equal(got[r, :r + 1].cpu().numpy().astype(np.int64), want)
         assert np.array_equal(low[r, :r + 1].cpu().numpy().astype(np.int64), want)
+
+
+# Each of G, H and H^T carries at most 8 2^-23 of its sum of magnitudes (the
+# derivation above), and those are at most 2, 1 and 1 times sum |a_l| |b_l|:
+# 4e-6.  A value alone in its row between 2^-28 and 2^-33 of the row's largest
+# has 2^-17 of itself as FP16 pieces, in the same four sums.
+@pytest.mark.parametrize("columns,depth", [(60, 13), (60, 26), (40, 34), (20, 60), (200, 27), (300, 28),
+                                           (8, 29), (2, 33), (1, 28), (1, 33), (1, 34), (1, 60)])
+def test_complex_fp32_class_entries_of_small_values_only(lib, columns, depth):
+    """Rows with `columns` values 2^-depth of the rest (one real value where it
+    is 1) against rows that are zero elsewhere: entries made of these alone."""
+    import torch
+    n, k, h = 96, 400, 48
+    rng = np.random.default_rng(100 * columns + depth)
+    part = [rng.uniform(1, 2, (n, k)) * rng.choice([-1, 1], (n, k)) for _ in range(2)]
+    A = part[0] + 1j * part[1]
+    A[:h, :columns] *= 2.0 ** -depth
+    A[h:, columns:] = 0
+    if columns == 1:
+        A[:h, 0] = A[:h, 0].real
+    A = np.ascontiguousarray(A[:, rng.permutation(k)].astype(np.complex64))
+    Z = A.astype(np.complex128)
+    tol = 4e-6 + (4 * 2.0 ** -17 if columns == 1 and 28 < depth <= 33 else 0)
+    Ad = torch.from_numpy(A).cuda()
+    Cp = torch.zeros((n, n), dtype=torch.complex64, device="cuda")
+    plan = lib.Plan([("aah", Ad, Cp, 0, lib.AAT_C_FP32)])
+    plan.execute()
+    for got, conj in ((lib.aah_complex(Ad), True), (lib.aat_complex(Ad), False),
+                      (lib.aat_complex_2m(Ad), False), (Cp, True)):
+        ref = (Z @ (Z.conj() if conj else Z).T)[h:, :h]
+        mag = (np.abs(Z) @ np.abs(Z).T)[h:, :h]
+        err = np.abs(got.cpu().numpy().astype(np.complex128)[h:, :h] - ref) / mag
+        assert err.max() <= tol
+    plan.close()
