@@ -567,6 +567,15 @@ static TcLeafArgs tc_args(const Ctx &c, const Planes &x, const Planes &y, int64_
   return a;
 }
 
+// Whether a part of a product (a window of its planes, a slice of K) has plane
+// products that do not vanish mod p.  A part whose group list cannot be built is
+// an error, as it is for a whole product, not an empty part.
+static bool live_part(Ctx &c, const TcLeafArgs &a) {
+  const int terms = leaf_tc_terms(a, c.m);
+  return check(c, terms < 0 ? cudaErrorInvalidValue : cudaSuccess, "leaf (tensor cores, groups)") &&
+         terms > 0;
+}
+
 static void leaf(Ctx &c, Operand X, Operand Y, bool same, int64_t M, int64_t N, int64_t K,
                  int32_t *out, int64_t ldo, int lower, uint32_t beta) {
   const Lin lin = lin_of(c.alpha, beta, c.m.p);
@@ -617,7 +626,7 @@ static void leaf(Ctx &c, Operand X, Operand Y, bool same, int64_t M, int64_t N, 
       Planes px = planes_window(c, M, K, q0, w), py = px;
       if (!same) py = planes_window(c, N, K, q0, w);
       const TcLeafArgs a = tc_args(c, px, py, M, N, K, out, ldo, lower, first ? beta : 1);
-      if (!c.ar.dry && c.err == AAT_OK && leaf_tc_terms(a, c.m) > 0) {
+      if (!c.ar.dry && c.err == AAT_OK && live_part(c, a)) {
         check(c, launch_split(X.x, X.ld, M, K, c.m, c.ds.b, px, c.st), "split");
         if (!same) check(c, launch_split(Y.x, Y.ld, N, K, c.m, c.ds.b, py, c.st), "split");
         check(c, launch_leaf_tc(a, c.m, c.st), "leaf (tensor cores, plane pass)");
@@ -625,7 +634,7 @@ static void leaf(Ctx &c, Operand X, Operand Y, bool same, int64_t M, int64_t N, 
       }
       c.ar.used = mk;
     }
-    if (!c.ar.dry && first && beta == 0)  // every term vanished mod p
+    if (!c.ar.dry && c.err == AAT_OK && first && beta == 0)  // every term vanished mod p
       check(c, cudaMemset2DAsync(out, (size_t)ldo * 4, 0, (size_t)N * 4, (size_t)M, c.st),
             "zero product");
     c.ar.used = mark;
@@ -663,7 +672,7 @@ static void leaf(Ctx &c, Operand X, Operand Y, bool same, int64_t M, int64_t N, 
           return Q;
         };
         TcLeafArgs b = tc_args(c, part(X.pl, true), part(Y.pl, sums), M, N, kw, nullptr, ldw, lower, 0);
-        if (c.ar.dry || leaf_tc_terms(b, c.m) > 0) parts.push_back(b);
+        if (c.ar.dry || live_part(c, b)) parts.push_back(b);
       }
     int32_t *W = (int32_t *)c.ar.get(parts.size() * (size_t)stride * 4);
     for (size_t q = 0; q < parts.size(); ++q) parts[q].out = c.ar.dry ? nullptr : W + q * stride;

@@ -438,3 +438,22 @@ def test_complex_fp32_class_entries_of_small_values_only(lib, columns, depth):
         err = np.abs(got.cpu().numpy().astype(np.complex128)[h:, :h] - ref) / mag
         assert err.max() <= tol
     plan.close()
+
+
+@pytest.mark.parametrize("p", [65521, 131071, 2**31 - 1])
+@pytest.mark.parametrize("n,k", [(600, 3001), (130, 5000), (3000, 700)])
+def test_exact_bits_too_few_for_the_digits_is_an_error(lib, monkeypatch, n, k, p):
+    """A bound on the partial sums that the digits cannot keep: no part of a
+    split product and no plane pass is left out silently."""
+    import torch
+    A = torch.from_numpy(synth.residues(n + k, (n, k), p)).cuda()
+    calls = [lambda: lib.aat_gemm_modp(A, A, p), lambda: lib.aat_modp(A, p, levels=0),
+             lambda: lib.aat_modp(A, p, levels=0, flags=lib.AAT_LOW_MEMORY)]
+    want = [c().tril() for c in calls]
+    with monkeypatch.context() as m:
+        m.setenv("AAT_EXACT_BITS", "20")
+        for call in calls:
+            with pytest.raises(lib.AatError):
+                call()
+    for call, w in zip(calls, want):
+        assert torch.equal(call().tril(), w)
