@@ -148,7 +148,9 @@ AAT_API int aah_quat_modp(const int32_t *A, const int32_t *B, const int32_t *C, 
  * copied back in bands of 512 rows, band [a, b) carrying columns [0, b).
  * When a recursion level runs, A's top-left block A11 is copied first and
  * the product P1 = Low(A11 A11^T) runs while the rest of A arrives, and the
- * rows below n/2 of C go back while the last product still computes.
+ * rows below n/2 of C go back while the last product still computes (where
+ * they are fewer than 8 MB at one level, the last product joins the others'
+ * launch instead and C goes back after it).
  * Without recursion levels a large product runs in two row parts, the rest
  * of A arriving and the first rows of C going back beside the launches.  With
  * AAT_ZERO_UPPER the whole of C (upper triangle zero) is copied back; with

@@ -836,6 +836,16 @@ static int fuse_override() {
   return v;
 }
 
+// Whether the top level's rows [h, 2h) are worth having early: final before P2,
+// which is then a launch of its own, so that they go back to the host meanwhile.
+// From host memory with one level, P2 in the joint launch / on its own, us:
+// 512^2 mod 65521 152 / 158, 2048^2 274 / 278, 2500^2 396 / 378, 8192^2 3004 /
+// 2883; mod 2^31 - 1 512^2 224 / 231, 2048 x 8192 735 / 756, 2500^2 525 / 457, 8192^2
+// 4626 / 4219.  The line is 8 MB of them, 40 us of the host link.
+static bool early_rows(const Ctx &c, int64_t h, int levels) {
+  return c.split_ev && levels == c.top_levels && 1.5 * 4.0 * (double)h * h >= 8e6;
+}
+
 // Low(A A^T) mod p -> Low(C) by Algorithm 1 with `levels` levels (times
 // c.alpha).  n must be divisible by 2^levels and k by 2^levels (2^(levels+1)
 // for a kind-2 Y).  `ap` optionally holds the digit planes of A
@@ -913,18 +923,27 @@ static void rec(Ctx &c, const int32_t *A, int64_t lda, int64_t n, int64_t k, int
     wino_products(c, L, A + h * lda + kap, lda, h, kap, C21, C22, ldc, sym, p1_first ? 1 : 2);
   } else if (nfa > 0 && (fo == 1 || (fo < 0 && leaf_tc_fuse_pays(fa, nfa)))) {
     // P2 joins them, into workspace, and steps 6-8 become one kernel: the same
-    // traffic as P2 accumulating onto P1 in a launch of its own, one launch fewer
-    const int64_t ldp2 = (h + 3) / 4 * 4;
-    int32_t *P2 = (int32_t *)c.ar.get((size_t)h * ldp2 * 4);
-    fa[nfa++] = tc_args(c, L.pA12, L.pA12, h, h, kap, P2, ldp2, 1, 0);
-    for (int q = 0; q < nfa; ++q) count_leaf(c, fa[q].M, fa[q].N, fa[q].K, fa[q].lower);
-    if (!c.ar.dry && c.err == AAT_OK)
-      check(c, launch_leaf_tc_multi(fa, nfa, c.m, c.st), "leaf (tensor cores, P1 .. P5)");
-    const bool zero = c.want_zero && levels == c.zero_levels;
-    if (!c.ar.dry && c.err == AAT_OK)
-      check(c, launch_postadd_p2(C11, P2, ldp2, C12, C21, C22, ldc, h, zero, c.m, c.st), "postadd");
-    if (zero) c.zeroed = true;
-    p2_done = true;
+    // traffic as P2 accumulating onto P1 in a launch of its own, one launch fewer.
+    // Not where the rows below h go back to the host while P2 computes, unless
+    // they are few (early_rows)
+    if (early_rows(c, h, levels)) {
+      for (int q = 0; q < nfa; ++q) count_leaf(c, fa[q].M, fa[q].N, fa[q].K, fa[q].lower);
+      if (!c.ar.dry && c.err == AAT_OK)
+        check(c, launch_leaf_tc_multi(fa, nfa, c.m, c.st), "leaf (tensor cores, P1 P3 P4 P5)");
+    } else {
+      const int64_t ldp2 = (h + 3) / 4 * 4;
+      int32_t *P2 = (int32_t *)c.ar.get((size_t)h * ldp2 * 4);
+      fa[nfa++] = tc_args(c, L.pA12, L.pA12, h, h, kap, P2, ldp2, 1, 0);
+      for (int q = 0; q < nfa; ++q) count_leaf(c, fa[q].M, fa[q].N, fa[q].K, fa[q].lower);
+      if (!c.ar.dry && c.err == AAT_OK)
+        check(c, launch_leaf_tc_multi(fa, nfa, c.m, c.st), "leaf (tensor cores, P1 .. P5)");
+      const bool zero = c.want_zero && levels == c.zero_levels;
+      if (!c.ar.dry && c.err == AAT_OK)
+        check(c, launch_postadd_p2(C11, P2, ldp2, C12, C21, C22, ldc, h, zero, c.m, c.st),
+              "postadd");
+      if (zero) c.zeroed = true;
+      p2_done = true;
+    }
   } else {
     // 2. P4^T = S2 S1^T -> C22
     leaf(c, L.oS2, L.oS1, false, h, h, kap, C22, ldc, 0, 0);
@@ -1481,6 +1500,7 @@ static int modp_device(const int32_t *A, int64_t n, int64_t k, int64_t lda, uint
   c.in_rest = in_rest;
   c.in_bands = in_bands;
   c.nbands = in_bands ? nbands : 0;
+  c.split_ev = split_ev;
   size_t need = choose_schedule(c, A, n, k, lda, C, ldc, flags);
   void *ws = nullptr;
   if ((e = ensure_workspace(need, &ws))) {
@@ -1492,7 +1512,6 @@ static int modp_device(const int32_t *A, int64_t n, int64_t k, int64_t lda, uint
     g_last_error.clear();
   }
   c.err = AAT_OK;
-  c.split_ev = split_ev;
   run_plan(c, A, n, k, lda, C, ldc, flags, false, (char *)ws);
   if (split_row) *split_row = c.split_row;
   return c.err;

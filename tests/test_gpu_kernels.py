@@ -457,3 +457,29 @@ def test_exact_bits_too_few_for_the_digits_is_an_error(lib, monkeypatch, n, k, p
                 call()
     for call, w in zip(calls, want):
         assert torch.equal(call().tril(), w)
+
+
+@pytest.mark.parametrize("pinned", [False, True])
+@pytest.mark.parametrize("p", [65521, 131071])
+@pytest.mark.parametrize("n,k,leaves", [(512, 300, 2), (2308, 140, 2), (2312, 140, 3), (4096, 516, 3)])
+def test_host_product_with_a_level_sends_the_lower_rows_early(lib, n, k, leaves, p, pinned):
+    """One level from host memory: P1 first, then the other products, P2 in a
+    launch of its own (behind the event that lets the rows below n/2 go back)
+    where those rows are many; every entry of the lower triangle."""
+    import ctypes
+    import torch
+    from paper_2101_01025_gb300 import _native as nat
+    A = torch.from_numpy(synth.residues(n + k, (n, k), p, balanced=True))
+    C = torch.full((n, n), -3, dtype=torch.int32)
+    if pinned:
+        A, C = A.pin_memory(), C.pin_memory()
+    D = A.cuda().double()                        # |sums| < 2^53
+    ref = torch.remainder((D @ D.T).to(torch.int64), p).tril()
+    prof = nat.Profile()
+    for _ in range(2):
+        C.fill_(-3)
+        nat.check(nat.lib().aat_profile_begin())
+        lib.aat_modp_host(A, p, C=C, levels=1)
+        nat.check(nat.lib().aat_profile_end(ctypes.byref(prof)))
+        assert torch.equal(C.cuda().to(torch.int64).tril(), ref)
+        assert prof.launches[2] == leaves        # AAT_K_LEAF_TC
