@@ -298,6 +298,7 @@ struct DeviceState {
   void *ws = nullptr;
   size_t ws_size = 0;
   int32_t *status = nullptr;
+  uint32_t pace_next = 0;  // pacing slots follow the status word (kPaceOffset)
   // buffers of the end-to-end host entry point
   void *e2e_a = nullptr, *e2e_c = nullptr;
   size_t e2e_a_size = 0, e2e_c_size = 0;
@@ -310,6 +311,7 @@ struct DeviceState {
 
 static std::mutex g_state_mu;
 static std::map<int, DeviceState> g_states;
+constexpr size_t kPaceOffset = 256;
 
 static DeviceState &state() {
   int dev = 0;
@@ -321,10 +323,18 @@ int32_t *device_status_ptr() {
   std::lock_guard<std::mutex> lock(g_state_mu);
   DeviceState &s = state();
   if (!s.status) {
-    if (cudaMalloc(&s.status, sizeof(int32_t)) != cudaSuccess) return nullptr;
+    if (cudaMalloc(&s.status, kPaceOffset + sizeof(uint32_t) * kPaceSlots * kPaceMax) != cudaSuccess)
+      return nullptr;
     cudaMemset(s.status, 0, sizeof(int32_t));
   }
   return s.status;
+}
+
+uint32_t *device_pace_slot() {
+  std::lock_guard<std::mutex> lock(g_state_mu);
+  DeviceState &s = state();
+  if (!s.status) return nullptr;
+  return (uint32_t *)((char *)s.status + kPaceOffset) + (s.pace_next++ % kPaceSlots) * kPaceMax;
 }
 
 // Test hook: workspace requests above this many bytes fail with AAT_ENOMEM

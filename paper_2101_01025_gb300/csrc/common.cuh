@@ -301,6 +301,13 @@ __device__ __forceinline__ void store_digits_t(const Planes &P, int64_t r, int64
 
 // Sticky status word written by kernels whose bounded waits give up.
 int32_t *device_status_ptr();
+// Counters for pacing one leaf launch (k_leaf_tc.cu): one of kPaceSlots arrays of
+// kPaceMax words per device, in turn, so that launches on other streams and in
+// captured plans count in arrays of their own.  They are allocated with the status
+// word, before any launch: nothing is allocated here.  Null: none.
+constexpr uint32_t kPaceMax = 4096;
+constexpr int kPaceSlots = 16;
+uint32_t *device_pace_slot();
 
 // --------------------------------------------------- instrumentation
 

@@ -313,7 +313,6 @@ struct Shape {
 // pairs that never run together only lose that time.  8192^3 mod 2^31 - 1: DRAM
 // reads 17-23 -> 11.4 GB, 5.9-6.25 -> 5.73 ms; 16384 x 16384 26.0-26.5 ->
 // 24.8 ms a pass under the power cap (limits of 3 and 10 us alike).
-constexpr uint32_t kPaceMax = 4096;
 constexpr unsigned long long kPaceNs = 5000;
 
 // Epilogue warps of the single-problem launches and of the batched launch
@@ -1118,9 +1117,6 @@ int pair_override() {
   return v;
 }
 
-// The pacing counters of the current device, cleared on `st`, for a launch whose
-// groups are long enough to drift apart in; null (no pacing) otherwise.
-std::map<int, uint32_t *> g_pace;
 // Shared-memory limits of the single-product kernel's forms (pair_units sets the
 // whole pair form's), set
 // together whichever entry point launches first (g_mu held).
@@ -1160,14 +1156,13 @@ enum Form { kCta = 1, kPair = 2, kNarrow = 3, kPairHalf = 4 };
 bool is_pair(Form f) { return f == kPair || f == kPairHalf; }
 int form_tm(Form f) { return is_pair(f) ? 256 : 128; }
 int form_tn(Form f) { return f == kNarrow ? kTnNarrow : f == kPairHalf ? kTnHalf : BN; }
-uint32_t *pace_for(int dev, Form f, int64_t K, int ntiles, int units, int ngroups,
+
+// Pacing counters, cleared on `st`, for a launch whose groups are long enough to
+// drift apart in; null (no pacing) otherwise.
+uint32_t *pace_for(Form f, int64_t K, int ntiles, int units, int ngroups,
                    cudaStream_t st) {
   if (f != kPair || K < 2048 || ntiles < 2 * units) return nullptr;
-  uint32_t *&p = g_pace[dev];
-  if (!p && cudaMalloc(&p, kPaceMax * sizeof(uint32_t)) != cudaSuccess) {
-    cudaGetLastError();
-    p = nullptr;
-  }
+  uint32_t *p = device_pace_slot();
   const int64_t n = std::min<int64_t>(kPaceMax, (int64_t)((ntiles + units - 1) / units) * ngroups);
   if (!p || cudaMemsetAsync(p, 0, (size_t)n * 4, st) != cudaSuccess) {
     cudaGetLastError();
@@ -1306,7 +1301,7 @@ cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) 
   }
   P->tiles = tiles;
   P->ntiles = nt;
-  P->pace = pace_for(dev, form, a.K, nt, units, ng, st);
+  P->pace = pace_for(form, a.K, nt, units, ng, st);
   if ((e = set_single_attrs(dev)) != cudaSuccess) { delete P; return e; }
   if (nt > 0) {
     // algorithmic tensor work: one BF16 product of the ring MACs per plane
@@ -1735,9 +1730,6 @@ void leaf_tc_release() {
   for (auto &kv : g_mtiles)
     if (kv.second.first) cudaFree(kv.second.first);
   g_mtiles.clear();
-  for (auto &kv : g_pace)
-    if (kv.second) cudaFree(kv.second);
-  g_pace.clear();
   g_attr_set.clear();
   g_pair_units.clear();
 }

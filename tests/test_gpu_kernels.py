@@ -483,3 +483,58 @@ def test_host_product_with_a_level_sends_the_lower_rows_early(lib, n, k, leaves,
         nat.check(nat.lib().aat_profile_end(ctypes.byref(prof)))
         assert torch.equal(C.cuda().to(torch.int64).tril(), ref)
         assert prof.launches[2] == leaves        # AAT_K_LEAF_TC
+
+
+def test_paced_product_is_capturable_once_its_tiles_are_known(lib):
+    """In a fresh process: a short product of CTA pairs makes every cache of its
+    shape, then a longer one, whose pairs are paced, is captured and replayed."""
+    import os
+    import subprocess
+    import sys
+    code = """
+import torch
+import paper_2101_01025_gb300 as aat
+from paper_2101_01025_gb300 import _native as nat
+p = 65521
+A = torch.randint(0, p, (6144, 2048), dtype=torch.int32, device="cuda")
+C = torch.zeros((6144, 6144), dtype=torch.int32, device="cuda")
+nat.check(nat.lib().aatx_workspace_reserve(1 << 28))
+aat.aat_modp(A[:, :1024], p, C=C, levels=0)
+torch.cuda.synchronize()
+g = torch.cuda.CUDAGraph()
+with torch.cuda.graph(g):
+    aat.aat_modp(A, p, C=C, levels=0)
+D = A.double()
+ref = torch.remainder((D @ D.T).long(), p).tril()
+for _ in range(3):
+    C.zero_()
+    g.replay()
+    assert torch.equal(C.long().tril(), ref)
+print("ok")
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
+
+
+def test_paced_products_at_once(lib):
+    """Two plans of paced products on two streams, more launches than there are
+    counter arrays."""
+    import torch
+    p = 65521
+    mats = [torch.from_numpy(synth.residues(i, (6144, 2048), p)).cuda() for i in range(2)]
+    outs = [[torch.zeros((6144, 6144), dtype=torch.int32, device="cuda") for _ in range(2)] for _ in mats]
+    plans = [lib.Plan([("modp", A, C, p, lib.AAT_ZERO_UPPER) for C in cs]) for A, cs in zip(mats, outs)]
+    streams = [torch.cuda.Stream() for _ in plans]
+    torch.cuda.synchronize()
+    for _ in range(6):
+        for plan, s in zip(plans, streams):
+            plan.execute(stream=s)
+    torch.cuda.synchronize()
+    for A, cs in zip(mats, outs):
+        D = A.double()
+        ref = torch.remainder((D @ D.T).to(torch.int64), p).tril()
+        assert all(torch.equal(C.to(torch.int64), ref) for C in cs)
+    for plan in plans:
+        plan.close()
