@@ -310,10 +310,16 @@ struct Shape {
 // same plane product and K position, and nothing but their equal speed keeps
 // them there.  At the start of each group a pair's producer counts itself and
 // waits for the others of its wave, at most kPaceNs: a hint, not a barrier, so
-// pairs that never run together only lose that time.  8192^3 mod 2^31 - 1: DRAM
-// reads 17-23 -> 11.4 GB, 5.9-6.25 -> 5.73 ms; 16384 x 16384 26.0-26.5 ->
-// 24.8 ms a pass under the power cap (limits of 3 and 10 us alike).
+// pairs that never run together (other work holds SMs) only lose that time,
+// kPaceTries times in a row.  8192^3 mod 2^31 - 1: DRAM reads 17-23 -> 11.4 GB,
+// 5.9-6.25 -> 5.73 ms; 16384 x 16384 26.0-26.5 -> 24.8 ms a pass under the power
+// cap (limits of 3 and 10 us alike).  With 100 blocks of another kernel on the
+// SMs all the while, 16384 x 4096 mod 2^31 - 1: waiting at every group 18.4 ms,
+// giving up after 8 or 20 in a row 16.4, unpaced 16.3.  Giving up after 3 stops
+// pairs that are only slow (12000 x 6000 x 12000 mod 2^31 - 1 10.9 -> 11.4 ms; 8
+// and 20 10.9).
 constexpr unsigned long long kPaceNs = 5000;
+constexpr int kPaceTries = 10;
 
 // Epilogue warps of the single-problem launches and of the batched launch
 // (whose tiles are mostly short in K, so the per-tile epilogue dominates).
@@ -410,6 +416,7 @@ __global__ void __launch_bounds__(Shape<PAIR, EW, TN>::THREADS, 1)
       // both CTAs' copies of a stage complete on the leader's FULL barrier
       const uint32_t full0 = PAIR ? map_to_rank(FULL(0), 0) : FULL(0);
       uint32_t seq = 0;
+      int tries = kPaceTries;
       for (int t = (int)unit0; t < P.ntiles && ok; t += (int)nunits) {
         const TileView v = tile_view<MODE>(P, t);
         const int rowx = v.I * S::TM + (int)rank * BM;
@@ -420,8 +427,12 @@ __global__ void __launch_bounds__(Shape<PAIR, EW, TN>::THREADS, 1)
             if (P.pace && leader && seq < kPaceMax) {
               const uint32_t all = (uint32_t)min((int)nunits, P.ntiles - (t - (int)unit0));
               atomicAdd(P.pace + seq, 1u);
-              const unsigned long long t0 = gtimer();
-              while (*(volatile uint32_t *)(P.pace + seq) < all && gtimer() - t0 < kPaceNs) {
+              if (tries) {
+                const unsigned long long t0 = gtimer();
+                bool late = false;
+                while (*(volatile uint32_t *)(P.pace + seq) < all && !late)
+                  late = gtimer() - t0 >= kPaceNs;
+                tries = late ? tries - 1 : kPaceTries;
               }
             }
             ++seq;
@@ -1157,26 +1168,35 @@ bool is_pair(Form f) { return f == kPair || f == kPairHalf; }
 int form_tm(Form f) { return is_pair(f) ? 256 : 128; }
 int form_tn(Form f) { return f == kNarrow ? kTnNarrow : f == kPairHalf ? kTnHalf : BN; }
 
-// Pacing counters, cleared on `st`, for a launch whose groups are long enough to
-// drift apart in; null (no pacing) otherwise.
-uint32_t *pace_for(Form f, int64_t K, int ntiles, int units, int ngroups,
+// Plane products per ring multiply-add of a leaf.
+int term_count(const TcLeafArgs &a) {
+  return a.dx.nsum > 0 ? std::min(a.x.L, a.y.L) : a.x.L * a.y.L;
+}
+
+// Pacing counters, cleared on `st`, for a launch long enough for its pairs to
+// drift apart; null (no pacing) otherwise.  A group start costs every pair a
+// fraction of a microsecond; what it saves grows with the launch: waves x K x
+// plane products, 400 thousand being about 1.7 ms.  Unpaced / paced time, lower
+// products, on two boxes: 8192 x 2048 mod 65521 (43 k) 0.97, 0.98; 16384 x 4096
+// (344 k) 0.99, 0.98; 12000 x 2048 mod 2^31 - 1 (307 k) 0.99, 0.98; 8192 x 6000
+// (420 k) 1.014, 1.00; 16384 x 3072 mod 1000003 (516 k) 0.99, 1.00; 12000^2 mod 65521
+// (540 k) 1.03; 8192^2 mod 2^31 - 1 (573 k) 1.03; 16384 x 8192 mod 65521 (688 k) 1.00,
+// 1.06; 16384 x 3072 mod 2^31 - 1 (860 k) 0.99, 1.08; 16384^2 (4.6 M) 1.11.
+uint32_t *pace_for(Form f, const TcLeafArgs &a, int ntiles, int units, int ngroups,
                    cudaStream_t st) {
-  if (f != kPair || K < 2048 || ntiles < 2 * units) return nullptr;
+  const int64_t waves = units > 0 ? (ntiles + units - 1) / units : 0;
+  if (f != kPair || a.K < 2048 || waves < 2 || waves * a.K * term_count(a) < 400000) return nullptr;
   uint32_t *p = device_pace_slot();
-  const int64_t n = std::min<int64_t>(kPaceMax, (int64_t)((ntiles + units - 1) / units) * ngroups);
+  const int64_t n = std::min<int64_t>(kPaceMax, waves * ngroups);
   if (!p || cudaMemsetAsync(p, 0, (size_t)n * 4, st) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }
   return p;
 }
+
 // rows of Y per CTA and stage
 int form_yrows(Form f) { return is_pair(f) ? form_tn(f) / 2 : form_tn(f); }
-
-// Plane products per ring multiply-add of a leaf.
-int term_count(const TcLeafArgs &a) {
-  return a.dx.nsum > 0 ? std::min(a.x.L, a.y.L) : a.x.L * a.y.L;
-}
 
 // Modelled SM cycles of one tile of a one-CTA form: per plane product its K
 // blocks, a Horner step and a drain; prologue, fill and store.  Fitted to
@@ -1301,7 +1321,7 @@ cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) 
   }
   P->tiles = tiles;
   P->ntiles = nt;
-  P->pace = pace_for(form, a.K, nt, units, ng, st);
+  P->pace = pace_for(form, a, nt, units, ng, st);
   if ((e = set_single_attrs(dev)) != cudaSuccess) { delete P; return e; }
   if (nt > 0) {
     // algorithmic tensor work: one BF16 product of the ring MACs per plane

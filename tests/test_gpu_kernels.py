@@ -496,9 +496,9 @@ import torch
 import paper_2101_01025_gb300 as aat
 from paper_2101_01025_gb300 import _native as nat
 p = 65521
-A = torch.randint(0, p, (6144, 2048), dtype=torch.int32, device="cuda")
+A = torch.randint(0, p, (6144, 33344), dtype=torch.int32, device="cuda")
 C = torch.zeros((6144, 6144), dtype=torch.int32, device="cuda")
-nat.check(nat.lib().aatx_workspace_reserve(1 << 28))
+nat.check(nat.lib().aatx_workspace_reserve(1 << 31))
 aat.aat_modp(A[:, :1024], p, C=C, levels=0)
 torch.cuda.synchronize()
 g = torch.cuda.CUDAGraph()
@@ -523,12 +523,15 @@ def test_paced_products_at_once(lib):
     counter arrays."""
     import torch
     p = 65521
-    mats = [torch.from_numpy(synth.residues(i, (6144, 2048), p)).cuda() for i in range(2)]
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    mats = [torch.randint(0, p, (6144, 33344), dtype=torch.int32, device="cuda", generator=g)
+            for _ in range(2)]
     outs = [[torch.zeros((6144, 6144), dtype=torch.int32, device="cuda") for _ in range(2)] for _ in mats]
     plans = [lib.Plan([("modp", A, C, p, lib.AAT_ZERO_UPPER) for C in cs]) for A, cs in zip(mats, outs)]
     streams = [torch.cuda.Stream() for _ in plans]
     torch.cuda.synchronize()
-    for _ in range(6):
+    for _ in range(5):
         for plan, s in zip(plans, streams):
             plan.execute(stream=s)
     torch.cuda.synchronize()
