@@ -1652,7 +1652,12 @@ int aat_modp(const int32_t *A, int64_t n, int64_t k, uint32_t p, int32_t *C, voi
 // Copies, product and copies one after the other took 2.85 ms at 6000 x 5000
 // mod 2^31 - 1 (0.6 + 1.5 + 0.7), two parts 2.49 ms; 8192 x 8192 5.9 -> 4.5 ms.
 // The row split with the shortest modelled sequence: the first rows in, both
-// launches (whole waves of tiles), the last rows out.  0: one part.
+// launches (whole waves of tiles), the last rows out, and 10 us for the further
+// launches; against them the one product as it would run, in parts of plane
+// products where its tiles are few, with 45 us for the 17 copies in which A comes
+// in without AAT_ZERO_UPPER.  Two row parts / one, us, upper triangle cleared: 1024 x
+// 256 mod 65521 79 / 69, 1536^2 146 / 163, 2048 x 8192 mod 2^31 - 1 852 / 746, 3000^2
+// 548 / 711; not cleared: 105 / 99, 136 / 192, 761 / 756, 522 / 699.  0: one part.
 static int64_t host_two_parts_rows(const Ctx &c, int64_t n, int64_t k, uint32_t flags) {
   TuneVal tv;
   if (c.leaf != AAT_LEAF_TC || c.passes || prepare_levels(n, k, c.m.p, flags) != 0 ||
@@ -1663,15 +1668,16 @@ static int64_t host_two_parts_rows(const Ctx &c, int64_t n, int64_t k, uint32_t 
   auto model = [&](int64_t r1) {
     const Planes P1 = planes_for(c.ds, r1, k), P2 = planes_for(c.ds, n - r1, k);
     const TcLeafArgs a = tc_args(c, P1, P1, r1, r1, k, nullptr, n, 1, 0);
-    double t = (double)r1 * k * 4.0 * us_per_byte + leaf_tc_model_us(&a, 1);
-    if (r1 == n) return t + (zero ? (double)n * n : 0.5 * (double)n * n) * 4.0 * us_per_byte;
+    double t = (double)r1 * k * 4.0 * us_per_byte + leaf_tc_model_us(&a, 1, r1 == n);
+    if (r1 == n)
+      return t + (zero ? (double)n * n : 0.5 * (double)n * n) * 4.0 * us_per_byte + (zero ? 0.0 : 45.0);
     const TcLeafArgs b[2] = {tc_args(c, P2, P1, n - r1, r1, k, nullptr, n, 0, 0),
                              tc_args(c, P2, P2, n - r1, n - r1, k, nullptr, n, 1, 0)};
-    t += leaf_tc_model_us(b, 2);
+    t += leaf_tc_model_us(b, 2) + 10.0;
     return t + (double)(n - r1) * n * 4.0 * us_per_byte;
   };
   int64_t best = 0;
-  double bt = 0.9 * model(n);
+  double bt = 0.95 * model(n);
   // multiples of 512, as the bands in which the lower triangle goes back
   for (int64_t r1 = 512; r1 + 512 <= n; r1 += 512) {
     const double t = model(r1);

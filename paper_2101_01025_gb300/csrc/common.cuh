@@ -473,14 +473,15 @@ struct LeafSplit {
   int window = 0, slices = 1;
   int64_t slice_k = 0;
 };
-LeafSplit leaf_tc_split(const TcLeafArgs &a);
+LeafSplit leaf_tc_split(const TcLeafArgs &a, double *cycles = nullptr);
 // out <- sum of `parts` canonical M x N blocks W + q stride (row stride ldw)
 // + beta out mod p (lower: i >= j; zero: the strict upper triangle is cleared).
 cudaError_t launch_partial_sum(const int32_t *W, int64_t ldw, int64_t stride, int parts,
                                int32_t *out, int64_t ldo, int64_t M, int64_t N, int lower,
                                bool zero, const MulConst &beta, const ModP &m, cudaStream_t st);
-// Modelled time of one launch over `count` products.
-double leaf_tc_model_us(const TcLeafArgs *as, int count);
+// Modelled time of one launch over `count` products; parts: of one product, as
+// parts where leaf_tc_split makes them.
+double leaf_tc_model_us(const TcLeafArgs *as, int count, bool parts = false);
 // Whether that one launch is expected to beat one launch per product (the
 // idle share of the separate launches' last waves).
 bool leaf_tc_fuse_pays(const TcLeafArgs *as, int count);

@@ -1408,7 +1408,7 @@ bool leaf_tc_fuse_pays(const TcLeafArgs *as, int count) {
 // x 1001 x 3001 (lower) mod 2^31 - 1: 72 narrow tiles 69 us; two parts of five
 // plane products, 144 units, 38 + 6 us; five parts of two on wide tiles, 100
 // units, 46 + 7 us.
-LeafSplit leaf_tc_split(const TcLeafArgs &a) {
+LeafSplit leaf_tc_split(const TcLeafArgs &a, double *cycles) {
   LeafSplit best;
   if (a.form != 0 || pair_override() >= 0 || a.x.q0 || a.y.q0) return best;
   int dev = 0;
@@ -1451,10 +1451,11 @@ LeafSplit leaf_tc_split(const TcLeafArgs &a) {
         best.slice_k = (kblocks + s - 1) / s * BK;
       }
     }
+  if (cycles && best.window > 0) *cycles = bc;
   return best;
 }
 
-double leaf_tc_model_us(const TcLeafArgs *as, int count) {
+double leaf_tc_model_us(const TcLeafArgs *as, int count, bool parts) {
   int dev = 0, units = 0;
   cudaGetDevice(&dev);
   {
@@ -1463,6 +1464,7 @@ double leaf_tc_model_us(const TcLeafArgs *as, int count) {
   }
   double cycles = 0.0;
   leaf_form(as, count, units, sm_count(dev), &cycles);
+  if (parts && count == 1) leaf_tc_split(as[0], &cycles);
   return cycles / 1.9e3;  // at 1.9 GHz
 }
 

@@ -541,3 +541,26 @@ def test_paced_products_at_once(lib):
         assert all(torch.equal(C.to(torch.int64), ref) for C in cs)
     for plan in plans:
         plan.close()
+
+
+@pytest.mark.parametrize("p,n,k,launches", [(2**31 - 1, 2048, 8192, 1), (65521, 1024, 256, 1),
+                                            (65521, 3000, 3000, 2), (2**31 - 1, 3000, 3000, 2)])
+def test_host_row_parts_against_the_one_product_as_it_runs(lib, p, n, k, launches):
+    """Two row parts only where the one product, itself in parts of plane
+    products where its tiles are few, takes longer (leaf launches of a call)."""
+    import ctypes
+    import torch
+    from paper_2101_01025_gb300 import _native as nat
+    A = torch.from_numpy(synth.residues(n + k, (n, k), p, balanced=True)).pin_memory()
+    C = torch.zeros((n, n), dtype=torch.int32).pin_memory()
+    prof = nat.Profile()
+    nat.check(nat.lib().aat_profile_begin())
+    lib.aat_modp_host(A, p, C=C, flags=lib.AAT_ZERO_UPPER)
+    nat.check(nat.lib().aat_profile_end(ctypes.byref(prof)))
+    assert prof.launches[2] == launches          # AAT_K_LEAF_TC
+    assert torch.equal(C, lib.aat_modp(A.cuda(), p, flags=lib.AAT_ZERO_UPPER).cpu())
+    X = A.numpy().astype(np.int64)
+    rows = [0, 1, 511, 512, n // 2, n - 1]
+    ref = ((X @ (X[rows] >> 16).T) % p * 65536 + X @ (X[rows] & 0xffff).T) % p
+    for i, r in enumerate(rows):
+        assert np.array_equal(C[r, :r + 1].numpy().astype(np.int64), ref[:r + 1, i])
