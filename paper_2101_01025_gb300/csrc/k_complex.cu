@@ -1215,6 +1215,12 @@ struct FusedLaunch {
   FForm form = kFCta;
 };
 
+static int sm_count_c(int dev) {
+  int sms = 148;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
 static cudaError_t fused_table(const std::vector<FusedJob> &jobs, int np, int64_t K,
                                void *table_mem, cudaStream_t st, int32_t *wide,
                                FusedLaunch *out) {
@@ -1224,8 +1230,7 @@ static cudaError_t fused_table(const std::vector<FusedJob> &jobs, int np, int64_
   int dev = 0;
   cudaGetDevice(&dev);
   const int units = pair_units_c(dev);
-  int sms = 148;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = sm_count_c(dev);
   const int kblocks = (int)((K + BK - 1) / BK);
   bool pair = units > 0;
   int64_t pt = 0;
@@ -1240,19 +1245,26 @@ static cudaError_t fused_table(const std::vector<FusedJob> &jobs, int np, int64_
   if (!pair) {
     // 64-column tiles when that shortens the longest CTA: waves of tiles times
     // modelled SM cycles of a tile, 512 (wide) or 240 (narrow) per K block and
-    // piece product.  A A^H per call, FP32 class: 300 x 300 42 -> 30 us, 500 x
+    // piece product of its job.  A A^H per call, FP32 class: 300 x 300 42 -> 30 us, 500 x
     // 2000 104 -> 56 us, 100 x 5000 208 -> 99 us (half of it the FP16 pieces).
     double cost[2];
     for (int w = 0; w < 2; ++w) {
       const int tn = w ? kFNarrow : BN;
       int64_t tiles = 0;
-      for (const FusedJob &j : jobs)
+      double cycles = 0.0;
+      for (const FusedJob &j : jobs) {
+        int pairs[6][2];
+        const int products = wide ? kHalfTerms : piece_pairs(std::min(j.keep, np), pairs);
+        int64_t t = 0;
         for (int64_t i = 0; i < (j.M + BM - 1) / BM; ++i) {
           const int64_t TJ = (j.N + tn - 1) / tn;
-          tiles += j.lower ? std::min(TJ, (i * BM + BM - 1) / tn + 1) : TJ;
+          t += j.lower ? std::min(TJ, (i * BM + BM - 1) / tn + 1) : TJ;
         }
-      cost[w] = (double)((tiles + sms - 1) / sms) *
-                (w ? 240.0 * 3.0 * kblocks + 5000.0 : 512.0 * 3.0 * kblocks + 14000.0);
+        cycles += (double)t * (w ? 240.0 * products * kblocks + 5000.0
+                                 : 512.0 * products * kblocks + 14000.0);
+        tiles += t;
+      }
+      cost[w] = cycles / (double)tiles * (double)((tiles + sms - 1) / sms);
     }
     if (cost[1] < cost[0]) form = kFNarrowForm;
   }
@@ -1638,6 +1650,19 @@ static void csplit(CCtx &c, const float2 *A, int64_t lda, int64_t rows, int64_t 
   cchk(c, cudaGetLastError(), "complex split");
 }
 
+// FP16 pieces for an n x k product of the FP32 class (three pieces; whether its
+// values allow them is decided on the device).  A A^H reads A for its diagonal
+// anyway; A A^T pays a launch and a pass for the row scales, so only where the three
+// products it saves take longer than that (~3 us).  One rule for single calls and
+// plans.
+static bool half_pieces(int np, int herm, int64_t n, int64_t k) {
+  if (np != 3 || herm) return np == 3;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const double waves = std::ceil(1.5 * (double)n * n / ((double)(BM * BN) * sm_count_c(dev)));
+  return waves * (double)((k + BK - 1) / BK) * 3.0 * 512.0 > 6000.0;
+}
+
 // Algorithm 2: Low(X phi(X)) into C (herm: phi = conjugate transposition).
 static void c_two_m(CCtx &c, const float2 *A, int64_t lda, int64_t n, int64_t k, float2 *C,
                     int64_t ldc, int herm) {
@@ -1650,14 +1675,8 @@ static void c_two_m(CCtx &c, const float2 *A, int64_t lda, int64_t n, int64_t k,
   float *H = (float *)c.ar.get((size_t)n * n * 4);
   float *G = (float *)c.ar.get((size_t)n * n * 4);
   void *table = c.ar.get(fused_table_bytes());
-  // FP32 class (three pieces): FP16 pieces, decided on the device.  A A^H reads
-  // A for its diagonal anyway; A A^T pays a launch and a pass for the row
-  // scales, so only where the three products it saves take longer than that
-  // (~3 us).
   RowScale rs = {};
-  const double saved = std::ceil(1.5 * (double)n * n / (BM * BN * 152.0)) *
-                       (double)((k + BK - 1) / BK) * 3.0 * 512.0;
-  if (c.np == 3 && (herm || saved > 6000.0)) {
+  if (half_pieces(c.np, herm, n, k)) {
     rs.e = (int32_t *)c.ar.get((size_t)(n + 1) * 4);
     rs.wide = rs.e + n;
   }
@@ -2033,7 +2052,7 @@ cudaError_t cbatch_build(const CBInput *in, int count, char *ws, CBatch *out) {
     w += r256c((size_t)q.n * q.n * 4);
     b.G = (float *)w;
     w += r256c((size_t)q.n * q.n * 4);
-    if (np == 3) {  // as c_two_m
+    if (half_pieces(np, q.herm, q.n, q.k)) {
       b.rs.e = (int32_t *)w;
       b.rs.wide = L->flags + i;
     }
