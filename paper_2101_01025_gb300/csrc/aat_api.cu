@@ -2261,6 +2261,8 @@ int aatx_plan_stats(int64_t n, int64_t k, uint32_t p, uint32_t flags, aatx_plan_
   Ctx c;
   int e = setup(c, p, flags, nullptr);
   if (e) return e;
+  c.use_product_digits(flags);
+  c.small_ok = true;
   c.stats = out;
   out->workspace_bytes = run_plan(c, nullptr, n, k, k, nullptr, n, flags, true, nullptr);
   return AAT_OK;

@@ -368,3 +368,14 @@ def test_wait_probe_rejects_bad_arguments():
     assert lib.aatx_wait_probe(2, 1000, None) == _native.AAT_EINVAL
     assert lib.aatx_wait_probe(0, 0, None) == _native.AAT_EINVAL
     assert lib.aatx_wait_probe(0, 3 * 10**9, None) == _native.AAT_EINVAL
+
+
+@pytest.mark.parametrize("p", [13, 65521, 65537, 131071, 1000003, 2**31 - 1])
+@pytest.mark.parametrize("n,k", [(33, 40), (96, 160), (512, 512), (1001, 3000), (4096, 2048)])
+def test_plan_statistics_report_the_products_workspace(p, n, k):
+    """The statistics' workspace is that of the product itself (its digit
+    form, no workspace where one CUDA-core launch does it)."""
+    lib = _native.lib()
+    for flags in (0, _native.AAT_LEVELS(0), _native.AAT_LEVELS(1), _native.AAT_LEVELS(2),
+                  _native.AAT_LEVELS(1) | _native.AAT_DIGITS_PLAIN, _native.AAT_ZERO_UPPER):
+        assert T.plan_stats(n, k, p, flags).workspace_bytes == lib.aat_workspace_size(n, k, p, flags)
