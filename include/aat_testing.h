@@ -69,7 +69,7 @@ AAT_API int aatx_sblocks(const int32_t *A, int64_t n, int64_t k, int64_t lda, ui
 
 /* Digit planes (then pair-sum planes) of the residue block X (rows x cols)
  * as raw bf16 bits: planes[(d * rows + r) * kstride + c], kstride = cols
- * rounded up to 8; planes 8-byte aligned. */
+ * rounded up to 8, the columns from cols on zero. */
 AAT_API int aatx_split(const int32_t *X, int64_t rows, int64_t cols, int64_t ldx, uint32_t p,
                uint16_t *planes, void *stream);
 

@@ -2294,7 +2294,17 @@ int aatx_split(const int32_t *X, int64_t rows, int64_t cols, int64_t ldx, uint32
   if ((e = check_device())) return e;
   Planes P = planes_for(c.ds, rows, cols);
   P.ptr = (__nv_bfloat16 *)planes;
+  // the kernels store quads: planes off 8 bytes are written by way of the workspace
+  const bool off = ((uintptr_t)planes & 7) != 0 && rows > 0 && cols > 0;
+  const size_t bytes = (size_t)P.L * rows * P.kstride * 2;
+  if (off) {
+    void *ws = nullptr;
+    if ((e = ensure_workspace(bytes, &ws))) return e;
+    P.ptr = (__nv_bfloat16 *)ws;
+  }
   cudaError_t ce = launch_split(X, ldx, rows, cols, c.m, c.ds.b, P, c.st);
+  if (ce == cudaSuccess && off)
+    ce = cudaMemcpyAsync(planes, P.ptr, bytes, cudaMemcpyDeviceToDevice, c.st);
   return ce == cudaSuccess ? AAT_OK : cuda_fail(ce, "split");
 }
 

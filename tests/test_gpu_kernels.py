@@ -564,3 +564,20 @@ def test_host_row_parts_against_the_one_product_as_it_runs(lib, p, n, k, launche
     ref = ((X @ (X[rows] >> 16).T) % p * 65536 + X @ (X[rows] & 0xffff).T) % p
     for i, r in enumerate(rows):
         assert np.array_equal(C[r, :r + 1].numpy().astype(np.int64), ref[:r + 1, i])
+
+
+@pytest.mark.parametrize("off", [0, 1, 2, 3, 4])
+@pytest.mark.parametrize("rows,cols", [(3, 8), (5, 13)])
+def test_split_into_planes_at_any_offset(lib, rows, cols, off):
+    """Planes whose first word lies `off` words of 16 bits from 16 bytes."""
+    import torch
+    from paper_2101_01025_gb300 import _native as nat
+    from paper_2101_01025_gb300 import testing as T
+    p = 2**31 - 1
+    X = torch.from_numpy(synth.residues(rows, (rows, cols), p, balanced=True)).cuda()
+    want = T.split(X, p).view(torch.int16).flatten()
+    buf = torch.full((want.numel() + off + 8,), 77, dtype=torch.int16, device="cuda")
+    nat.check(nat.lib().aatx_split(X.data_ptr(), rows, cols, X.stride(0), p,
+                                   buf.data_ptr() + 2 * off, T._stream()))
+    assert torch.equal(buf[off:off + want.numel()], want)
+    assert bool((buf[:off] == 77).all()) and bool((buf[off + want.numel():] == 77).all())
