@@ -566,13 +566,13 @@ __device__ __forceinline__ void cload4(const float2 *__restrict__ a_row, int64_t
   }
 }
 
-// The pieces of 4 consecutive values a[0..nv) of row r, columns c0.., into
-// every plane set of o: one 8-byte store per plane (kstride is a multiple of
-// 8); a ragged last quad stores element by element.
+// The pieces of 4 consecutive values of row r, columns c0.., into every plane
+// set of o: one 8-byte store per plane (kstride is a multiple of 8; a ragged last
+// quad stores zeros into the row padding).
 // sc != 0: two FP16 pieces of the values times sc (a power of two), the second
 // one times kHalfUp.
-__device__ __forceinline__ void csplit_store(const float2 (&a)[4], int64_t r, int64_t c0, int nv,
-                                             int np, const CSplitOut &o, float sc = 0.0f) {
+__device__ __forceinline__ void csplit_store(const float2 (&a)[4], int64_t r, int64_t c0, int np,
+                                             const CSplitOut &o, float sc = 0.0f) {
   const Planes *outs[4] = {&o.re, &o.im, &o.s, &o.d};
 #pragma unroll
   for (int w = 0; w < 4; ++w) {
@@ -622,13 +622,7 @@ __device__ __forceinline__ void csplit_store(const float2 (&a)[4], int64_t r, in
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
       if (q >= nq) break;
-      if (nv == 4) {
-        *reinterpret_cast<uint2 *>(dst + q * plane) = pc[q];
-      } else {
-        const uint16_t pv[4] = {(uint16_t)pc[q].x, (uint16_t)(pc[q].x >> 16), (uint16_t)pc[q].y,
-                                (uint16_t)(pc[q].y >> 16)};
-        for (int v = 0; v < nv; ++v) dst[q * plane + v] = pv[v];
-      }
+      *reinterpret_cast<uint2 *>(dst + q * plane) = pc[q];
     }
   }
 }
@@ -664,11 +658,12 @@ __device__ __forceinline__ void csplit_quad(const float2 *__restrict__ a_row, in
   const int nv = (int)min((int64_t)4, cols - c0);
   float2 a[4];
   cload4(a_row, c0, nv, a);
-  csplit_store(a, r, c0, nv, np, o, sc);
+  csplit_store(a, r, c0, np, o, sc);
 }
 
-__global__ void csplit_kernel(const float2 *__restrict__ A, int64_t lda, int64_t rows, int64_t cols,
-                              int np, CSplitOut o, RowScale rs) {
+__global__ void __launch_bounds__(256, 4)
+    csplit_kernel(const float2 *__restrict__ A, int64_t lda, int64_t rows, int64_t cols, int np,
+                  CSplitOut o, RowScale rs) {
   const int64_t cq = (cols + 3) / 4;
   for (int64_t r = blockIdx.y; r < rows; r += gridDim.y) {
     const float sc = row_scale(rs, r);
@@ -1462,13 +1457,17 @@ __global__ void csblocks_kernel(const float2 *__restrict__ A, int64_t lda, int64
 // The last level of Algorithm 1 over C (Y = i I) in one pass over A: the S
 // blocks S1 = (A21 - A11) i, S2 = A22 - A21 i, S3 = S1 - A22, S4 = S3 + A12
 // are formed in registers and, with A11, A12, A22, written straight out as
-// the BF16 pieces of the operand sets of the level's fused products.
+// the BF16 pieces of the operand sets of the level's fused products.  Bound by HBM.
+// FP32 class, 8192^2 444 us, 3790 x 3634 121, 3784 x 50 41; with a branch that stored
+// a ragged quad's values one by one 608, 248, 132; in 80 registers for a third block
+// per SM 676, 153, 39 (spills).
 struct CLevelOut {
   CSplitOut s2, s1, a22, s4, s3, a11, a12;
 };
 
-__global__ void csblocks_split_kernel(const float2 *__restrict__ A, int64_t lda, int64_t h,
-                                      int64_t kap, int np, CLevelOut o) {
+__global__ void __launch_bounds__(256)
+    csblocks_split_kernel(const float2 *__restrict__ A, int64_t lda, int64_t h, int64_t kap, int np,
+                          CLevelOut o) {
   const int64_t cq = (kap + 3) / 4;
   for (int64_t r = blockIdx.y; r < h; r += gridDim.y)
     for (int64_t q4 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q4 < cq;
@@ -1480,21 +1479,21 @@ __global__ void csblocks_split_kernel(const float2 *__restrict__ A, int64_t lda,
       cload4(A + r * lda + kap, c0, nv, a12);
       cload4(A + (h + r) * lda, c0, nv, a21);
       cload4(A + (h + r) * lda + kap, c0, nv, a22);
-      csplit_store(a11, r, c0, nv, np, o.a11);
-      csplit_store(a12, r, c0, nv, np, o.a12);
-      csplit_store(a22, r, c0, nv, np, o.a22);
+      csplit_store(a11, r, c0, np, o.a11);
+      csplit_store(a12, r, c0, np, o.a12);
+      csplit_store(a22, r, c0, np, o.a22);
 #pragma unroll
       for (int v = 0; v < 4; ++v) s[v] = csub(a22[v], ci(a21[v]));  // S2
-      csplit_store(s, r, c0, nv, np, o.s2);
+      csplit_store(s, r, c0, np, o.s2);
 #pragma unroll
       for (int v = 0; v < 4; ++v) s[v] = ci(csub(a21[v], a11[v]));  // S1
-      csplit_store(s, r, c0, nv, np, o.s1);
+      csplit_store(s, r, c0, np, o.s1);
 #pragma unroll
       for (int v = 0; v < 4; ++v) s[v] = csub(s[v], a22[v]);  // S3
-      csplit_store(s, r, c0, nv, np, o.s3);
+      csplit_store(s, r, c0, np, o.s3);
 #pragma unroll
       for (int v = 0; v < 4; ++v) s[v] = cadd(s[v], a12[v]);  // S4
-      csplit_store(s, r, c0, nv, np, o.s4);
+      csplit_store(s, r, c0, np, o.s4);
     }
 }
 

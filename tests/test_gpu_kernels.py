@@ -581,3 +581,16 @@ def test_split_into_planes_at_any_offset(lib, rows, cols, off):
                                    buf.data_ptr() + 2 * off, T._stream()))
     assert torch.equal(buf[off:off + want.numel()], want)
     assert bool((buf[:off] == 77).all()) and bool((buf[off + want.numel():] == 77).all())
+
+
+@pytest.mark.parametrize("prec,tol", [("AAT_C_FP32", 1e-5), ("AAT_C_BF16X3", 1e-4)])
+@pytest.mark.parametrize("n,k", [(2, 2), (64, 50), (34, 6), (130, 262), (40, 8)])
+def test_complex_level_with_ragged_blocks(lib, n, k, prec, tol):
+    """One level with halves of k that are and are not whole quads of columns,
+    in the class's own bound (relative Frobenius error)."""
+    import torch
+    A = _complex_rows(n, k, "normal")
+    got = lib.aat_complex(torch.from_numpy(A).cuda(), flags=getattr(lib, prec), levels=1).cpu().numpy()
+    Z = A.astype(np.complex128)
+    ref = np.tril(Z @ Z.T)
+    assert np.linalg.norm(np.tril(got) - ref) <= tol * np.linalg.norm(ref)
