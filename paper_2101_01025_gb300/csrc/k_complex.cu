@@ -1238,15 +1238,18 @@ static cudaError_t fused_table(const std::vector<FusedJob> &jobs, int np, int64_
   pair = ev ? (atoi(ev) > 0 && units > 0) : (pair && pt >= units);
   FForm form = pair ? kFPair : kFCta;
   if (!pair) {
-    // 64-column tiles when that shortens the longest CTA: waves of tiles times
-    // modelled SM cycles of a tile, 512 (wide) or 240 (narrow) per K block and
-    // piece product of its job.  A A^H per call, FP32 class: 300 x 300 42 -> 30 us, 500 x
-    // 2000 104 -> 56 us, 100 x 5000 208 -> 99 us (half of it the FP16 pieces).
+    // 64-column tiles when that shortens the longest CTA: waves of average tiles,
+    // or the longest tile, in modelled SM cycles: 600 (wide) or 490 (narrow) per K
+    // block and piece product of its job, 17 and 8 thousand besides.  Leaf of A A^H,
+    // FP32 class, wide / narrow, us: one wave either way, 300 x 300 18.6 / 12.4,
+    // 500 x 2000 42.5 / 33.8, 500 x 6000 100 / 82; two waves of narrow tiles, 900 x 900
+    // 28.6 / 34.9, 900 x 3000 58.2 / 85.6, 1200 x 2000 45.2 / 62.8; three, 1300 x 1000
+    // 29.7 / 50.5.
     double cost[2];
     for (int w = 0; w < 2; ++w) {
       const int tn = w ? kFNarrow : BN;
       int64_t tiles = 0;
-      double cycles = 0.0;
+      double cycles = 0.0, longest = 0.0;
       for (const FusedJob &j : jobs) {
         int pairs[6][2];
         const int products = wide ? kHalfTerms : piece_pairs(std::min(j.keep, np), pairs);
@@ -1255,11 +1258,13 @@ static cudaError_t fused_table(const std::vector<FusedJob> &jobs, int np, int64_
           const int64_t TJ = (j.N + tn - 1) / tn;
           t += j.lower ? std::min(TJ, (i * BM + BM - 1) / tn + 1) : TJ;
         }
-        cycles += (double)t * (w ? 240.0 * products * kblocks + 5000.0
-                                 : 512.0 * products * kblocks + 14000.0);
+        const double tile =
+            w ? 490.0 * products * kblocks + 8000.0 : 600.0 * products * kblocks + 17000.0;
+        longest = std::max(longest, tile);
+        cycles += (double)t * tile;
         tiles += t;
       }
-      cost[w] = cycles / (double)tiles * (double)((tiles + sms - 1) / sms);
+      cost[w] = std::max(longest, cycles / (double)tiles * (double)((tiles + sms - 1) / sms));
     }
     if (cost[1] < cost[0]) form = kFNarrowForm;
   }
