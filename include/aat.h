@@ -89,7 +89,9 @@ extern "C" {
  * at n = k = 16384 over F_{2^31-1}: 27.9 ms with 1 GiB (4-plane windows)
  * against 24.9 ms with 8.75 GiB; 37.9 ms with 0.25 GiB (1 plane).  Applies
  * to the tensor-core leaf with the pair-sum digit form (p = 2^31 - 1, 65521,
- * ...); other leaf and digit forms run the fast schedule.  Same result. */
+ * ...); other leaf and digit forms run the fast schedule, and primes between
+ * 2^16 and 2^17 + 1 the fast schedule on two planes unless the limit or the
+ * memory is too small for it.  Same result. */
 #define AAT_LOW_MEMORY (1u << 14)
 
 /*

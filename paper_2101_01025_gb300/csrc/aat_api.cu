@@ -440,10 +440,16 @@ struct Ctx {
   aatx_plan_stats_t *stats;  // optional counters
   int err = AAT_OK;
   // the digit form of products (entry points; the single-step hooks keep
-  // make_digits' form)
+  // make_digits' form).  Digits of opposite signs are three planes instead of two,
+  // so not with AAT_LOW_MEMORY.
   void use_product_digits(uint32_t flags) {
-    if (!(flags & AAT_DIGITS_PLAIN)) ds = product_digits(m.p);
+    if (flags & AAT_DIGITS_PLAIN) return;
+    const DigitSpec d = product_digits(m.p);
+    opp_ok = d.opp;
+    if (!opp_ok || !(flags & AAT_LOW_MEMORY)) ds = d;
   }
+  bool opp_ok = false;    // the prime has digits of opposite signs
+  bool no_plain = false;  // no memory for the plain form's fast schedule
   // optional: recorded on `st` as soon as rows [split_row, n) of C are final
   // (after the top level's post-additions; at the end when C is padded)
   cudaEvent_t split_ev = nullptr;
@@ -1315,6 +1321,16 @@ static size_t choose_schedule(Ctx &c, const int32_t *A, int64_t n, int64_t k, in
     if (need <= limit) return need;
     c.passes = true;
   }
+  // Digits of opposite signs: one product per digit pair needs two planes instead
+  // of three and no passes; the passes are for what a limit rules out even so
+  // (5382 x 1651 mod 131071, no level: 233 us, in passes 300; 1468 x 204, two levels:
+  // 318 and 765).
+  if (c.opp_ok && !c.no_plain) {
+    c.ds = make_digits(c.m.p);
+    const size_t need = run_plan(c, A, n, k, lda, C, ldc, flags, true, nullptr);
+    if (need <= limit) return need;
+  }
+  if (c.opp_ok) c.ds = product_digits(c.m.p);
   const char *epw = getenv("AAT_PASS_PLANES");
   if (epw) {
     c.pass_w = std::max(1, atoi(epw));
@@ -1517,8 +1533,15 @@ static int modp_device(const int32_t *A, int64_t n, int64_t k, int64_t lda, uint
     // the fast schedule's workspace cannot be had: the low-memory schedule
     if (e != AAT_ENOMEM || c.passes) return e;
     c.passes = true;
-    const size_t low = choose_schedule(c, A, n, k, lda, C, ldc, flags);
-    if (low >= need || (e = ensure_workspace(low, &ws))) return e ? e : AAT_ENOMEM;
+    size_t low = choose_schedule(c, A, n, k, lda, C, ldc, flags);
+    if (low >= need) return e;
+    e = ensure_workspace(low, &ws);
+    if (e == AAT_ENOMEM && c.opp_ok && !c.ds.opp) {  // then the passes
+      c.no_plain = true;
+      low = choose_schedule(c, A, n, k, lda, C, ldc, flags);
+      if (low < need) e = ensure_workspace(low, &ws);
+    }
+    if (e) return e;
     g_last_error.clear();
   }
   c.err = AAT_OK;

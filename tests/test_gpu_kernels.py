@@ -594,3 +594,42 @@ def test_complex_level_with_ragged_blocks(lib, n, k, prec, tol):
     Z = A.astype(np.complex128)
     ref = np.tril(Z @ Z.T)
     assert np.linalg.norm(np.tril(got) - ref) <= tol * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n,k,levels", [(300, 700, 0), (260, 132, 1), (1030, 600, 2)])
+def test_scratch_limits_with_digits_of_opposite_signs(lib, n, k, levels):
+    """Three planes, two planes and plane passes, by flag, limit and failed
+    allocation: the same result."""
+    import torch
+    from paper_2101_01025_gb300 import _native as nat
+    p = 131071
+    A = torch.from_numpy(synth.residues(n + k, (n, k), p)).cuda()
+    D = A.double()
+    ref = torch.remainder((D @ D.T).to(torch.int64), p).tril()
+    plain = lib.aat_workspace_size(n, k, p, lib.AAT_LEVELS(levels) | nat.AAT_DIGITS_PLAIN)
+    fast = lib.aat_workspace_size(n, k, p, lib.AAT_LEVELS(levels))
+
+    def same(flags=0):
+        got = lib.aat_modp(A, p, levels=levels, flags=lib.AAT_ZERO_UPPER | flags)
+        assert torch.equal(got.to(torch.int64), ref)
+    same()
+    same(lib.AAT_LOW_MEMORY)
+    C = torch.zeros((n, n), dtype=torch.int32, device="cuda")
+    lib.aat_syrk_modp(3, A, 0, C, p, flags=lib.AAT_LOW_MEMORY, levels=levels)
+    assert torch.equal(C.to(torch.int64).tril(), torch.remainder(3 * ref, p))
+    for limit in (max(fast, plain + 1) - 1, plain - 1):
+        for flags in (0, lib.AAT_LOW_MEMORY):
+            try:
+                lib.aat_set_workspace_limit(limit)
+                same(flags)
+            finally:
+                lib.aat_set_workspace_limit(None)
+        lib.aat_shutdown()
+        try:
+            nat.lib().aatx_set_alloc_limit(limit)
+            same()
+        except lib.AatError as e:
+            # no level: the passes need as much as two whole planes
+            assert levels == 0 and limit < plain and e.code == nat.AAT_ENOMEM
+        finally:
+            nat.lib().aatx_set_alloc_limit(2**64 - 1)

@@ -379,3 +379,24 @@ def test_plan_statistics_report_the_products_workspace(p, n, k):
     for flags in (0, _native.AAT_LEVELS(0), _native.AAT_LEVELS(1), _native.AAT_LEVELS(2),
                   _native.AAT_LEVELS(1) | _native.AAT_DIGITS_PLAIN, _native.AAT_ZERO_UPPER):
         assert T.plan_stats(n, k, p, flags).workspace_bytes == lib.aat_workspace_size(n, k, p, flags)
+
+
+@pytest.mark.parametrize("n,k,levels", [(5382, 1651, 0), (4096, 4096, 1), (1468, 204, 2)])
+def test_low_memory_of_primes_with_digits_of_opposite_signs(n, k, levels):
+    """Two planes and no passes where AAT_LOW_MEMORY or a limit rules out the
+    three planes; passes where a limit rules out two as well."""
+    lib = _native.lib()
+    p, lv = 131071, _native.AAT_LEVELS(levels)
+
+    def size(flags=0):
+        return lib.aat_workspace_size(n, k, p, lv | flags)
+    fast, plain = size(), size(_native.AAT_DIGITS_PLAIN)
+    assert plain < fast and size(_native.AAT_LOW_MEMORY) == plain
+    try:
+        lib.aat_set_workspace_limit(fast - 1)
+        assert size() == size(_native.AAT_LOW_MEMORY) == plain
+        lib.aat_set_workspace_limit(plain - 1)
+        assert size() == size(_native.AAT_LOW_MEMORY) <= plain
+        assert levels == 0 or size() < plain
+    finally:
+        lib.aat_set_workspace_limit(2**64 - 1)
