@@ -318,14 +318,19 @@ def run_configs(peaks):
                     5, "Low(A A^T) mod %d, %d recursion levels (default depth)" % (p, lv),
                     "leaf_tc")
             del A, C
-    # complex 8192 x 8192: A A^H by 2M and A A^T by Algorithm 1, FP32 class
+    # complex 8192 x 8192: A A^H by 2M, A A^T at the default depth and by
+    # Algorithm 1, FP32 class
     gen.manual_seed(synth.SEED_BASE + 3)
     Z = torch.view_as_complex(torch.randn((8192, 8192, 2), device="cuda", generator=gen))
     CZ = torch.empty((8192, 8192), dtype=torch.complex64, device="cuda")
     measure("complex8192_aah_2m_fp32", lambda: aat.aah_complex(Z, C=CZ), 8192.0**3, 5,
             "Low(A A^H) by 2M, FP32-accurate (2 FP16 pieces, 3 piece products)", "leaf_f32")
-    measure("complex8192_aat_alg1_fp32", lambda: aat.aat_complex(Z, C=CZ), 8192.0**3, 5,
-            "Low(A A^T) by Algorithm 1 (Y = i I, default depth), FP32-accurate", "leaf_f32")
+    measure("complex8192_aat_default_fp32", lambda: aat.aat_complex(Z, C=CZ), 8192.0**3, 5,
+            "Low(A A^T) at the default depth (2M without a level, as A A^H), FP32-accurate",
+            "leaf_f32")
+    measure("complex8192_aat_alg1_fp32", lambda: aat.aat_complex(Z, C=CZ, levels=1), 8192.0**3, 5,
+            "Low(A A^T) by Algorithm 1 (Y = i I), one level, FP32-accurate (3 BF16 pieces, 6 "
+            "piece products)", "leaf_f32")
     del Z, CZ
     # batch: 256 problems over F_65521 + 64 complex A A^H, log-uniform sizes
     ns = synth.log_uniform_ints(synth.SEED_BASE + 4, 256, 64, 2048)

@@ -8,7 +8,8 @@
 
 leaf: one leaf product X Y^T mod p of n x n x n (digit planes split first);
 aah / aatc2m / aatc: complex A A^H by 2M, A A^T by 2M, A A^T by Algorithm 1
-with Y = i I (--prec: BF16 pieces per FP32 value);
+with Y = i I (--levels; without it the default depth, which is 2M in the FP32
+class; --prec: the accuracy class);
 syrk: Low(X X^T) with 0 recursion levels; aat: Low(A A^T) by Algorithm 1;
 full: the plain full product A A^T; peaks: the rates of the mma.sync
 instructions of the INT8 and FP64 leaves (n blocks per SM).  Inputs are

@@ -400,3 +400,17 @@ def test_low_memory_of_primes_with_digits_of_opposite_signs(n, k, levels):
         assert levels == 0 or size() < plain
     finally:
         lib.aat_set_workspace_limit(2**64 - 1)
+
+
+def test_bench_row_of_complex_algorithm_1_asks_for_a_level():
+    """The default depth of aat_complex has no level in the FP32 class: a row
+    named after Algorithm 1 has to ask for one."""
+    import ast
+    with open(os.path.join(ROOT, "bench.py")) as f:
+        calls = [c for c in ast.walk(ast.parse(f.read())) if isinstance(c, ast.Call)
+                 and getattr(c.func, "id", "") == "measure" and isinstance(c.args[0], ast.Constant)]
+    rows = [c for c in calls if "alg1" in c.args[0].value]
+    assert rows
+    for c in rows:
+        kw = {k.arg: k.value for k in c.args[1].body.keywords}
+        assert kw["levels"].value >= 1
