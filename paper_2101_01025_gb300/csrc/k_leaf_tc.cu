@@ -1361,13 +1361,7 @@ cudaError_t launch_leaf_tc(const TcLeafArgs &a, const ModP &m, cudaStream_t st) 
   return cudaGetLastError();
 }
 
-// Whether one launch over the tiles of several products beats one launch
-// per product: the launches of single products leave part of the GPU idle
-// in their last wave (tiles / units rounded up).  Measured on GB300: one
-// launch wins by 5-10 % when those last waves waste 10-16 % of the slots
-// (4096-sized products), and loses ~5 % at 3-4 % (8192-sized products in
-// a second-long run under the power cap, where idle tails let the clock
-// rise).  So: one launch when more than 6 % of the slots would be idle.
+// Plane products of a leaf that do not vanish mod p; -1: no group list fits.
 int leaf_tc_terms(const TcLeafArgs &a, const ModP &m) {
   std::vector<Group> g(MAX_GROUPS);
   int ng = 0, nprod = 0;
@@ -1375,6 +1369,17 @@ int leaf_tc_terms(const TcLeafArgs &a, const ModP &m) {
   return nprod;
 }
 
+// Whether one launch over the tiles of several products beats one launch
+// per product: the launches of single products leave part of the GPU idle
+// in their last wave (tiles / units rounded up).  One launch wins by 5-10 % when
+// those last waves waste 10-16 % of the slots (4096-sized products), and loses
+// ~5 % at 3-4 % (8192-sized products in a second-long run under the power cap,
+// where idle tails let the clock rise).  So: one launch when more than 6 % of the
+// slots would be idle, counted in 256-column tiles whatever the single launches
+// would take: products so small that they would take narrower tiles or run in
+// parts are better off jointly too (a level of 256^2 .. 10240^2 and quaternion
+// products of 64^2 .. 5120 x 2000 mod 65521 and 2^31 - 1, 76 shapes: the joint launch
+// won all of them, 1.05-2.8 times as fast, and is chosen).
 bool leaf_tc_fuse_pays(const TcLeafArgs *as, int count) {
   int dev = 0;
   cudaGetDevice(&dev);
