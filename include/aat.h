@@ -23,7 +23,10 @@
  *     AAT_ZERO_UPPER is given.
  *   - Calls are asynchronous on `stream` (a cudaStream_t, NULL = legacy
  *     default stream) unless stated.  Internal workspace is owned by the
- *     library, grown on demand and released by aat_shutdown().
+ *     library, one per device, grown on demand and released by
+ *     aat_shutdown(): calls that use it on several streams have to be ordered
+ *     by their caller (plans own theirs).  The first call of a shape, prime and
+ *     flags may allocate; after it such a call can be captured.
  *   - Return codes: AAT_OK or a negative AAT_E*; aat_last_error() gives a
  *     message for the calling thread.  No entry point falls back to the
  *     CPU: without a usable sm_103a GPU they fail with AAT_ECUDA.
@@ -170,7 +173,7 @@ AAT_API int64_t aat_modp_host_d2h_bytes(int64_t n, uint32_t flags);
  * The choices tuned: the recursion depth (the cut-off of Algorithm 1's
  * recursion, Sec. 3; the paper leaves it to the implementation, Sec. 7), the
  * leaf kernel form (form 1: one CTA per 128 x 256 or 128 x 64 tile; form 2: CTA pairs,
- * 256 x 256 tiles), the digit-product form (plain_digits 1: one product per
+ * 256 x 256 or 256 x 128 tiles), the digit-product form (plain_digits 1: one product per
  * digit pair) and Winograd's form for the last level's general products
  * (winograd 1, as AAT_WINOGRAD).  aat_tune_modp runs every candidate on
  * synthetic balanced

@@ -272,7 +272,7 @@ __device__ __forceinline__ OutView tile_out(const Params &P, int t) {
 //   and stores of a tile with twice the threads (the epilogue's per-entry
 //   work is latency-bound at 2 warps per scheduler: the 128 live
 //   accumulators leave few registers for independent temporaries); the
-//   price is 96 registers per thread (and some spills).
+//   price is 96 registers per thread.
 //   TN: tile columns.  64 instead of 256 in the narrow one-CTA form
 //   (leaf_form): four times as many CTAs share the work of a product with
 //   few tiles, and each epilogue thread converts, multiplies and stores 32
