@@ -857,30 +857,32 @@ __device__ __forceinline__ void row_stats(const float2 *__restrict__ A, int64_t 
   if (row >= n) return;
   const float2 *a_row = A + row * lda;
   RowAcc a = {0.f, 0.f, 0.f, 0.f, 0u, 0xffffffffu};
-  int64_t l = 0;
-  if ((reinterpret_cast<uintptr_t>(a_row) & 15) == 0) {
-    // two complex values per lane per 16-byte load, four loads in flight
-    const float4 *a4 = reinterpret_cast<const float4 *>(a_row);
-    const int64_t k2 = k / 2;
-    int64_t q = lane;
-    for (; q + 96 < k2; q += 128) {
-      float4 v[4];
+  // two complex values per lane per 16-byte load, four loads in flight; a first
+  // value off 16 bytes and an odd last one go to lane 0 (710 rows of 4745 values, every
+  // second row off 16 bytes: 27 us, one value per load in those 39)
+  const int64_t head = (int64_t)((reinterpret_cast<uintptr_t>(a_row) >> 3) & 1);
+  const float4 *a4 = reinterpret_cast<const float4 *>(a_row + head);
+  const int64_t k2 = (k - head) / 2;
+  int64_t q = lane;
+  for (; q + 96 < k2; q += 128) {
+    float4 v[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) v[i] = a4[q + 32 * i];
+    for (int i = 0; i < 4; ++i) v[i] = a4[q + 32 * i];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        row_acc<DIAG, SCALE>(make_float2(v[i].x, v[i].y), a);
-        row_acc<DIAG, SCALE>(make_float2(v[i].z, v[i].w), a);
-      }
+    for (int i = 0; i < 4; ++i) {
+      row_acc<DIAG, SCALE>(make_float2(v[i].x, v[i].y), a);
+      row_acc<DIAG, SCALE>(make_float2(v[i].z, v[i].w), a);
     }
-    for (; q < k2; q += 32) {
-      const float4 v = a4[q];
-      row_acc<DIAG, SCALE>(make_float2(v.x, v.y), a);
-      row_acc<DIAG, SCALE>(make_float2(v.z, v.w), a);
-    }
-    l = 2 * k2;  // an odd last column is left to the loop below
   }
-  for (l += lane; l < k; l += 32) row_acc<DIAG, SCALE>(a_row[l], a);
+  for (; q < k2; q += 32) {
+    const float4 v = a4[q];
+    row_acc<DIAG, SCALE>(make_float2(v.x, v.y), a);
+    row_acc<DIAG, SCALE>(make_float2(v.z, v.w), a);
+  }
+  if (lane == 0) {
+    if (head) row_acc<DIAG, SCALE>(a_row[0], a);
+    if (head + 2 * k2 < k) row_acc<DIAG, SCALE>(a_row[k - 1], a);
+  }
   if constexpr (DIAG) {
     double s = ((double)a.h0 + (double)a.l0) + ((double)a.h1 + (double)a.l1);
     for (int off = 16; off; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
