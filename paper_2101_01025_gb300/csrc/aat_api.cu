@@ -1693,7 +1693,8 @@ static int64_t host_two_parts_rows(const Ctx &c, int64_t n, int64_t k, uint32_t 
     const TcLeafArgs a = tc_args(c, P1, P1, r1, r1, k, nullptr, n, 1, 0);
     double t = (double)r1 * k * 4.0 * us_per_byte + leaf_tc_model_us(&a, 1, r1 == n);
     if (r1 == n)
-      return t + (zero ? (double)n * n : 0.5 * (double)n * n) * 4.0 * us_per_byte + (zero ? 0.0 : 45.0);
+      return t + (zero ? (double)n * n * 4.0 * us_per_byte
+                       : 0.5 * (double)n * n * 4.0 * us_per_byte + 45.0);
     const TcLeafArgs b[2] = {tc_args(c, P2, P1, n - r1, r1, k, nullptr, n, 0, 0),
                              tc_args(c, P2, P2, n - r1, n - r1, k, nullptr, n, 1, 0)};
     t += leaf_tc_model_us(b, 2) + 10.0;

@@ -35,8 +35,8 @@
 // ends of FP32's range, the whole product runs on the six BF16 products instead
 // (`wide` != 0).  An entry made only of a row's small values (the other row
 // zero elsewhere) then keeps FP32's accuracy; with the second piece unscaled
-// and a limit of 2^8 on the average spread of a row, 15 % of the values 2^-26 below the rest came out 3.7e-4
-// wrong and 5 % at 2^-60 were lost.  N(0, 1) rows of 32768 values have a value
+// and a limit of 2^8 on the average spread of a row, 15 % of the values 2^-26
+// below the rest came out 3.7e-4 wrong and 5 % at 2^-60 were lost.  N(0, 1) rows of 32768 values have a value
 // 2^-28 below the largest in one row of 2500, one at 2^-33 in one of 80000.
 // Relative Frobenius error against 64 bits at n = k = 8192,
 // N(0, 1): A A^H 1.8e-7 (3.4e-7 by the six BF16 products), A A^T by 2M 3.1e-7
